@@ -64,6 +64,7 @@ struct Grid {
     float *d_s2f = nullptr;     // the same rounded to FP32 (the knot-segment search)
     float *d_ctab = nullptr;    // tensor-core cosine table (TF32 hi/lo, core-matrix layout)
     int nkc_tab = 0;            // 32-sample chunks the cosine table covers
+    float2 *d_cos2n = nullptr;  // cos(pi t / N), t < 2N, as TF32 (hi, lo): samples past that table
     float *d_ctabP = nullptr;   // knot-projection cosine table: per chunk of 32 modes, 128 taps of
                                 // each flavour (TF32 hi/lo, core-matrix layout)
     int nmc_p = 0;              // its chunks of 32 modes
@@ -118,6 +119,8 @@ struct Kernel {
     int max_stage_rows16 = 0;  // the same for blocks of 16 rings
     int max_union4 = 0;        // largest union band of rings 4g .. 4g+3
     int max_stage_rows_g4 = 0, max_stage_rows16_g4 = 0;  // staged rows with groups of four
+    int max_free_taps = 0;     // most samples of a pair whose coefficients are not tabulated
+    int max_win_rows = 0;      // rows of a 32-slot window over a block of 16 in groups of four
     int polar_pairs = 0;       // leading pairs whose coefficients are tabulated per call
     int knot_fft_pairs = 0;    // leading pairs whose knot-gradient projection runs by FFT
     bool proj_tc_ok = false;   // the other pairs have at most 128 samples (tensor-core projection)
@@ -291,9 +294,16 @@ int contract_band_limit();
 int contract_band_rings();
 cudaError_t launch_contract_band(const ContractArgs &a, int nchunks, int max_union, cudaStream_t st);
 // tensor-core contraction over blocks of rb (8 or 16) representative rings, a thread taking
-// a group of gs (2 or 4) rings
-cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, int nchunks, const float *ctab, int nkc_tab,
-                               int srows, int want_nbuf, cudaStream_t st);
+// a group of gs (2 or 4) rings; the wide form takes bands of any width
+struct TcTables {
+    const float *ctab;    // cosines of the first 32 nkc samples in the operand layout
+    const float2 *cos2n;  // cos(pi t / N), t < 2N (hi, lo)
+    int nkc;
+};
+cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, int nchunks, const TcTables &tb, int srows,
+                               int want_nbuf, cudaStream_t st);
+cudaError_t launch_contract_tc_wide(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, cudaStream_t st);
+bool contract_tc_wide_fits(int srows);
 int contract_tc_nbuf(int rb, int gs, int srows, int want_nbuf);
 size_t contract_tc_smem(int rb, int gs, int srows, int want_nbuf);
 int contract_tc_modes();

@@ -81,6 +81,7 @@ void free_grid_dev(Grid &g)
     cudaFree(g.d_s2f);
     cudaFree(g.d_ctab);
     cudaFree(g.d_ctabP);
+    cudaFree(g.d_cos2n);
     cudaFree(g.d_fb);
     cudaFree(g.d_fboff);
     for (auto &c : g.fft) cudaFree(c.reps);
@@ -130,6 +131,15 @@ arkcos_status build_cos_table(Grid &g)
             }
     arkcos_status st = upload(&g.d_ctab, tab);
     if (st != ARKCOS_OK) return st;
+    // samples past that table (pairs of more than 128 next to the poles): the same split values
+    // by angle, gathered by the kernel
+    std::vector<float2> c2(2 * (size_t)g.N);
+    for (int t = 0; t < 2 * g.N; ++t) {
+        const double v = cos(M_PI * (double)t / (double)g.N);
+        const float h = tf32_rna((float)v);
+        c2[t] = make_float2(h, tf32_rna((float)(v - (double)h)));
+    }
+    if ((st = upload(&g.d_cos2n, c2)) != ARKCOS_OK) return st;
     // the knot-projection table: chunk c of 32 modes m = 32 c + k, rows r = 128 f + t:
     // cos(pi m (2t + f) / N) (zero past N/2)
     const int nmc = (NH + 31) / 32;
@@ -628,7 +638,8 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
 {
     const int H = contract_ring_block();
     int maxband = 0, maxunion = 0, maxunion2 = 0, maxunion4 = 0;
-    int srows[2][2] = {{0, 0}, {0, 0}};  // [16-ring blocks][groups of four]
+    int srows[2][2] = {{0, 0}, {0, 0}}, wrows = 0;  // [16-ring blocks][groups of four]; wide form
+    int maxfree = 0;  // most samples of a pair without tabulated coefficients
     for (int64_t k = 0; k < nk; ++k) {
         const Kernel &K = ks[k]->k;
         maxband = std::max(maxband, K.maxband);
@@ -639,10 +650,19 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
         srows[0][1] = std::max(srows[0][1], K.max_stage_rows_g4);
         srows[1][0] = std::max(srows[1][0], K.max_stage_rows16);
         srows[1][1] = std::max(srows[1][1], K.max_stage_rows16_g4);
+        wrows = std::max(wrows, K.max_win_rows);
+        maxfree = std::max(maxfree, K.max_free_taps);
     }
     // the register-resident fast path covers bands of up to contract_band_limit() rings
     const bool fast = maxband <= contract_band_limit() && 2 * maxunion * 64 * 16 <= 200 * 1024;
-    const bool tc = tf32 && maxunion2 <= contract_band_limit() && contract_tc_smem(8, 2, srows[0][0], 0) <= 200 * 1024;
+    const bool tc = tf32 && maxunion2 <= contract_band_limit() && maxfree <= 32 * g.nkc_tab &&
+                    contract_tc_smem(8, 2, srows[0][0], 0) <= 200 * 1024;
+    // bands whose ring groups see more than 32 input rings, or pairs with more samples than one
+    // run of the kernel and no tabulated coefficients: the tensor-core form with the 32
+    // slots moving along the band (contraction of 77.1 -> 4.5 ms for one nside-2048 map at a degree of support
+    // against k_contract<8>, which remains for the plain FP32 form)
+    const bool tc_wide = tf32 && !tc && contract_tc_wide_fits(wrows);
+    const TcTables tb{g.d_ctab, g.d_cos2n, g.nkc_tab};
     // tensor-core form: groups of four rings when their union bands fit the 32 slots, blocks of
     // 16 rings when two staging buffers fit beside one CTA per SM; the autotuner's choice, else
     // the default: for a shared beam groups of four in blocks of 16 where they fit; for per-map
@@ -666,7 +686,7 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
     auto kof = [&](int64_t v) { return kdiv > 0 ? v % kdiv : v; };  // kernel of map v
     const int64_t groups = per_map ? (nmaps + kMaxKernelsPerLaunch - 1) / kMaxKernelsPerLaunch : 1;
     StageScope sc(ST_CONTRACT, (int)groups, st);
-    if (kdiv > 0 && polar_table && (tc || fast)) {
+    if (kdiv > 0 && polar_table && (tc || tc_wide || fast)) {
         // several maps share each kernel: its polar coefficient table is computed once
         for (int64_t k0 = 0; k0 < kdiv; k0 += kMaxKernelsPerLaunch) {
             ContractArgs a;
@@ -735,11 +755,12 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
             a.B = (int)cnt;
             a.map_base = 0;
         }
-        if ((tc || fast) && polar_table && kdiv == 0 && maxpolar > 0) {
+        if ((tc || tc_wide || fast) && polar_table && kdiv == 0 && maxpolar > 0) {
             CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, st));
             ++sc.launches;
         }
-        if (tc) CK(launch_contract_tc(a, tc_rb, tc_gs, nchunks, g.d_ctab, g.nkc_tab, tc_srows, tc_want, st));
+        if (tc) CK(launch_contract_tc(a, tc_rb, tc_gs, nchunks, tb, tc_srows, tc_want, st));
+        else if (tc_wide) CK(launch_contract_tc_wide(a, nchunks, tb, wrows, st));
         else if (fast) CK(launch_contract_band(a, nchunks, maxunion, st));
         else CK(launch_contract(a, nchunks, smem, st));
     }
@@ -1026,6 +1047,7 @@ arkcos_status arkcos_set_kernel(arkcos_grid grid, const double *knots, int64_t n
                                     : (gs == 2 ? K.max_stage_rows16 : K.max_stage_rows16_g4);
                 for (int q = r0; q <= r1; q += gs) {
                     rows = std::max(rows, jlo[q] - jlo[r0] + 32);
+                    if (rb == 16 && gs == 4) K.max_win_rows = std::max(K.max_win_rows, jlo[q] - jlo[r0] + 32);
                     if (gs == 4) K.max_union4 = std::max(K.max_union4, jhi[std::min(q + 3, r1)] - jlo[q] + 1);
                 }
                 rows = std::max(rows, jhi[r1] - jlo[r0] + 1);
@@ -1086,6 +1108,8 @@ arkcos_status arkcos_set_kernel(arkcos_grid grid, const double *knots, int64_t n
         int mx = 0;
         for (int p = K.knot_fft_pairs; p < K.npairs; ++p) mx = std::max(mx, std::max(S0[p], S1[p]) + 1);
         K.proj_tc_ok = mx <= 128;
+        for (int p = K.polar_pairs; p < K.npairs; ++p)
+            K.max_free_taps = std::max(K.max_free_taps, std::max(S0[p], S1[p]) + 1);
     }
     std::vector<int> ufix, unofix;
     const int ut_step = knot_proj_taps();

@@ -4,20 +4,40 @@
 // For a block of RB (8 or 16) representative output rings x 128 modes the coefficients are a
 // dense product  rho[m, col] = sum_k C_f[m, k] T[k, col]  with C_f[m, k] = cos(pi m (2k + f) / N)
 // (f = the pair's sample offset, see contract.cu) and T the FP32 kernel samples.  The CTA
-// stages C (an exact FP64 table split into TF32 hi + lo parts, prepared per grid in the
-// tensor-core layout) and T (split into hi + lo on the fly) in shared memory, chunk by chunk of
-// 32 samples with the next chunk's loads in flight, and one thread issues tcgen05.mma
-// kind::tf32 with the accumulator in tensor memory:
+// stages C (exact FP64 values split into TF32 hi + lo parts, prepared per grid) and T (split
+// into hi + lo on the fly) in shared memory, a pass of 16 samples at a time with the next pass's
+// loads in flight, and one thread issues tcgen05.mma kind::tf32 with the accumulator in tensor
+// memory:
 //     D = C_hi T_hi + C_hi T_lo + C_lo T_hi      (3xTF32, FP32 accumulation).
-// Pairs of the two offsets accumulate into the same columns with the other offset's samples
-// zeroed.  The rings of the block go in groups of G (2 or 4) consecutive rings; column
-// 32 (G g + t) + u holds the pair of ring G g + t with input ring jlo(G g) + u (zero when that
-// ring is outside its band), so the rings of a group index one common run of 32 input rings.
+// The rings of the block go in groups of G (2 or 4) consecutive rings; slot u of ring l holds
+// the pair of that ring with input ring jlo(first ring of its group) + u (zero when that ring is
+// outside its band), so the rings of a group index one common run of 32 input rings.  On the
+// equatorial belt the sample offset f alternates with the parity of i + j, so the 32 RB columns
+// are split by the parity of u + l into two tiles: there each tile has one f, and one pass
+// serves both with a cosine operand each (no products with the other offset's zeros); tiles
+// that hold both offsets (blocks at the edge of the belt) take a pass for each.
 // Each thread (mode, group) reads slices of its G x 32 coefficients of D with tcgen05.ld and
-// contracts every staged input coefficient into all G rings' outputs.  Waits on the MMA
-// completion barriers are bounded: on expiry the kernel records an error (reported by
-// arkcos_sync_status) and still frees its tensor memory.
+// contracts every staged input coefficient into all G rings' outputs.
+//
+// Bands wider than 32 rings take the 32 slots as a window that moves along the band, and pairs
+// of more than 128 samples (untabulated rings next to the poles) are generated 128 samples at a
+// time: the outputs are linear in the coefficients, so every (window, run of 128 samples) is
+// generated, contracted and added in FP32.  No sum on the tensor core is longer than 128
+// samples (its accumulator's additions do not round to nearest), and no table grows with the
+// support.
+//
+// What bounds it: with many maps the contraction on the CUDA cores (0.155 ms per nside-2048
+// map, issue); with one map per kernel the generation (tap loads, splits, one pass's round
+// trip), which is why a pass stages no more samples and cosines than its K-steps read, serves
+// both offsets and overlaps the copy of the first map: 64 nside-1024 maps with a beam each
+// 9.05 -> 7.22 ms against passes of 32 samples per offset, one nside-2048 map 0.67 -> 0.51 ms,
+// 16 maps with one beam 2.99 -> 2.94 ms.  Wide bands, one nside-2048 map at a degree of support
+// (about 105 rings): 4.5 ms, against 77.1 ms generated and contracted on the CUDA cores.
+// Waits on the MMA completion barriers are bounded: on expiry the kernel records an error
+// (reported by arkcos_sync_status) and still frees its tensor memory.
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "tcgen05.cuh"
 
@@ -31,17 +51,23 @@ using namespace tc;
 
 constexpr int kTcModes = 128;          // M of the MMA: modes per CTA (TMEM lanes)
 constexpr int kTcBand = 32;            // input-ring slots per group (columns per ring)
-constexpr int kTcNTile = 256;          // N of one MMA: 8 rings x 32 slots
-constexpr int kTcKChunk = 32;          // taps per shared-memory chunk (4 MMA K-steps of 8)
+constexpr int kTcK = 16;               // samples per pass (2 MMA K-steps of 8)
+constexpr int kTcRun = 128;            // samples per generated run (longest tensor-core sum)
+constexpr uint32_t kTcSBO = 4 * kLBO;  // row octets of an operand of 16 samples
 
 // A CTA takes RB representative output rings (8 or 16) x kTcModes modes: RB / G ring groups
 // of G (2 or 4) consecutive rings, one warp per group and lane quarter; RB x 32 tensor-memory
-// columns, filled by RB / 8 MMAs of N = 256 per K-step.
+// columns in two tiles.  A stage holds the cosines of both tiles and the samples of every
+// column for one pass; RB = 16 (one CTA per SM) has two stages, so that a pass is staged while
+// the MMAs of the one before it run, RB = 8 has one (two CTAs per SM overlap instead).
 template <int RB, int G>
 struct TcShape {
-    static constexpr int kRings = RB, kGroups = RB / G, kThreads = kTcModes * kGroups;
-    static constexpr int kN = RB * kTcBand, kTiles = kN / kTcNTile, kTmemCols = kN;
-    static constexpr size_t kAB = 2 * 16384 + 2 * (size_t)kN / 8 * kSBO;  // A hi | lo, B hi | lo
+    static constexpr int kGroups = RB / G, kThreads = kTcModes * kGroups;
+    static constexpr int kN = RB * kTcBand, kTile = kN / 2, kTmemCols = kN;
+    static constexpr uint32_t kA = kTcModes / 8 * kTcSBO;  // one cosine operand (hi or lo)
+    static constexpr uint32_t kB = kN / 8 * kTcSBO;        // the samples (hi or lo) of every column
+    static constexpr uint32_t kStage = 4 * kA + 2 * kB;
+    static constexpr int kStages = RB / 8;
 };
 
 // acc += c v for the four lanes of v, as two packed two-lane FMAs (each lane rounds as fmaf)
@@ -53,38 +79,49 @@ __device__ __forceinline__ void fma4(float4 &acc, float c, const float4 &v)
     acc = make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
-template <int RB, int G>
+// Issue the copies of input rings [j0, j0 + rows) x kTcModes modes from m0 (zero past N/2) into
+// shared memory, raw paired rows: a thread keeps its mode.
+template <int THREADS>
+__device__ __forceinline__ void stage_rows(float4 *dst, const float4 *__restrict__ sp4b, int j0, int rows, int m0,
+                                           int R, int NH)
+{
+    const int c = threadIdx.x % kTcModes, mm = m0 + c;
+    const bool mv = mm < NH;
+    const float4 *src = sp4b + (mv ? mm : 0);
+    for (int jj = threadIdx.x / kTcModes; jj < rows; jj += THREADS / kTcModes) {
+        const int j = j0 + jj;
+        cp_async16(&dst[jj * kTcModes + c], src + (mv ? (int64_t)min(j, R - 1 - j) * NH : 0), mv ? 16 : 0);
+    }
+    cp_async_commit();
+}
+
+template <int RB, int G, bool WIDE>
 __global__ void __launch_bounds__(TcShape<RB, G>::kThreads, 16 / RB)
-k_contract_tc(ContractArgs a, const float *__restrict__ ctab, int nkc_tab, int srows, int nbuf)
+k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__restrict__ cos2n, int nkc_tab, int srows,
+              int nbuf, uint32_t rows0, uint32_t ctl)
 {
     using Sh = TcShape<RB, G>;
-    constexpr int kTcRings = Sh::kRings, kTcN = Sh::kN, kTcTmemCols = Sh::kTmemCols;
+    constexpr int kTcN = Sh::kN, kTile = Sh::kTile;
     extern __shared__ __align__(1024) unsigned char smem[];
-    // A hi | A lo (16 KiB each) and B hi | B lo (32 KiB each), then reused for the
-    // staged spectra; the last 16 bytes hold the MMA barrier and the tensor-memory address
-    const size_t stage_bytes = (size_t)nbuf * srows * kTcModes * sizeof(float4);
-    const size_t ab_bytes = Sh::kAB;
-    const size_t ctl = ((stage_bytes > ab_bytes ? stage_bytes : ab_bytes) + 15) & ~size_t(15);
+    // per stage: cosines hi | lo of tile 0, of tile 1, samples hi | lo of every column; then
+    // reused for the staged spectra; at ctl the MMA barriers and the tensor-memory address
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + ctl);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + ctl + 8);
-    unsigned char *Ahi = smem, *Alo = smem + 16384;
-    unsigned char *Bhi = smem + 32768, *Blo = Bhi + kTcN / 8 * kSBO;
-    float4 *sh4 = reinterpret_cast<float4 *>(smem);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + ctl + 16);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q4 = warp & 3, grp = warp >> 2;  // lane quarter of TMEM, ring group
     const int mrow = q4 * 32 + lane;           // mode within the block
-    const int m = blockIdx.x * kTcModes + mrow;
+    const int m0 = blockIdx.x * kTcModes, m = m0 + mrow;
     const bool mv = m < a.NH;
-    const int r0 = blockIdx.y * kTcRings;
-    const int nr = min(kTcRings, a.nrep - r0);
+    const int r0 = blockIdx.y * RB;
+    const int nr = min(RB, a.nrep - r0);
     if (a.basic) {
         // BASIC variant: output ring i keeps only its modes m <= n_i / 2 (Sec. 4.1 truncation;
         // the inverse transform reads no others), so a block of modes above the Nyquist
         // frequency of every ring of the block (and of their mirrors) has nothing to compute
         int nmax = 0;
         for (int t = 0; t < nr; ++t) nmax = max(nmax, __ldg(&a.rd.n[r0 + t]));
-        if ((int)blockIdx.x * kTcModes > nmax / 2) return;
+        if (m0 > nmax / 2) return;
     }
     const int b0 = blockIdx.z * a.maps_per_chunk;
     const int b1 = min(a.B, b0 + a.maps_per_chunk);
@@ -97,272 +134,398 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, int nkc_tab, int s
     const bool v0 = G * grp < nr;
     const int jg0 = v0 ? kd.jlo[i0] : 0;
     const int ju0 = kd.jlo[r0];
-    const int nu = kd.jhi[r0 + nr - 1] - ju0 + 1;
+    const int jlast = kd.jhi[r0 + nr - 1];
+    // the groups' common runs are covered by windows of 32 slots
+    int nwin = 1;
+    if constexpr (WIDE) {
+        int len = 1;
+        for (int g = 0; g < nr; g += G) len = max(len, kd.jhi[r0 + min(g + G, nr) - 1] - kd.jlo[r0 + g] + 1);
+        nwin = (len + kTcBand - 1) / kTcBand;
+    }
 
-    // ---- tensor memory and the completion barrier
+    // ---- tensor memory and the completion barriers
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"((uint32_t)__cvta_generic_to_shared(tslot)), "r"(kTcTmemCols));
+                     ::"r"((uint32_t)__cvta_generic_to_shared(tslot)), "r"(Sh::kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;"
-                     ::"r"((uint32_t)__cvta_generic_to_shared(mbar)));
+        for (int q = 0; q < 2; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;"
+                         ::"r"((uint32_t)__cvta_generic_to_shared(mbar + q)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // per column: sample offset in `taps`, last sample and offset flavour (S = -1: empty), and
+    // the pair; the largest sample count per tile and flavour
+    __shared__ int s_kmax[2][2];
+    __shared__ int s_toff[kTcN], s_S[kTcN], s_p[kTcN];  // s_S = 2 S + f
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (tid < 4) s_kmax[tid >> 1][tid & 1] = 0;
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
     const uint32_t mbar_s = (uint32_t)__cvta_generic_to_shared(mbar);
-
-    // per pair slot: sample offset in `taps`, last sample and offset flavour (S = -1: empty);
-    // and the largest sample count of the block's pairs per flavour
-    __shared__ int s_kmax[2];
-    __shared__ int s_toff[kTcN], s_S[kTcN], s_f[kTcN], s_p[kTcN];
-    if (tid < 2) s_kmax[tid] = 0;
-    __syncthreads();
-    for (int c = tid; c < kTcN; c += blockDim.x) {
-        // column c: ring l = c / 32 of the block, input ring jlo(first ring of l's group) + c % 32;
-        // the table is laid out per block of 8 rings
-        const int blk8 = blockIdx.y * (RB / 8) + c / kTcNTile;
-        const int4 *ct = G == 2 ? kd.coltab : kd.coltab4;
-        const int4 e = 8 * blk8 < a.nrep ? __ldg(&ct[(size_t)blk8 * kTcNTile + c % kTcNTile])
-                                         : make_int4(-1, 0, -1, -2);
-        int toff = 0, S = -1, f = 0, p = 0;
-        if (e.x >= 0) {
-            p = e.x;
-            toff = e.y;
-            f = a.shift_fix ? (e.w & 1) : 0;
-            S = f ? (e.w >> 1) : e.z;
-            atomicMax(&s_kmax[f], S + 1);
-        }
-        s_toff[c] = toff;
-        s_S[c] = S;
-        s_f[c] = f;
-        s_p[c] = p;
-    }
-    __syncthreads();
-    const int kmax0 = s_kmax[0], kmax1 = s_kmax[1];
-    const int kcap = nkc_tab * kTcKChunk;  // samples the cosine table covers
-    // blocks whose pairs all have tabulated coefficients read them (whatever the block size,
-    // so both block sizes give the same result); the others generate theirs on the tensor
-    // cores when the cosine table covers their samples
-    const bool tabulated = kd.pstart[r0 + nr] <= kd.polar_pairs;
-    const bool use_tc = !tabulated && kmax0 <= kcap && kmax1 <= kcap;
-    // the coefficients stay in tensor memory: lane = mode, column 32 l + u (see above)
+    const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16);
-    const uint32_t colg = lane_base + (uint32_t)(G * grp * kTcBand);  // the group's first column
-    bool have_rho = kmax0 + kmax1 > 0;  // CTA-uniform: some column has samples
-    if (use_tc) {
-        // once any CTA has seen an expired wait the results are invalid anyway: skip the MMAs
-        bool ok = *((volatile int *)&g_tc_error) == 0;
-        ok = __syncthreads_and(ok);
-        uint32_t phase = 0;
-        bool first = true;  // meaningful in the issuing thread only
-        const uint32_t idesc = tf32_idesc(kTcModes, kTcNTile);
-        // the chunks of 32 samples, flavour 0 first: the samples of chunk i + 1 are loaded into
-        // registers while the MMAs of chunk i run, and its cosine tile is copied asynchronously
-        // while its samples are split into the B operand
-        const int n0 = (kmax0 + kTcKChunk - 1) / kTcKChunk, nch = n0 + (kmax1 + kTcKChunk - 1) / kTcKChunk;
-        constexpr int kUnits = Sh::kN * 2 / Sh::kThreads;  // (column, 16 samples) units per thread
-        float4 pre[kUnits][4];
-        // a thread takes 16 consecutive samples of one column, loaded four at a time (tap
-        // offsets are multiples of 4 and each pair's slots are padded to 4, so a float4 that
-        // starts at or before the last sample stays inside the pair); others read as zero
-        auto load_taps = [&](int i) {
-            const int f = i < n0 ? 0 : 1, kc = f ? i - n0 : i;
-#pragma unroll
-            for (int u = 0; u < kUnits; ++u) {
-                const int e = tid + u * blockDim.x, c = e >> 1, k0 = (e & 1) * 16;
-                const int S = s_f[c] == f ? s_S[c] : -1;
-                const float *tp = taps + s_toff[c];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int kk = kc * kTcKChunk + k0 + 4 * q;
-                    pre[u][q] = kk <= S ? __ldg(reinterpret_cast<const float4 *>(tp + kk))
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-        };
-        if (nch > 0) load_taps(0);
-        for (int i = 0; i < nch; ++i) {
-            const int f = i < n0 ? 0 : 1, kc = f ? i - n0 : i;
-            const int kf = f ? kmax1 : kmax0;
-            const int ksteps = min(4, (kf - kc * kTcKChunk + 7) / 8);
-            // A: this mode block's cosine chunk (hi, lo), prepared in the core layout
-            const float *src = ctab + ((((size_t)blockIdx.x * 2 + f) * nkc_tab + kc) * 2) * 4096;
-            for (int e = tid; e < 2 * 1024; e += blockDim.x) cp_async16(Ahi + 16 * e, src + 4 * e, 16);
-            cp_async_commit();
-            // B: the samples of every column of the block for this flavour, split hi / lo
-#pragma unroll
-            for (int u = 0; u < kUnits; ++u) {
-                const int e = tid + u * blockDim.x, c = e >> 1, k0 = (e & 1) * 16;
-                const int S = s_f[c] == f ? s_S[c] : -1;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int kk = kc * kTcKChunk + k0 + 4 * q;
-                    const float v[4] = {pre[u][q].x, pre[u][q].y, pre[u][q].z, pre[u][q].w};
-                    float4 hi4, lo4;
-                    float *hp = &hi4.x, *lp = &lo4.x;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float x = kk + j <= S ? v[j] : 0.f;
-                        hp[j] = tf32_round(x);
-                        lp[j] = tf32_round(x - hp[j]);
-                    }
-                    const uint32_t off = core_offset(c, k0 + 4 * q);
-                    *reinterpret_cast<float4 *>(Bhi + off) = hi4;
-                    *reinterpret_cast<float4 *>(Blo + off) = lo4;
-                }
-            }
-            if (i + 1 < nch) load_taps(i + 1);
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncthreads();
-            // CTA-uniform: whether this chunk's MMAs and their commit are issued (the test
-            // knob withholds them, so that the wait below runs out)
-            const bool issued = ok && !a.withhold_mma;
-            if (tid == 0 && issued) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t sa_hi = (uint32_t)__cvta_generic_to_shared(Ahi);
-                const uint32_t sa_lo = (uint32_t)__cvta_generic_to_shared(Alo);
-                const uint32_t sb_hi = (uint32_t)__cvta_generic_to_shared(Bhi);
-                const uint32_t sb_lo = (uint32_t)__cvta_generic_to_shared(Blo);
-                for (int ks = 0; ks < ksteps; ++ks) {
-                    const uint32_t o = ks * 2 * kLBO;  // 8 TF32 values = two core columns
-#pragma unroll
-                    for (int t = 0; t < Sh::kTiles; ++t) {
-                        // tile t: columns [256 t, 256 t + 256), its B rows 32 KiB further on
-                        const uint32_t d = tmem + (uint32_t)(t * kTcNTile);
-                        const uint32_t ob = o + (uint32_t)t * (kTcNTile / 8) * kSBO;
-                        mma_tf32(d, smem_desc(sa_hi + o), smem_desc(sb_hi + ob), idesc, first ? 0 : 1);
-                        mma_tf32(d, smem_desc(sa_hi + o), smem_desc(sb_lo + ob), idesc, 1);
-                        mma_tf32(d, smem_desc(sa_lo + o), smem_desc(sb_hi + ob), idesc, 1);
-                    }
-                    first = false;
-                }
-                mma_commit(mbar_s);
-            }
-            // every thread waits for the MMAs before the next chunk reuses shared memory; a
-            // wait that expires is recorded and stops further MMAs.  An issued commit is
-            // waited for once more (bounded) before anything reuses the memory its MMAs use;
-            // nothing is in flight when the issue was withheld
-            if (ok) {
-                bool done = mbar_wait(mbar_s, phase);
-                if (!done && issued) done = mbar_wait(mbar_s, phase);
-                ok = done;
-            }
-            ok = __syncthreads_and(ok);
-            if (!ok && tid == 0) atomicOr(&g_tc_error, 1);
-            phase ^= 1;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        have_rho = have_rho && ok;
-    } else {
-        // blocks next to the poles have more samples per pair than the cosine table holds:
-        // their coefficients were tabulated before this launch, or are generated here on the
-        // CUDA cores; either way they go to the same tensor-memory columns, 16 at a time
-        const bool tab = tabulated;
-        const float *pr = a.prho[kid];
-#pragma unroll 1
-        for (int h = 0; h < G * kTcBand; h += 16) {
-            const int cb = G * grp * kTcBand + h;  // first of 16 columns (one ring's half)
-            float r[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int c = cb + u;
-                float x = 0.f;
-                if (mv && s_S[c] >= 0)
-                    x = tab ? __ldg(&pr[(int64_t)s_p[c] * a.NH + m])
-                            : gen_rho(reinterpret_cast<const float4 *>(taps + s_toff[c]), s_S[c], s_f[c], m, a.N);
-                r[u] = x;
-            }
-            tmem_st16(colg + (uint32_t)h, r);
-        }
-    }
-    const int joff = jg0 - ju0;  // the group's first input ring within the staged band
-    __syncthreads();
 
-    // ---- band contraction.  The union band of each map goes to shared memory by 16-byte
-    // asynchronous copies that every thread issues (the copy engine of one thread per CTA
-    // cannot keep enough bytes in flight); rows beyond the band stay zero, so every group
-    // runs its 32 slots unpredicated (its coefficients are zero there).  nbuf == 2: the next
-    // map is copied while this one is contracted; nbuf == 1: one buffer (the 8-ring form that
-    // keeps two CTAs on an SM, or bands too wide for two).
+    // blocks whose pairs all have tabulated coefficients read them (whatever the block size,
+    // so both block sizes give the same result)
+    const bool tabulated = kd.pstart[r0 + nr] <= kd.polar_pairs;
+    // once any CTA has seen an expired wait the results are invalid anyway: skip the MMAs
+    bool ok = *((volatile int *)&g_tc_error) == 0;
+    uint32_t ph = 0;  // bit s: parity of the next completion of stage s
+
+    // ---- staged spectra: rows of the window's input rings, copied by 16-byte asynchronous
+    // copies that every thread issues (the copy engine of one thread per CTA cannot keep enough
+    // bytes in flight).  nbuf == 2: the next map is copied while this one is contracted;
+    // nbuf == 1: one buffer.  Rows past the band read as zero, so every group runs its slots
+    // unpredicated (its coefficients are zero there).  rows0 > 0: the first buffer lies past the
+    // first stage of the operands, so that the first map is copied while a single pass generates
+    // the coefficients.
     const int mid = (a.R - 1) / 2;
-    const bool crosses = ju0 + nu - 1 > mid;
-    const int sstar = mid - jg0 + 1;  // first slot of the group's run that is a southern ring
-    const size_t bufsz = (size_t)srows * kTcModes;
-    const int m0 = blockIdx.x * kTcModes;
-    for (size_t e = tid; e < (size_t)nbuf * bufsz; e += blockDim.x) sh4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    auto issue = [&](int bb, int q) {
-        stage_band_async(sh4 + q * bufsz, map_spec4(a, bb), ju0, nu, m0, kTcModes, a.R, a.NH);
+    const int row_bytes = kTcModes * (int)sizeof(float4);
+    const uint32_t off0 = rows0, off1 = rows0 ? 0 : srows * row_bytes;
+    auto issue = [&](int w, int bb, int q) {
+        const int j0 = ju0 + w * kTcBand;
+        stage_rows<Sh::kThreads>(reinterpret_cast<float4 *>(smem + (q ? off1 : off0)), map_spec4(a, bb), j0,
+                                 min(srows, jlast - j0 + 1), m0, a.R, a.NH);
     };
-    if (b0 < b1) issue(b0, 0);
-    for (int b = b0; b < b1; ++b) {
-        const int cur = nbuf == 2 ? (b - b0) & 1 : 0;
-        if (nbuf == 2 && b + 1 < b1) {
-            issue(b + 1, cur ^ 1);
-            cp_async_wait1();  // this map's copies (all but the newest group) have landed
-        } else {
-            asm volatile("cp.async.wait_all;" ::: "memory");
+    const int joff = jg0 - ju0;  // the group's first row within the staged rows
+    float4 acc[G];
+#pragma unroll
+    for (int t = 0; t < G; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool fresh = true;  // nothing contracted yet
+    auto put = [&](int b) {
+        if (!mv) return;
+        float2 *cb = a.c + (int64_t)b * a.R * a.NH + m;
+#pragma unroll
+        for (int t = 0; t < G; ++t) {
+            const int i = i0 + t;
+            if (G * grp + t < nr) {
+                cb[(int64_t)i * a.NH] = make_float2(acc[t].x, acc[t].y);
+                if (a.R - 1 - i != i) cb[(int64_t)(a.R - 1 - i) * a.NH] = make_float2(acc[t].z, acc[t].w);
+            }
+        }
+    };
+
+    for (int w = 0; w < nwin; ++w) {
+        // ---- the window's columns
+        for (int c = tid; c < kTcN; c += blockDim.x) {
+            const int tile = c / kTile, l = c % kTile / 16, u = 2 * (c & 15) + ((tile + l) & 1);
+            int toff = 0, S = -1, f = 0, p = 0;
+            if constexpr (WIDE) {
+                const int lg = l - l % G;
+                if (l < nr) {
+                    const int jl = kd.jlo[r0 + l], j = kd.jlo[r0 + lg] + w * kTcBand + u;
+                    if (j >= jl && j <= kd.jhi[r0 + l]) {
+                        p = kd.pstart[r0 + l] + j - jl;
+                        toff = kd.toff[p];
+                        f = a.shift_fix ? kd.fl[p] : 0;
+                        S = f ? kd.S1[p] : kd.S0[p];
+                    }
+                }
+            } else {
+                // the table of columns is laid out per block of 8 rings
+                const int blk8 = blockIdx.y * (RB / 8) + l / 8;
+                const int4 *ct = G == 2 ? kd.coltab : kd.coltab4;
+                const int4 e = 8 * blk8 < a.nrep ? __ldg(&ct[(size_t)blk8 * 256 + (l & 7) * kTcBand + u])
+                                                 : make_int4(-1, 0, -1, -2);
+                if (e.x >= 0) {
+                    p = e.x;
+                    toff = e.y;
+                    f = a.shift_fix ? (e.w & 1) : 0;
+                    S = f ? (e.w >> 1) : e.z;
+                }
+            }
+            if (S >= 0) atomicMax(&s_kmax[tile][f], S + 1);
+            s_toff[c] = toff;
+            s_S[c] = 2 * S + f;
+            s_p[c] = p;
         }
         __syncthreads();
-        float4 acc[G];
+        const int k00 = s_kmax[0][0], k01 = s_kmax[0][1], k10 = s_kmax[1][0], k11 = s_kmax[1][1];
+        const int kall = max(max(k00, k01), max(k10, k11));
+        // tiles of one offset each: one pass serves both
+        const bool single = !(k00 && k01) && !(k10 && k11);
+        const int f0s = k01 ? 1 : 0, f1s = k11 ? 1 : 0;
+        // runs of up to 128 samples (0: no samples in the window; the narrow form is launched
+        // with at most one)
+        const int nrun = tabulated ? 1 : (WIDE ? (kall + kTcRun - 1) / kTcRun : min(kall, 1));
+        bool early = false;
+        for (int run = 0; run < nrun; ++run) {
+            bool have = true;
+            if (!tabulated) {
+                // passes of this run: (first sample, offset of tile 0, offset of tile 1).  The
+                // accumulator truncates each addition at the size of the running sum, so what is
+                // small comes first: the last samples of a run (a beam's tail) before the first,
+                // and the cross terms of a pass before its hi x hi products
+                const int kb = run * kTcRun;
+                auto cap = [&](int k) { return max(0, min(kTcRun, k - kb)); };
+                const int n0 = single ? (cap(kall) + kTcK - 1) / kTcK : (cap(max(k00, k10)) + kTcK - 1) / kTcK;
+                const int np = single ? n0 : n0 + (cap(max(k01, k11)) + kTcK - 1) / kTcK;
+                early = rows0 != 0 && np == 1 && b0 < b1;
+                // a thread takes 8 samples of a column, loaded four at a time (tap offsets are
+                // multiples of 4 and each pair's slots are padded to 4, so a float4 that starts at
+                // or before the last sample stays inside the pair); others read as zero
+                constexpr int kUnits = 2 * kTcN / Sh::kThreads;
+                float4 pre[kUnits][2];
+                auto load_taps = [&](int i) {
+                    const bool second = !single && i >= n0;
+                    const int k0 = kb + (second ? np - 1 - i : n0 - 1 - i) * kTcK;
 #pragma unroll
-        for (int t = 0; t < G; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (v0 && have_rho) {  // warp-uniform: the tensor-memory loads are warp-collective
-            const float4 *col = sh4 + cur * bufsz + joff * kTcModes + mrow;
-            // slots in chunks of CH: the chunk's coefficients of the G rings, then CH staged
-            // values, each used by all G rings
-            constexpr int CH = G == 2 ? 16 : 8;
+                    for (int u = 0; u < kUnits; ++u) {
+                        const int e = tid + u * Sh::kThreads, c = e % kTcN, kk = k0 + 8 * (e / kTcN);
+                        const int fp = single ? (c < kTile ? f0s : f1s) : (int)second;
+                        const int sf = s_S[c], S = (sf & 1) == fp ? sf >> 1 : -1;
+                        const float *tp = taps + s_toff[c] + kk;
 #pragma unroll
-            for (int h = 0; h < kTcBand; h += CH) {
-                uint32_t cr[G][CH];
-#pragma unroll
-                for (int t = 0; t < G; ++t) tmem_ld_async(colg + (uint32_t)(t * kTcBand + h), cr[t]);
-                tmem_wait_ld();
-                if (!crosses) {
-#pragma unroll
-                    for (int u = 0; u < CH; ++u) {
-                        const float4 v = col[(h + u) * kTcModes];
-#pragma unroll
-                        for (int t = 0; t < G; ++t) fma4(acc[t], __uint_as_float(cr[t][u]), v);
+                        for (int q = 0; q < 2; ++q)
+                            pre[u][q] = kk + 4 * q <= S ? __ldg(reinterpret_cast<const float4 *>(tp + 4 * q))
+                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
+                };
+                uint32_t pend = 0;    // bit s: a pass of stage s not yet seen complete
+                uint32_t issued = 0;  // bit s: its MMAs were issued
+                auto await = [&](int st) {
+                    if (pend >> st & 1) {
+                        if (ok) {
+                            bool done = mbar_wait(mbar_s + 8u * st, (ph >> st) & 1);
+                            // an issued commit is waited for once more (bounded) before anything
+                            // reuses the memory its MMAs use
+                            if (!done && (issued >> st & 1)) done = mbar_wait(mbar_s + 8u * st, (ph >> st) & 1);
+                            if (!done) atomicOr(&g_tc_error, 1);
+                            ok = done;
+                        } else if (issued >> st & 1) {
+                            (void)mbar_wait(mbar_s + 8u * st, (ph >> st) & 1);
+                        }
+                        ph ^= 1u << st;
+                        pend &= ~(1u << st);
+                    }
+                };
+                bool first = true;
+                load_taps(0);
+                for (int i = 0; i < np; ++i) {
+                    const int st = Sh::kStages == 2 ? (i & 1) : 0;
+                    const bool second = !single && i >= n0;
+                    const int k0 = kb + (second ? np - 1 - i : n0 - 1 - i) * kTcK;  // first sample of the pass
+                    const int fA = single ? f0s : (int)second, fB = single ? f1s : (int)second;
+                    const int krem = (single ? kall : (second ? max(k01, k11) : max(k00, k10))) - k0;
+                    const int ksteps = krem > 8 ? 2 : 1;
+                    unsigned char *A = smem + st * Sh::kStage, *Bh = A + 4 * Sh::kA, *Bl = Bh + Sh::kB;
+                    await(st);  // the MMAs of the pass that used this stage
+                    // A: this mode block's cosines of the pass (hi, lo), for tile 1 apart when its
+                    // offset differs
+                    const int ncos = fA == fB ? 1 : 2;
+                    if (!WIDE || k0 < nkc_tab * 32) {
+                        // prepared in the core layout, 32 samples to a tile
+                        const int lp = 3 + ksteps;  // 16 or 32 16-byte units of a row octet
+                        for (int e = tid; e < ncos << (lp + 5); e += Sh::kThreads) {
+                            const int wi = e & ((1 << lp) - 1), oct = e >> lp & 15, part = e >> (lp + 4);  // 2 tile + lo
+                            const float *src = ctab +
+                                ((((size_t)blockIdx.x * 2 + (part >> 1 ? fB : fA)) * nkc_tab + (k0 >> 5)) * 2 + (part & 1)) * 4096;
+                            cp_async16(A + part * Sh::kA + oct * kTcSBO + wi * 16,
+                                       src + oct * 256 + (k0 & 16) * 8 + wi * 4, 16);
+                        }
+                    } else {
+                        // past the tables: the exact values of cos(pi t / N), t = m (2k + f) mod 2N
+                        const bool pow2 = (a.N & (a.N - 1)) == 0;
+                        for (int e = tid; e < ncos * kTcModes * kTcK; e += Sh::kThreads) {
+                            const int x = e % (kTcModes * kTcK), tl = e / (kTcModes * kTcK);
+                            const int k = (x & 3) + 4 * (x >> 5 & 3), r = (x >> 2 & 7) + 8 * (x >> 7);
+                            const int ang = (m0 + r) * (2 * (k0 + k) + (tl ? fB : fA));
+                            const float2 v = __ldg(&cos2n[pow2 ? ang & (2 * a.N - 1) : ang % (2 * a.N)]);
+                            const uint32_t off = (r >> 3) * kTcSBO + (k >> 2) * kLBO + (r & 7) * 16 + (k & 3) * 4;
+                            *reinterpret_cast<float *>(A + 2 * tl * Sh::kA + off) = v.x;
+                            *reinterpret_cast<float *>(A + (2 * tl + 1) * Sh::kA + off) = v.y;
+                        }
+                    }
+                    cp_async_commit();
+                    // B: the samples of every column for its tile's offset, split hi / lo
+#pragma unroll
+                    for (int u = 0; u < kUnits; ++u) {
+                        const int e = tid + u * Sh::kThreads, c = e % kTcN, ks = e / kTcN;
+                        if (ks >= ksteps) continue;
+                        const int sf = s_S[c], kk = k0 + 8 * ks;
+                        const uint32_t off = (c >> 3) * kTcSBO + 2 * ks * kLBO + (c & 7) * 16;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const float v[4] = {pre[u][q].x, pre[u][q].y, pre[u][q].z, pre[u][q].w};
+                            float4 hi4, lo4;
+                            float *hp = &hi4.x, *lp = &lo4.x;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float x = kk + 4 * q + j <= (sf >> 1) ? v[j] : 0.f;
+                                hp[j] = tf32_round(x);
+                                lp[j] = tf32_round(x - hp[j]);
+                            }
+                            *reinterpret_cast<float4 *>(Bh + off + q * kLBO) = hi4;
+                            *reinterpret_cast<float4 *>(Bl + off + q * kLBO) = lo4;
+                        }
+                    }
+                    if (i + 1 < np) load_taps(i + 1);
+                    if (early) issue(w, b0, 0);
+                    else cp_async_commit();
+                    cp_async_wait1();  // the cosines have landed (all but the newest group)
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    ok = __syncthreads_and(ok);
+                    // CTA-uniform: whether this pass's MMAs and their commit are issued (the test
+                    // knob withholds them, so that the wait runs out)
+                    const bool go = ok && !a.withhold_mma;
+                    if (ok) pend |= 1u << st;
+                    issued = go ? issued | (1u << st) : issued & ~(1u << st);
+                    if (tid == 0 && go) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        constexpr uint32_t idesc = tf32_idesc(kTcModes, kTile);
+                        const uint32_t sa = smem_s + st * Sh::kStage, sb = sa + 4 * Sh::kA;
+#pragma unroll 1
+                        for (int x = 0; x < 3 * ksteps; ++x) {  // C_lo T_hi, C_hi T_lo, C_hi T_hi
+                            const int prod = x / ksteps, ks = ksteps - 1 - x % ksteps;
+                            const uint32_t o = ks * 2 * kLBO;  // 8 TF32 values = two core columns
+#pragma unroll
+                            for (int t = 0; t < 2; ++t) {
+                                const uint32_t ca = sa + (t && ncos == 2 ? 2 * Sh::kA : 0) + (prod == 0 ? Sh::kA : 0) + o;
+                                const uint32_t cb = sb + (uint32_t)t * (kTile / 8) * kTcSBO + (prod == 1 ? Sh::kB : 0) + o;
+                                mma_tf32(tmem + (uint32_t)(t * kTile), smem_desc(ca, kTcSBO), smem_desc(cb, kTcSBO),
+                                         idesc, first ? 0 : 1);
+                            }
+                            first = false;
+                        }
+                        mma_commit(mbar_s + 8u * st);
+                    }
+                }
+                for (int st = 0; st < Sh::kStages; ++st) await((np + st) % Sh::kStages);
+                ok = __syncthreads_and(ok);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                have = ok;
+            } else {
+                // blocks next to the poles have more samples per pair than the cosine tables hold:
+                // their coefficients were tabulated before this launch; they go to the same
+                // tensor-memory columns, a ring's 16 slots at a time
+                const float *pr = a.prho[kid];
+#pragma unroll 1
+                for (int h = 0; h < G * 2; ++h) {
+                    const int l = G * grp + h / 2, c0 = l * 16 + (h & 1) * 8;
+#pragma unroll
+                    for (int tile = 0; tile < 2; ++tile) {
+                        float r[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const int c = tile * kTile + c0 + u;
+                            r[u] = mv && s_S[c] >= 0 ? __ldg(&pr[(int64_t)s_p[c] * a.NH + m]) : 0.f;
+                        }
+                        tmem_st8(lane_base + (uint32_t)(tile * kTile + c0), r);
+                    }
+                }
+                __syncthreads();
+            }
+
+            // ---- band contraction of the window's slots, for every map
+            const int jw = jg0 + w * kTcBand;     // input ring of the group's first slot
+            const int sstar = mid - jw + 1;       // first slot that is a southern ring
+            const bool crosses = jlast > mid;
+            // whole windows inside the band of every ring of the group run without a test; at the
+            // ends of a wide band a slot outside a ring's band is left out (a non-finite input
+            // ring reaches only outputs whose support holds it)
+            int lo[G], hi[G];
+            bool inner = true;
+            if constexpr (WIDE) {
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    const int i = r0 + min(G * grp + t, nr - 1);
+                    lo[t] = kd.jlo[i] - jw;
+                    hi[t] = kd.jhi[i] - jw;
+                    inner = inner && lo[t] <= 0 && hi[t] >= kTcBand - 1;
+                }
+            }
+            if (!early && b0 < b1) issue(w, b0, 0);
+            // the rows past the band read as zero
+            for (int e = min(srows, jlast - ju0 - w * kTcBand + 1) * kTcModes + tid; e < srows * kTcModes; e += Sh::kThreads) {
+                reinterpret_cast<float4 *>(smem + off0)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (nbuf == 2) reinterpret_cast<float4 *>(smem + off1)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            for (int b = b0; b < b1; ++b) {
+                const int cur = nbuf == 2 ? (b - b0) & 1 : 0;
+                if (nbuf == 2 && b + 1 < b1) {
+                    issue(w, b + 1, cur ^ 1);
+                    cp_async_wait1();  // this map's copies (all but the newest group) have landed
                 } else {
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                }
+                __syncthreads();
+                // outputs of earlier windows and runs: in registers for one map, else written by
+                // this thread before
+                if (!WIDE || fresh) {
 #pragma unroll
-                    for (int u = 0; u < CH; ++u) {
-                        float4 v = col[(h + u) * kTcModes];
-                        if (h + u >= sstar) v = make_float4(v.z, v.w, v.x, v.y);
+                    for (int t = 0; t < G; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                } else if (b1 - b0 > 1 && mv) {
+                    const float2 *cb = a.c + (int64_t)b * a.R * a.NH + m;
 #pragma unroll
-                        for (int t = 0; t < G; ++t) fma4(acc[t], __uint_as_float(cr[t][u]), v);
+                    for (int t = 0; t < G; ++t) {
+                        const int i = i0 + t;
+                        if (G * grp + t < nr) {
+                            const float2 x = cb[(int64_t)i * a.NH], y = cb[(int64_t)(a.R - 1 - i) * a.NH];
+                            acc[t] = make_float4(x.x, x.y, y.x, y.y);
+                        }
                     }
                 }
-            }
-        }
-        if (mv) {
-            float2 *cb = a.c + (int64_t)b * a.R * a.NH + m;
+                if (v0 && have) {  // warp-uniform: the tensor-memory loads are warp-collective
+                    const float4 *col = reinterpret_cast<const float4 *>(smem + (cur ? off1 : off0)) + joff * kTcModes + mrow;
+                    // CH slots at a time, in the order of the input rings (whatever the groups): the
+                    // coefficients of the G rings (a ring's even and odd slots lie in different
+                    // tiles), then the staged values, each used by all G rings
+                    constexpr int CH = 8, UNROLL = WIDE ? 1 : kTcBand / CH;  // (wide: less code, 4.5 against 5.1 ms)
+#pragma unroll(UNROLL)
+                    for (int h = 0; h < kTcBand; h += CH) {
+                        uint32_t cr[G][2][CH / 2];
 #pragma unroll
-            for (int t = 0; t < G; ++t) {
-                const int i = i0 + t;
-                if (G * grp + t < nr) {
-                    cb[(int64_t)i * a.NH] = make_float2(acc[t].x, acc[t].y);
-                    if (a.R - 1 - i != i) cb[(int64_t)(a.R - 1 - i) * a.NH] = make_float2(acc[t].z, acc[t].w);
+                        for (int t = 0; t < G; ++t)
+#pragma unroll
+                            for (int o = 0; o < 2; ++o)
+                                tmem_ld_async(lane_base + (uint32_t)(((t + o) & 1) * kTile + (G * grp + t) * 16 + h / 2),
+                                              cr[t][o]);
+                        tmem_wait_ld();
+                        if (!crosses && (!WIDE || inner)) {
+#pragma unroll
+                            for (int u = 0; u < CH; ++u) {
+                                const float4 v = col[(h + u) * kTcModes];
+#pragma unroll
+                                for (int t = 0; t < G; ++t) fma4(acc[t], __uint_as_float(cr[t][u & 1][u >> 1]), v);
+                            }
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < CH; ++u) {
+                                float4 v = col[(h + u) * kTcModes];
+                                if (h + u >= sstar) v = make_float4(v.z, v.w, v.x, v.y);
+#pragma unroll
+                                for (int t = 0; t < G; ++t)
+                                    if (!WIDE || (h + u >= lo[t] && h + u <= hi[t]))
+                                        fma4(acc[t], __uint_as_float(cr[t][u & 1][u >> 1]), v);
+                            }
+                        }
+                    }
                 }
+                if (!WIDE || b1 - b0 > 1) put(b);
+                __syncthreads();
+                if (nbuf == 1 && b + 1 < b1) issue(w, b + 1, 0);
             }
+            fresh = false;
         }
-        __syncthreads();
-        if (nbuf == 1 && b + 1 < b1) issue(b + 1, 0);
+        if (WIDE && w + 1 < nwin) {
+            if (tid < 4) s_kmax[tid >> 1][tid & 1] = 0;
+            __syncthreads();
+        }
     }
+    // the wide form's sums of one map were kept in registers; no samples at all: zero outputs
+    if (fresh || (WIDE && b1 - b0 == 1))
+        for (int b = b0; b < b1; ++b) put(b);
 
     // ---- release tensor memory
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Sh::kTmemCols));
 }
 
 // Knot-gradient projection on the tensor cores (the 3xTF32 form of the backward pass):
@@ -548,52 +711,82 @@ k_knot_proj_tc(KnotGradArgs a, const float *__restrict__ Q, const float *__restr
 
 }  // namespace
 
-int contract_tc_kchunks(int max_taps) { return (max_taps + kTcKChunk - 1) / kTcKChunk; }
 int contract_tc_modes() { return kTcModes; }
 
 constexpr size_t kTcSmemLimit = 216 * 1024;  // dynamic shared memory of a one-CTA-per-SM launch
+constexpr size_t kTcRow = (size_t)kTcModes * sizeof(float4);
 
 // Staging buffers of srows rows for blocks of rb rings in groups of gs.  Two CTAs per SM
-// (rb == 8): by default two buffers when they fit in the operand area, else one; `want` (1 or
-// 2) overrides when it fits in 200 KiB.  One CTA per SM (rb == 16): two when they fit.
+// (rb == 8): one, unless `want` == 2 and two fit in 200 KiB.  One CTA per SM (rb == 16): two when
+// they fit.
 int contract_tc_nbuf(int rb, int gs, int srows, int want)
 {
-    const size_t row = (size_t)kTcModes * sizeof(float4);
-    if (rb == 16) return 2 * srows * row + 32 <= kTcSmemLimit ? 2 : 1;
-    if (want == 1) return 1;
-    if (want == 2 && 2 * srows * row + 32 <= 200 * 1024) return 2;
-    return 2 * srows * row <= (gs == 2 ? TcShape<8, 2>::kAB : TcShape<8, 4>::kAB) ? 2 : 1;
+    (void)gs;
+    if (rb == 16) return 2 * srows * kTcRow + 32 <= kTcSmemLimit ? 2 : 1;
+    return want == 2 && 2 * srows * kTcRow + 32 <= 200 * 1024 ? 2 : 1;
 }
+
+namespace {
+
+// Offset of the first staging buffer: past the first operand stage where two buffers (the
+// second over that stage) fit a CTA that has the SM to itself.
+uint32_t tc_rows0(int rb, int srows)
+{
+    const uint32_t st = TcShape<16, 4>::kStage;
+    return rb == 16 && srows * kTcRow <= st && st + srows * kTcRow + 32 <= kTcSmemLimit ? st : 0;
+}
+
+// Offset of the barriers behind the operand stages and the staging buffers.
+size_t tc_ctl(int rb, int nbuf, int srows)
+{
+    const uint32_t rows0 = tc_rows0(rb, srows);
+    const size_t stages = rb == 16 ? 2 * (size_t)TcShape<16, 4>::kStage : (size_t)TcShape<8, 4>::kStage;
+    const size_t rows = rows0 ? rows0 + srows * kTcRow : nbuf * srows * kTcRow;
+    return (std::max(stages, rows) + 15) & ~size_t(15);
+}
+
+}  // namespace
 
 size_t contract_tc_smem(int rb, int gs, int srows, int want_nbuf)
 {
-    const size_t stage_bytes = (size_t)contract_tc_nbuf(rb, gs, srows, want_nbuf) * srows * kTcModes * sizeof(float4);
-    const size_t ab_bytes = rb == 16 ? TcShape<16, 2>::kAB : TcShape<8, 2>::kAB;
-    return (((stage_bytes > ab_bytes ? stage_bytes : ab_bytes) + 15) & ~size_t(15)) + 32;
+    return tc_ctl(rb, contract_tc_nbuf(rb, gs, srows, want_nbuf), srows) + 32;
 }
 
-template <int RB, int G>
-cudaError_t launch_tc(const ContractArgs &a, int nchunks, const float *ctab, int nkc_tab, int srows, int nbuf,
-                      size_t smem, cudaStream_t st)
+// Whether blocks of 16 rings with moving windows of srows staged rows fit an SM.
+bool contract_tc_wide_fits(int srows) { return contract_tc_smem(16, 4, srows, 0) <= kTcSmemLimit; }
+
+namespace {
+
+template <int RB, int G, bool WIDE>
+cudaError_t launch_tc(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, int nbuf, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_tc<RB, G>,
+    const size_t ctl = tc_ctl(RB, nbuf, srows), smem = ctl + 32;
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_tc<RB, G, WIDE>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.NH + kTcModes - 1) / kTcModes, (a.nrep + RB - 1) / RB, nchunks);
-    k_contract_tc<RB, G><<<grid, TcShape<RB, G>::kThreads, smem, st>>>(a, ctab, nkc_tab, srows, nbuf);
+    k_contract_tc<RB, G, WIDE><<<grid, TcShape<RB, G>::kThreads, smem, st>>>(a, tb.ctab, tb.cos2n, tb.nkc, srows, nbuf,
+                                                                             tc_rows0(RB, srows), (uint32_t)ctl);
     return cudaGetLastError();
 }
 
-cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, int nchunks, const float *ctab, int nkc_tab,
-                               int srows, int want_nbuf, cudaStream_t st)
+}  // namespace
+
+cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, int nchunks, const TcTables &tb, int srows,
+                               int want_nbuf, cudaStream_t st)
 {
-    const size_t smem = contract_tc_smem(rb, gs, srows, want_nbuf);
     const int nbuf = contract_tc_nbuf(rb, gs, srows, want_nbuf);
     if (rb == 16)
-        return gs == 4 ? launch_tc<16, 4>(a, nchunks, ctab, nkc_tab, srows, nbuf, smem, st)
-                       : launch_tc<16, 2>(a, nchunks, ctab, nkc_tab, srows, nbuf, smem, st);
-    return gs == 4 ? launch_tc<8, 4>(a, nchunks, ctab, nkc_tab, srows, nbuf, smem, st)
-                   : launch_tc<8, 2>(a, nchunks, ctab, nkc_tab, srows, nbuf, smem, st);
+        return gs == 4 ? launch_tc<16, 4, false>(a, nchunks, tb, srows, nbuf, st)
+                       : launch_tc<16, 2, false>(a, nchunks, tb, srows, nbuf, st);
+    return gs == 4 ? launch_tc<8, 4, false>(a, nchunks, tb, srows, nbuf, st)
+                   : launch_tc<8, 2, false>(a, nchunks, tb, srows, nbuf, st);
+}
+
+// Bands of any width: blocks of 16 rings in groups of four, the 32 slots moving along the band.
+cudaError_t launch_contract_tc_wide(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, cudaStream_t st)
+{
+    return launch_tc<16, 4, true>(a, nchunks, tb, srows, contract_tc_nbuf(16, 4, srows, 0), st);
 }
 
 // Knot-gradient projection of pairs [pfirst, npairs) into X [npairs - pfirst][128] (rows of

@@ -16,7 +16,8 @@ constexpr uint64_t kTcTimeoutNs = 1000000000ull;
 constexpr uint32_t kTcMaxPolls = 1u << 26;
 
 // no-swizzle K-major tensor-core layout: 8-row x 16-byte core matrices, contiguous; core
-// matrices adjacent in K are 128 bytes apart (LBO), adjacent in M/N 1024 bytes apart (SBO)
+// matrices adjacent in K are 128 bytes apart (LBO), adjacent in M/N 1024 bytes apart (SBO, for
+// operands of 32 samples; others give theirs)
 constexpr uint32_t kLBO = 128, kSBO = 1024;
 
 __device__ __forceinline__ uint32_t core_offset(int row, int k)
@@ -24,11 +25,12 @@ __device__ __forceinline__ uint32_t core_offset(int row, int k)
     return (uint32_t)((row >> 3) * kSBO + (k >> 2) * kLBO + (row & 7) * 16 + (k & 3) * 4);
 }
 
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr)
+// descriptor of an operand whose row octets are sbo bytes apart
+__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t sbo = kSBO)
 {
     uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
     d |= (uint64_t)((kLBO >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((kSBO >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
     d |= (uint64_t)1 << 46;  // descriptor version
     return d;                // base offset 0, no swizzle
 }
@@ -86,7 +88,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase)
     return false;
 }
 
-// 32 lanes x n columns (n = 8 or 16) from tensor memory; the registers are valid after
+// 32 lanes x n columns (n = 4, 8 or 16) from tensor memory; the registers are valid after
 // tmem_wait_ld().
 __device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[16])
 {
@@ -107,21 +109,23 @@ __device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[8])
                  : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 32 lanes x 16 columns into tensor memory, completed before returning
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
+// 32 lanes x 8 columns into tensor memory, completed before returning
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8])
 {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-        ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-          "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-          "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-          "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-          "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-          "r"(__float_as_uint(v[15]))
-        : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                   "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+                   "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+                 : "memory");
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
