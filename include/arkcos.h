@@ -146,10 +146,10 @@ arkcos_status arkcos_multi_workspace_size(arkcos_grid grid, const arkcos_kernel 
  * `grid`):
  *   weights == NULL:  map_out[b][k] = L(kernels[k]) map_in[b]          ([nmaps][nkernels][npix]);
  *   weights != NULL:  map_out[b] = sum_k weights[k] L(kernels[k]) map_in[b]   ([nmaps][npix]),
- *                     weights a HOST array of nkernels FP64 values (used as FP32), the sum
- *                     formed on the kernel-grid coefficients in kernel order before one
- *                     inverse ring transform per map (the pole rings sum the kernels' direct
- *                     sums the same way).
+ *                     weights a HOST array of nkernels FP64 values (used as FP32): the
+ *                     kernels' weighted samples are summed, in kernel order, over the ring
+ *                     pairs of the widest one, and one convolution per map follows (the pole
+ *                     rings sum the kernels' direct sums).
  * map_in and map_out are DEVICE FP32 and must not overlap.  1 <= nkernels <= 256 (32 with
  * weights), nmaps x nkernels <= 256.  The workspace (DEVICE, 256-byte aligned) holds at least
  * arkcos_multi_workspace_size() bytes.  Enqueued on `stream`, no host synchronisation, no

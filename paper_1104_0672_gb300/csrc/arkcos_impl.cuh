@@ -97,6 +97,7 @@ struct KernDev {
     int nunit_fix, nunit_nofix;
     int T;
     int npairs;
+    int nrep;            // representative output rings
     int polar_pairs;     // pairs [0, polar_pairs) (rings next to the poles with many samples)
                          // take their coefficients from a table computed before the contraction
     double umax;
@@ -112,6 +113,7 @@ struct Kernel {
     int maxband = 0;
     int maxS = 0;
     int pole_band = 0;         // input rings inside the support of ring 0
+    int64_t pole_pixels = 0;   // their pixels
     int max_union8 = 0;        // largest union band of 8 consecutive representative rings
     int max_union2 = 0;        // largest union band of rings 2g, 2g+1 of those blocks of 8
     int max_stage_rows = 0;    // staged rows a tensor-core block of 8 rings needs: its union
@@ -131,12 +133,15 @@ struct Kernel {
 
 // ------------------------------------------------------------------ launch arguments
 struct TapArgs {
-    KernDev kd;
+    KernDev kd[kMaxKernelsPerLaunch];
+    float *taps[kMaxKernelsPerLaunch];  // [ntaps] of each kernel
     const double *s2;
     const float *s2f;
-    float *taps;   // [ntaps]
     int N;
     int shift_fix;
+    // ksum > 0: the samples of sum_k w[k] K_k, k < ksum, over the pairs of kernel kbase (the widest)
+    int ksum, kbase;
+    float w[kMaxKernelsPerLaunch];
 };
 
 struct FftFwdArgs {
@@ -170,6 +175,7 @@ struct FftInvArgs {
     int skip_poles;     // leave rings 0 and R-1 untouched (written by the pole kernel)
     int stage_c;        // stage coefficients in shared memory for rings with 4 n < N
     int tab;            // shared-memory words for the per-ring chirp and phase tables
+    int first;          // first class of the stage: its input comes from the kernel before it
 };
 
 struct ContractArgs {
@@ -237,7 +243,9 @@ __device__ __forceinline__ float4 paired_coeff(const float4 *__restrict__ sp4, i
 }
 
 // ------------------------------------------------------------------ launchers (return cuda error)
-cudaError_t launch_taps(const TapArgs &a, int npairs, cudaStream_t st);
+// Kernel samples of nk kernels (or the weighted sum, a.ksum); maxtaps: most tap slots of one.
+// after_prev: may begin while the kernel before it on the stream still runs.
+cudaError_t launch_taps(const TapArgs &a, int nk, int64_t maxtaps, cudaStream_t st, bool after_prev);
 cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs, const float2 *tw, int twM,
                              cudaStream_t st);
 size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads, bool split);  // shared memory of a ring FFT class
@@ -251,29 +259,39 @@ int fft_map_chunk(int count, int nmaps, int split_mult);  // maps per CTA of a r
 cudaError_t launch_fft_inv(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
 cudaError_t launch_fft_inv_split(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
 
-// Launch of kernel(a) with the programmatic-serialization attribute when after_prev.
-template <class Args>
-cudaError_t launch_class_kernel(void (*kernel)(Args), dim3 grid, int threads, size_t smem, cudaStream_t st,
-                                bool after_prev, const Args &a)
+// Launch of kernel(args...) in clusters of `cluster` CTAs along x, with the
+// programmatic-serialization attribute when after_prev: the kernel may then begin while the
+// kernel before it on the stream still runs, once all CTAs of that one have started and allowed
+// it, and waits for it (chain_wait) before it reads its results and before it ends, so that the
+// end of every kernel of a chain is the end of all before it.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                           bool after_prev, int cluster, const A &...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (after_prev) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = (unsigned)cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = after_prev ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 cudaError_t launch_contract(const ContractArgs &a, int nchunks, size_t smem, cudaStream_t st);
-cudaError_t launch_pole_fwd(const PoleArgs &a, cudaStream_t st);
-// csum[b] = sum_k w[k] c[b K + k] for b < nmaps ([R][NH] complex coefficient arrays), the sum
-// taken in order of k
-cudaError_t launch_weighted_sum(const float2 *c, float2 *csum, int64_t nmaps, int K, const double *w,
-                                int64_t per_map, cudaStream_t st);
+// band_pixels: pixels of the rings inside the support of a pole
+cudaError_t launch_pole_fwd(const PoleArgs &a, int64_t band_pixels, cudaStream_t st, bool after_prev);
 cudaError_t launch_pole_adj(const PoleArgs &a, int max_band_rings, cudaStream_t st);
 cudaError_t launch_knot_grad_q(const KnotGradArgs &a, float *Q, int max_band, int max_union, int max_union2,
                                int srows, cudaStream_t st);

@@ -32,51 +32,112 @@ constexpr int kMapGroups = 4;   // warp groups per CTA: they split the coefficie
 // u - u_t = 4B c2 + 4A s2 - u_t (two FMAs); the knot segment comes from an FP32 estimate of u
 // (next to a knot the neighbouring segment's line differs by rounding only, the profile being
 // continuous there) and the linear step runs in FP32 on tables pre-scaled by 1 / N.
-__global__ void __launch_bounds__(256) k_taps(TapArgs a)
+//
+// One launch serves every kernel of a call (blockIdx.y).  The pairs' slots are one array, so a
+// warp takes a run of 128-slot tiles and a lane four slots of one pair, found by a binary search
+// from the tile's first pair: most pairs have 6-24 samples, which left most lanes of a warp per
+// pair idle (one 15' kernel at nside 2048 150 -> 40 us, at a degree of support 315 -> 268 us; 64
+// kernels at nside 1024 in 64 launches 3.9 ms, now 0.55 ms).  FP64 bounds it (two FMAs and a
+// conversion per sample at two per SM and clock: 30 us of the 40).  One CTA per SM, as each
+// builds the knot tables with FP64 divisions (two of half the size: 50 us).
+constexpr int kTapThreads = 1024;
+
+__global__ void __launch_bounds__(kTapThreads) k_taps(const __grid_constant__ TapArgs a)
 {
     extern __shared__ double tsm[];
-    const int T = a.kd.T;
-    double *ut = tsm;                                  // [T] knots in u
-    float *utf = reinterpret_cast<float *>(tsm + T);   // [T] the same in FP32
-    float *f = utf + T, *slope = f + T, *span = slope + T;  // [T] profile / N, its slope, knot spacing
-    const double invN = 1.0 / (double)a.N;
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        ut[t] = a.kd.ut[t];
-        utf[t] = (float)a.kd.ut[t];
-        f[t] = (float)(a.kd.knots[t] * invN);
-        if (t < T - 1) {
-            const double du = a.kd.ut[t + 1] - a.kd.ut[t];
-            slope[t] = (float)((a.kd.knots[t + 1] - a.kd.knots[t]) / du * invN);
-            span[t] = (float)du;
-        }
-    }
-    __syncthreads();
+    chain_allow_next();
     const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    const float umaxf = (float)a.kd.umax;
-    for (int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < a.kd.npairs; p += warps) {
-        const int fl = a.shift_fix ? a.kd.fl[p] : 0;
-        const int S = fl ? a.kd.S1[p] : a.kd.S0[p];
-        const int t0 = a.kd.toff[p], t1 = a.kd.toff[p + 1];
-        const double A4 = 4.0 * a.kd.A[p], B4 = 4.0 * a.kd.B[p];
-        const float A4f = (float)A4, B4f = (float)B4;
-        for (int k = lane; k < t1 - t0; k += 32) {
-            float val = 0.f;
-            if (k <= S) {
-                const int t = 2 * k + fl;  // x_k / 2 = pi t / (2N)
-                const float uf = fminf(fmaf(B4f, a.s2f[a.N - t], A4f * a.s2f[t]), umaxf);
-                const int sg = knot_segment_f(uf, utf, T, a.kd.gscale);
-                const double d = fma(B4, a.s2[a.N - t], fma(A4, a.s2[t], -ut[sg]));
-                // u is clamped to u_max: the last segment ends at its knot
-                const float df = fminf((float)d, span[sg]);
-                const float K = fmaf(df, slope[sg], f[sg]);
-                val = (fl == 0 && (k == 0 || 2 * k == a.N)) ? K : 2.f * K;
+    const KernDev &kb = a.kd[a.ksum > 0 ? a.kbase : blockIdx.y];  // whose pairs and slots are filled
+    float *taps = a.taps[a.ksum > 0 ? a.kbase : blockIdx.y];
+    const int slots = kb.toff[kb.npairs], tiles = (slots + 127) / 128;
+    const int warps = gridDim.x * (kTapThreads / 32), per = (tiles + warps - 1) / warps;
+    const int first = (blockIdx.x * (kTapThreads / 32) + (threadIdx.x >> 5)) * per, last = min(tiles, first + per);
+    // last entry of tab[lo..hi] that is <= v (tab ascending, tab[lo] <= v)
+    auto find = [](const int *__restrict__ tab, int lo, int hi, int v) {
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(&tab[mid]) <= v) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    };
+    const int p0 = first < last ? find(kb.toff, 0, kb.npairs - 1, first * 128) : 0;
+    const int nk = a.ksum > 0 ? a.ksum : 1;
+    for (int q = 0; q < nk; ++q) {
+        const KernDev &kd = a.kd[a.ksum > 0 ? q : blockIdx.y];
+        const int T = kd.T;
+        double *ut = tsm;                                  // [T] knots in u
+        float *utf = reinterpret_cast<float *>(tsm + T);   // [T] the same in FP32
+        float *f = utf + T, *slope = f + T, *span = slope + T;  // [T] profile / N, its slope, knot spacing
+        const double invN = 1.0 / (double)a.N;
+        if (q > 0) __syncthreads();
+        for (int t = threadIdx.x; t < T; t += blockDim.x) {
+            ut[t] = kd.ut[t];
+            utf[t] = (float)kd.ut[t];
+            f[t] = (float)(kd.knots[t] * invN);
+            if (t < T - 1) {
+                const double du = kd.ut[t + 1] - kd.ut[t];
+                slope[t] = (float)((kd.knots[t + 1] - kd.knots[t]) / du * invN);
+                span[t] = (float)du;
             }
-            a.taps[t0 + k] = val;
+        }
+        __syncthreads();
+        const float umaxf = (float)kd.umax;
+        int p = p0;
+        for (int tile = first; tile < last; ++tile) {
+            const int s = tile * 128 + 4 * lane;
+            // the pair of this lane's slots: at most 32 pairs with slots begin in a tile, but pairs
+            // without any may lie between them, so the search ends at the last pair
+            int hi = min(p + 32, kb.npairs - 1);
+            if (__ldg(&kb.toff[hi + 1]) <= s) hi = kb.npairs - 1;
+            p = find(kb.toff, p, hi, s);
+            if (s < slots) {
+                const int k0 = s - __ldg(&kb.toff[p]);
+                int S = -1, fl = a.shift_fix ? __ldg(&kb.fl[p]) : 0;
+                if (a.ksum > 0) {
+                    // kernel q's own sample count for the pair's rings (i, j)
+                    const int i = find(kb.pstart, 0, (int)kb.nrep - 1, p), j = __ldg(&kb.jlo[i]) + p - __ldg(&kb.pstart[i]);
+                    const int jl = __ldg(&kd.jlo[i]);
+                    if (j >= jl && j <= __ldg(&kd.jhi[i])) {
+                        const int pq = __ldg(&kd.pstart[i]) + j - jl;
+                        S = fl ? __ldg(&kd.S1[pq]) : __ldg(&kd.S0[pq]);
+                    }
+                } else {
+                    S = fl ? __ldg(&kd.S1[p]) : __ldg(&kd.S0[p]);
+                }
+                const double A4 = 4.0 * __ldg(&kb.A[p]), B4 = 4.0 * __ldg(&kb.B[p]);
+                const float A4f = (float)A4, B4f = (float)B4;
+                float val[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int k = k0 + e;
+                    val[e] = 0.f;
+                    if (k <= S) {
+                        const int t = 2 * k + fl;  // x_k / 2 = pi t / (2N)
+                        const float uf = fminf(fmaf(B4f, __ldg(&a.s2f[a.N - t]), A4f * __ldg(&a.s2f[t])), umaxf);
+                        const int sg = knot_segment_f(uf, utf, T, kd.gscale);
+                        const double d = fma(B4, __ldg(&a.s2[a.N - t]), fma(A4, __ldg(&a.s2[t]), -ut[sg]));
+                        // u is clamped to u_max: the last segment ends at its knot
+                        const float df = fminf((float)d, span[sg]);
+                        const float K = fmaf(df, slope[sg], f[sg]);
+                        val[e] = (fl == 0 && (k == 0 || 2 * k == a.N)) ? K : 2.f * K;
+                    }
+                }
+                float4 *out = reinterpret_cast<float4 *>(taps + s);
+                if (a.ksum > 0) {
+                    const float w = a.w[q];
+                    float4 o = q > 0 ? *out : make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (k0 <= S) o = make_float4(fmaf(w, val[0], o.x), fmaf(w, val[1], o.y), fmaf(w, val[2], o.z), fmaf(w, val[3], o.w));
+                    *out = o;
+                } else {
+                    *out = make_float4(val[0], val[1], val[2], val[3]);
+                }
+            }
+            p = __shfl_sync(0xffffffffu, p, 31);
         }
     }
+    chain_wait();
 }
-
 
 template <int H>
 __global__ void __launch_bounds__(kModeBlock *kMapGroups) k_contract(ContractArgs a)
@@ -113,6 +174,8 @@ __global__ void __launch_bounds__(kModeBlock *kMapGroups) k_contract(ContractArg
 #pragma unroll
     for (int li = 1; li < H; ++li) ju1 = max(ju1, jhi[li]);
 
+    chain_allow_next();
+    chain_wait();  // the samples and spectra come from the kernels before
     for (int c0 = P0; c0 < P1; c0 += a.pair_chunk) {
         const int c1 = min(P1, c0 + a.pair_chunk);
         // ---- generation: rho for pairs [c0, c1), this thread's mode, pairs split by group
@@ -209,6 +272,8 @@ __global__ void __launch_bounds__(kModes2 *kRings2, 2) k_contract_band(ContractA
     const int ju0 = kd.jlo[r0];
     const int nu = kd.jhi[r0 + nr - 1] - ju0 + 1;
 
+    chain_allow_next();
+    chain_wait();  // the samples and spectra come from the kernels before
     // ---- coefficient generation into this thread's shared column, then registers
     for (int s = 0; s < blen; ++s) {
         const int p = ps + s;
@@ -292,8 +357,7 @@ cudaError_t launch_contract_band(const ContractArgs &a, int nchunks, int max_uni
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.NH + kModes2 - 1) / kModes2, (a.nrep + kRings2 - 1) / kRings2, nchunks);
-    k_contract_band<<<grid, kModes2 * kRings2, smem, st>>>(a, max_union);
-    return cudaGetLastError();
+    return launch_chained(k_contract_band, grid, kModes2 * kRings2, smem, st, true, 1, a, max_union);
 }
 
 namespace {
@@ -356,6 +420,8 @@ struct PolarFft {
 __global__ void __launch_bounds__(1024) k_polar_rho_fft(ContractArgs a, const float2 *tw, int logN)
 {
     extern __shared__ float2 fbuf[];
+    chain_allow_next();
+    chain_wait();
     const int kid = blockIdx.y, p0 = 2 * blockIdx.x;
     if (p0 >= a.kd[kid].polar_pairs) return;
     switch (logN) {
@@ -370,6 +436,8 @@ __global__ void __launch_bounds__(1024) k_polar_rho_fft(ContractArgs a, const fl
 // The same coefficients one thread per (pair, mode), for kernel grids without the FFT form.
 __global__ void __launch_bounds__(256) k_polar_rho(ContractArgs a)
 {
+    chain_allow_next();
+    chain_wait();
     const int kid = blockIdx.z, p = blockIdx.y;
     const KernDev &kd = a.kd[kid];
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -380,41 +448,7 @@ __global__ void __launch_bounds__(256) k_polar_rho(ContractArgs a)
     const_cast<float *>(a.prho[kid])[(int64_t)p * a.NH + m] = gen_rho(tp4, S, f, m, a.N);
 }
 
-// csum[b][e] = sum_k w_k c[b K + k][e], e over the [R][NH] coefficients of a map; FP32 FMAs in
-// order of k (deterministic).
-struct SumWeights {
-    float w[kMaxKernelsPerLaunch];
-};
-
-__global__ void __launch_bounds__(256) k_weighted_sum(const float2 *__restrict__ c, float2 *__restrict__ csum,
-                                                      int K, SumWeights w, int64_t per_map, int64_t total)
-{
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = idx / per_map, e = idx - b * per_map;
-        float2 acc = make_float2(0.f, 0.f);
-        for (int k = 0; k < K; ++k) {
-            const float2 v = __ldg(&c[((int64_t)b * K + k) * per_map + e]);
-            acc.x = fmaf(w.w[k], v.x, acc.x);
-            acc.y = fmaf(w.w[k], v.y, acc.y);
-        }
-        csum[idx] = acc;
-    }
-}
-
 }  // namespace
-
-cudaError_t launch_weighted_sum(const float2 *c, float2 *csum, int64_t nmaps, int K, const double *w,
-                                int64_t per_map, cudaStream_t st)
-{
-    if (K < 1 || K > kMaxKernelsPerLaunch) return cudaErrorInvalidValue;
-    SumWeights sw;
-    for (int k = 0; k < kMaxKernelsPerLaunch; ++k) sw.w[k] = k < K ? (float)w[k] : 0.f;
-    const int64_t total = nmaps * per_map;
-    const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)device_sms() * 16);
-    k_weighted_sum<<<blocks, 256, 0, st>>>(c, csum, K, sw, per_map, total);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs, const float2 *tw, int twM,
                              cudaStream_t st)
@@ -428,25 +462,25 @@ cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         dim3 grid((max_polar_pairs + 1) / 2, nk);
-        k_polar_rho_fft<<<grid, a.N / 16, smem, st>>>(a, tw, logN);
-        return cudaGetLastError();
+        return launch_chained(k_polar_rho_fft, grid, a.N / 16, smem, st, true, 1, a, tw, logN);
     }
     dim3 grid((a.NH + 255) / 256, max_polar_pairs, nk);
-    k_polar_rho<<<grid, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_polar_rho, grid, 256, 0, st, true, 1, a);
 }
 
-cudaError_t launch_taps(const TapArgs &a, int npairs, cudaStream_t st)
+cudaError_t launch_taps(const TapArgs &a, int nk, int64_t maxtaps, cudaStream_t st, bool after_prev)
 {
-    if (npairs <= 0) return cudaSuccess;
-    const size_t smem = (size_t)a.kd.T * (sizeof(double) + 4 * sizeof(float));
+    if (maxtaps <= 0) return cudaSuccess;
+    int T = 0;
+    for (int k = 0; k < std::max(nk, a.ksum); ++k) T = std::max(T, a.kd[k].T);
+    const size_t smem = (size_t)T * (sizeof(double) + 4 * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute((const void *)k_taps,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int blocks = (npairs + 7) / 8;
-    if (blocks > device_sms() * 8) blocks = device_sms() * 8;
-    k_taps<<<blocks, 256, smem, st>>>(a);
-    return cudaGetLastError();
+    // a warp per 128-slot tile while that fills at most one CTA per SM
+    const int64_t want = (maxtaps + 128 * (kTapThreads / 32) - 1) / (128 * (kTapThreads / 32));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, (device_sms() + nk - 1) / nk));
+    return launch_chained(k_taps, dim3(blocks, nk), kTapThreads, smem, st, after_prev, 1, a);
 }
 
 cudaError_t launch_contract(const ContractArgs &a, int nchunks, size_t smem, cudaStream_t st)
@@ -455,8 +489,7 @@ cudaError_t launch_contract(const ContractArgs &a, int nchunks, size_t smem, cud
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.NH + kModeBlock - 1) / kModeBlock, (a.nrep + kRingBlock - 1) / kRingBlock, nchunks);
-    k_contract<kRingBlock><<<grid, kModeBlock * kMapGroups, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_contract<kRingBlock>, grid, kModeBlock * kMapGroups, smem, st, true, 1, a);
 }
 
 }  // namespace arkcos

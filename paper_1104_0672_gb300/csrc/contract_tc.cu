@@ -121,7 +121,10 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
         // frequency of every ring of the block (and of their mirrors) has nothing to compute
         int nmax = 0;
         for (int t = 0; t < nr; ++t) nmax = max(nmax, __ldg(&a.rd.n[r0 + t]));
-        if (m0 > nmax / 2) return;
+        if (m0 > nmax / 2) {
+            chain_wait();
+            return;
+        }
     }
     const int b0 = blockIdx.z * a.maps_per_chunk;
     const int b1 = min(a.B, b0 + a.maps_per_chunk);
@@ -191,6 +194,10 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                                  min(srows, jlast - j0 + 1), m0, a.R, a.NH);
     };
     const int joff = jg0 - ju0;  // the group's first row within the staged rows
+    // everything up to here is set up beside the end of the kernels before; the samples and the
+    // spectra come from them
+    chain_allow_next();
+    chain_wait();
     float4 acc[G];
 #pragma unroll
     for (int t = 0; t < G; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -765,9 +772,8 @@ cudaError_t launch_tc(const ContractArgs &a, int nchunks, const TcTables &tb, in
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.NH + kTcModes - 1) / kTcModes, (a.nrep + RB - 1) / RB, nchunks);
-    k_contract_tc<RB, G, WIDE><<<grid, TcShape<RB, G>::kThreads, smem, st>>>(a, tb.ctab, tb.cos2n, tb.nkc, srows, nbuf,
-                                                                             tc_rows0(RB, srows), (uint32_t)ctl);
-    return cudaGetLastError();
+    return launch_chained(k_contract_tc<RB, G, WIDE>, grid, TcShape<RB, G>::kThreads, smem, st, true, 1, a, tb.ctab,
+                          tb.cos2n, tb.nkc, srows, nbuf, tc_rows0(RB, srows), (uint32_t)ctl);
 }
 
 }  // namespace

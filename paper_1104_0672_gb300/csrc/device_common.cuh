@@ -123,6 +123,12 @@ __device__ __forceinline__ float gen_rho(const float4 *__restrict__ tp4, int S, 
     return acc;
 }
 
+// Programmatic dependent launch (launch_chained): allow the next kernel of the stream to begin
+// once every CTA of this one has come here; wait until the kernel before this one has completed
+// and its results can be read.  Both do nothing in a launch without the attribute.
+__device__ __forceinline__ void chain_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // 16-byte asynchronous global -> shared copy (zero-filled when bytes == 0).
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, int bytes)
 {

@@ -2,23 +2,29 @@
 // each) are recomputed by the true-profile direct sum s_p = sum_q w_q f(gamma_pq) r_q over
 // the input rings inside the support, and the adjoint adds the transposed sum.  FP64 squared
 // chords and profile values, FP64 accumulation, deterministic block reductions.
+#include <cooperative_groups.h>
+
 #include "device_common.cuh"
 
 namespace arkcos {
 
 namespace {
 
-// Squared chord between pixel p of ring i and pixel q of ring j (exact longitudes
-// pi (2p + hs) / n reduced as rationals before the FP64 sincospi).
-__device__ __forceinline__ double pixel_chord2(const RingDev &rd, int i, int p, int j, int q)
+// Half of the longitude difference (over pi) between pixel p of ring i and pixel q of ring j
+// (pixels at longitudes pi (2p + hs) / n).
+__device__ __forceinline__ double half_lon(const RingDev &rd, int i, int p, int j, int q)
 {
-    const int ni = rd.n[i], nj = rd.n[j];
-    const double y = (double)(2 * p + rd.hs[i]) / (2.0 * ni) - (double)(2 * q + rd.hs[j]) / (2.0 * nj);
-    double sy, cy;
-    sincospi(y, &sy, &cy);  // x/2 = pi y
-    const double ti = rd.theta[i], tj = rd.theta[j];
-    const double sd = sin(0.5 * (ti - tj)), ss = sin(0.5 * (ti + tj));
-    return 4.0 * (sd * sd * cy * cy + ss * ss * sy * sy);
+    return (double)(2 * p + rd.hs[i]) / (2.0 * rd.n[i]) - (double)(2 * q + rd.hs[j]) / (2.0 * rd.n[j]);
+}
+
+// Squared chord between a pixel of the pole ring and one of the jj-th ring from that pole:
+// u = 4 (B cos^2(x/2) + A sin^2(x/2)) = 4 (B + (A - B) sin^2(x/2)), A - B = sin(theta_i)
+// sin(theta_j) >= 0, with the band table's A = sin^2 and B = sin^2 of the half sum and difference
+// of the colatitudes (the mirror pairs of the south pole share them).
+__device__ __forceinline__ double pole_chord2(const KernDev &kd, int jj, double y)
+{
+    const double s = sinpi(y), B = kd.B[jj];
+    return 4.0 * fma(kd.A[jj] - B, s * s, B);
 }
 
 __device__ double block_sum(double v, double *red)
@@ -34,42 +40,59 @@ __device__ double block_sum(double v, double *red)
     return s;
 }
 
-// Direct sum of kernel kd at pixel p of pole ring i over input map mp (this thread's share).
-__device__ double pole_sum(const PoleArgs &a, const KernDev &kd, const float *mp, int i, int p, int e)
+// Direct sum of kernel kd at pixel p of the pole ring over input map mp (this thread's share: the
+// CTAs of the cluster take the pixels of the band's rings, one run of the map, in turn).
+__device__ double pole_sum(const PoleArgs &a, const KernDev &kd, const float *mp, int p, int e, int rank, int ranks)
 {
-    const int jl = kd.jlo[0], jh = kd.jhi[0];
+    const int jh = kd.jhi[0], ja = e == 0 ? 0 : a.R - 1 - jh, jz = e == 0 ? jh : a.R - 1;
+    const int i = e == 0 ? 0 : a.R - 1;
+    const int64_t q0 = a.rd.poff[ja], q1 = a.rd.poff[jz] + a.rd.n[jz];
     double acc = 0.0;
-    for (int jj = jl; jj <= jh; ++jj) {
-        const int j = e == 0 ? jj : a.R - 1 - jj;
-        const int nj = a.rd.n[j];
-        const double wj = (double)a.rd.w[j];
-        for (int q = threadIdx.x; q < nj; q += blockDim.x) {
-            const double u = pixel_chord2(a.rd, i, p, j, q);
-            if (u <= kd.umax)
-                acc += wj * profile_eval(u, kd.ut, kd.knots, kd.T, kd.gscale) *
-                       (double)__ldg(&mp[a.rd.poff[j] + q]);
+    for (int64_t q = q0 + rank * blockDim.x + threadIdx.x; q < q1; q += ranks * blockDim.x) {
+        int j = ja, hi = jz;  // the pixel's ring
+        while (j < hi) {
+            const int mid = (j + hi + 1) >> 1;
+            if (__ldg(&a.rd.poff[mid]) <= q) j = mid;
+            else hi = mid - 1;
         }
+        const double u = pole_chord2(kd, e == 0 ? j : a.R - 1 - j, half_lon(a.rd, i, p, j, (int)(q - a.rd.poff[j])));
+        if (u <= kd.umax)
+            acc += (double)a.rd.w[j] * profile_eval(u, kd.ut, kd.knots, kd.T, kd.gscale) * (double)__ldg(&mp[q]);
     }
     return acc;
 }
 
-// grid: (pixel p of the pole ring, pole e in {0: ring 0, 1: ring R-1}, map b)
-__global__ void __launch_bounds__(256) k_pole_fwd(PoleArgs a)
+// One cluster per (pixel p of the pole ring, pole e in {0: ring 0, 1: ring R-1}, map b), its CTAs'
+// sums added in order.  It reads only the input maps and the inverse transforms leave these
+// rings alone, so it runs beside their end.  FP64 arithmetic (two FMAs per SM and clock) bounds
+// it: the chord from the band table and one sine per pixel, spread over more SMs, 14 us for one
+// nside-2048 map with a 15' support and 21 us at a degree, launch included, against 60 and 224 us
+// with three sines per pixel and a CTA per output pixel going ring by ring.
+__global__ void __launch_bounds__(256) k_pole_fwd(const __grid_constant__ PoleArgs a)
 {
-    __shared__ double red[8];
-    const int p = blockIdx.x, e = blockIdx.y, b = blockIdx.z;
-    const int i = e == 0 ? 0 : a.R - 1;
-    if (p >= a.rd.n[i]) return;
+    namespace cg = cooperative_groups;
+    __shared__ double red[8], part;
+    auto cluster = cg::this_cluster();
+    const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int p = blockIdx.x / ranks, e = blockIdx.y, b = blockIdx.z;
     const int src = a.vdiv > 1 ? (a.vbase + b) / a.vdiv : b;
     const float *mp = a.map + (int64_t)src * a.npix;
     double acc = 0.0;
     if (a.nsum > 0) {
         // the weighted sum over several kernels of one input map, in kernel order
-        for (int k = 0; k < a.nsum; ++k) acc += a.wsum[k] * block_sum(pole_sum(a, a.kd[k], mp, i, p, e), red);
+        for (int k = 0; k < a.nsum; ++k) acc += a.wsum[k] * pole_sum(a, a.kd[k], mp, p, e, rank, ranks);
     } else {
-        acc = block_sum(pole_sum(a, a.kd[a.per_map ? b - a.map_base : 0], mp, i, p, e), red);
+        acc = pole_sum(a, a.kd[a.per_map ? b - a.map_base : 0], mp, p, e, rank, ranks);
     }
-    if (threadIdx.x == 0) a.out[(int64_t)b * a.npix + a.rd.poff[i] + p] = (float)acc;
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) part = acc;
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        for (int r = 1; r < ranks; ++r) acc += *cluster.map_shared_rank(&part, r);
+        a.out[(int64_t)b * a.npix + a.rd.poff[e == 0 ? 0 : a.R - 1] + p] = (float)acc;
+    }
+    cluster.sync();
+    chain_wait();
 }
 
 // grid: (ring index within the pole band, side e, map b); adds the transposed direct sum of
@@ -94,7 +117,7 @@ __global__ void __launch_bounds__(256) k_pole_adj(PoleArgs a)
             const int jn = side == 0 ? j : a.R - 1 - j;  // distance in rings from that pole
             if (jn < jl || jn > jh) continue;
             for (int p = 0; p < a.rd.n[i]; ++p) {
-                const double u = pixel_chord2(a.rd, i, p, j, q);
+                const double u = pole_chord2(kd, jn, half_lon(a.rd, i, p, j, q));
                 if (u <= kd.umax)
                     acc += wj * profile_eval(u, kd.ut, kd.knots, kd.T, kd.gscale) *
                            (double)__ldg(&g[a.rd.poff[i] + p]);
@@ -106,11 +129,12 @@ __global__ void __launch_bounds__(256) k_pole_adj(PoleArgs a)
 
 }  // namespace
 
-cudaError_t launch_pole_fwd(const PoleArgs &a, cudaStream_t st)
+cudaError_t launch_pole_fwd(const PoleArgs &a, int64_t band_pixels, cudaStream_t st, bool after_prev)
 {
-    dim3 grid(4, 2, a.B);
-    k_pole_fwd<<<grid, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    // CTAs per cluster: about one pixel per thread, while the launch is not already some CTAs per SM
+    int c = 1;
+    while (c < 8 && 256 * (int64_t)c < band_pixels && 16 * (int64_t)c * a.B <= 4 * device_sms()) c *= 2;
+    return launch_chained(k_pole_fwd, dim3(4 * c, 2, a.B), 256, 0, st, after_prev, c, a);
 }
 
 cudaError_t launch_pole_adj(const PoleArgs &a, int max_band_rings, cudaStream_t st)

@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(512) k_fft_fwd_split(FftFwdArgs a)
 {
     // [buffer_words(a.M)] quarter-transform buffer | [n] spectrum | chirp of the quarter
     extern __shared__ float2 sbuf[];
-    ring::stage_allow_next();
+    chain_allow_next();
     const int j = a.reps[blockIdx.x];
     const int n = a.rd.n[j], q = n / 4;
     float2 *X = sbuf + fft::buffer_words(a.M);
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(512) k_fft_fwd_split(FftFwdArgs a)
     FwdSplitCta c{a, sbuf, X, chirp, a.rd.fb + a.rd.fboff[j], j, j2, n, a.rd.hs[j], j2 != j,
                   a.zero_poles && j == 0, a.weight ? a.rd.w[j] : 1.0f};
     c.run<13>();  // split rings have 2048 < q < 4096: quarter buffer 8192 (kMaxSplitM)
-    ring::stage_wait_prev();
+    chain_wait();
 }
 
 template <int LMAX>
@@ -329,7 +329,7 @@ k_fft_fwd(FftFwdArgs a)
     // [buffer_words(a.M)] pair buffer, then the chirp and phase tables of Bluestein rings
     extern __shared__ float4 smem4[];
     __shared__ cpair xh;
-    ring::stage_allow_next();
+    chain_allow_next();
     const int j = a.reps[blockIdx.x];
     const int n = a.rd.n[j], h = n / 2;
     const bool blu = ring::bluestein(h);
@@ -343,7 +343,7 @@ k_fft_fwd(FftFwdArgs a)
     FwdCta c{a, buf, &xh, chirp, phase, blu ? a.rd.fb + a.rd.fboff[j] : nullptr, j, j2, n, h, hs,
              j2 != j, blu, a.zero_poles && j == 0, a.weight ? a.rd.w[j] : 1.0f};
     ring::dispatch_upto<LMAX>(logM, c);
-    ring::stage_wait_prev();
+    chain_wait();
 }
 
 cudaError_t set_smem(const void *fn, size_t bytes)
@@ -378,8 +378,8 @@ cudaError_t launch_fft_fwd_split(const FftFwdArgs &a, int count, int threads, cu
     const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, threads, true);
     cudaError_t e = set_smem((const void *)k_fft_fwd_split, smem);
     if (e != cudaSuccess) return e;
-    return launch_class_kernel(k_fft_fwd_split, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), threads, smem, st,
-                               after_prev, a);
+    return launch_chained(k_fft_fwd_split, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), threads, smem, st,
+                          after_prev, 1, a);
 }
 
 template <int LMAX>
@@ -389,8 +389,8 @@ cudaError_t launch_fwd_class(const FftFwdArgs &a, int count, cudaStream_t st, bo
     const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, T, false);
     cudaError_t e = set_smem((const void *)k_fft_fwd<LMAX>, smem);
     if (e != cudaSuccess) return e;
-    return launch_class_kernel(k_fft_fwd<LMAX>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), T, smem, st,
-                               after_prev, a);
+    return launch_chained(k_fft_fwd<LMAX>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), T, smem, st,
+                          after_prev, 1, a);
 }
 
 cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev)

@@ -361,18 +361,25 @@ __global__ void __launch_bounds__(512) k_fft_inv_split(FftInvArgs a)
 {
     // [buffer_words(a.M)] quarter-transform buffer | [n] coefficients | chirp of the quarter
     extern __shared__ float2 sbuf[];
-    ring::stage_allow_next();
+    if (!a.first) chain_allow_next();
     const int i = a.reps[blockIdx.x];
-    if (a.skip_poles && i == 0) return;
+    if (a.skip_poles && i == 0) {
+        chain_wait();
+        return;
+    }
     const int n = a.rd.n[i], q = n / 4;
     float2 *X = sbuf + fft::buffer_words(a.M);
     float2 *chirp = X + n;
     ring::chirp_table(chirp, q, +1);
+    if (a.first) {
+        chain_wait();
+        chain_allow_next();
+    }
     const int i2 = a.R - 1 - i;
     InvSplitCta c{a, sbuf, X, chirp, a.rd.fb + a.rd.fboff[i], i, i2, n, a.rd.hs[i], i2 != i,
                   a.weight ? a.rd.w[i] : 1.0f};
     c.run<13>();  // split rings have 2048 < q < 4096: quarter buffer 8192 (kMaxSplitM)
-    ring::stage_wait_prev();
+    chain_wait();
 }
 
 template <int LMAX>
@@ -382,9 +389,12 @@ k_fft_inv(FftInvArgs a)
     // [buffer_words(a.M)] pair buffer | short-ring fold: [2 (N/8 + 1)] folded coefficients,
     // [2 blockDim] float4 partial sums | chirp and phase tables
     extern __shared__ float4 smem4[];
-    ring::stage_allow_next();
+    if (!a.first) chain_allow_next();
     const int i = a.reps[blockIdx.x];
-    if (a.skip_poles && i == 0) return;  // rings 0 and R-1 come from the pole kernel
+    if (a.skip_poles && i == 0) {  // rings 0 and R-1 come from the pole kernel
+        chain_wait();
+        return;
+    }
     const int n = a.rd.n[i], h = n / 2;
     const bool blu = ring::bluestein(h);
     const int logM = ring::log2_buffer(h);
@@ -396,11 +406,17 @@ k_fft_inv(FftInvArgs a)
     float2 *chirp = a.stage_c ? reinterpret_cast<float2 *>(part + 2 * blockDim.x) : D1;  // exp(+i pi k^2 / h)
     float2 *phase = chirp + (blu ? h / 2 + 1 : 0);                                    // exp(+i pi m / n)
     ring::tables(chirp, phase, n, h, +1, blu, a.tw);
+    if (a.first) {
+        // the first class of the stage starts beside the end of the contraction: its tables are
+        // ready when the coefficients are; the next class may only follow them
+        chain_wait();
+        chain_allow_next();
+    }
     const int i2 = a.R - 1 - i;
     InvCta c{a, buf, D1, D2, part, chirp, phase, blu ? a.rd.fb + a.rd.fboff[i] : nullptr,
              i, i2, n, h, hs, i2 != i, blu, stage, a.weight ? a.rd.w[i] : 1.0f};
     ring::dispatch_upto<LMAX>(logM, c);
-    ring::stage_wait_prev();
+    chain_wait();
 }
 
 }  // namespace
@@ -423,8 +439,8 @@ cudaError_t launch_fft_inv_split(const FftInvArgs &a, int count, int threads, cu
     cudaError_t e = cudaFuncSetAttribute((const void *)k_fft_inv_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_class_kernel(k_fft_inv_split, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), threads, smem, st,
-                               after_prev, a);
+    return launch_chained(k_fft_inv_split, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), threads, smem, st,
+                          after_prev, 1, a);
 }
 
 template <int LMAX>
@@ -435,8 +451,8 @@ cudaError_t launch_inv_class(const FftInvArgs &a, int count, cudaStream_t st, bo
     cudaError_t e = cudaFuncSetAttribute((const void *)k_fft_inv<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_class_kernel(k_fft_inv<LMAX>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), T, smem, st,
-                               after_prev, a);
+    return launch_chained(k_fft_inv<LMAX>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), T, smem, st,
+                          after_prev, 1, a);
 }
 
 cudaError_t launch_fft_inv(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev)
