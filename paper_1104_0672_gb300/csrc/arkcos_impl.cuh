@@ -13,7 +13,7 @@ namespace arkcos {
 
 constexpr int kMaxKernelsPerLaunch = 32;  // per-map beams handled per contraction launch
 constexpr int kMaxPolarPairs = 16384;      // most pairs whose coefficients are tabulated per call
-constexpr int kModeBlock = 128;           // modes per contraction CTA (one per thread)
+constexpr int kModeBlock = 128;           // modes per CTA of the generic knot-gradient kernel
 constexpr int kMaxFftM = 8192;            // largest in-shared-memory ring FFT buffer (complex pairs)
 constexpr int kMaxSplitM = 8192;          // buffer of the quarter transforms of split rings
 constexpr int kSplitClass = 15;           // FFT class index of the split rings
@@ -191,7 +191,6 @@ struct ContractArgs {
     int per_map;        // 1: map b uses kd[b - map_base]
     int map_base;
     int basic, shift_fix;
-    int pair_chunk;     // pairs whose coefficients fit in shared memory at once
     int withhold_mma;   // test knob: issue no tensor-core MMA, so the completion waits expire
     int vbase, vdiv;    // vdiv > 1 (several kernels on one input): map b of the launch reads the
                         // spectra of input (vbase + b) / vdiv of spec4; else those of map b
@@ -289,7 +288,6 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t 
     cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
-cudaError_t launch_contract(const ContractArgs &a, int nchunks, size_t smem, cudaStream_t st);
 // band_pixels: pixels of the rings inside the support of a pole
 cudaError_t launch_pole_fwd(const PoleArgs &a, int64_t band_pixels, cudaStream_t st, bool after_prev);
 cudaError_t launch_pole_adj(const PoleArgs &a, int max_band_rings, cudaStream_t st);
@@ -306,11 +304,8 @@ int knot_proj_blocks();
 int knot_proj_taps();
 cudaError_t launch_knot_reduce(const double *partial, int nrows, int T, double *out,
                                cudaStream_t st);
-int contract_ring_block();
 void set_last_error(const char *msg);  // sets the message arkcos_last_error() returns
 int contract_band_limit();
-int contract_band_rings();
-cudaError_t launch_contract_band(const ContractArgs &a, int nchunks, int max_union, cudaStream_t st);
 // tensor-core contraction over blocks of rb (8 or 16) representative rings, a thread taking
 // a group of gs (2 or 4) rings; the wide form takes bands of any width
 struct TcTables {
@@ -318,10 +313,10 @@ struct TcTables {
     const float2 *cos2n;  // cos(pi t / N), t < 2N (hi, lo)
     int nkc;
 };
-cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, int nchunks, const TcTables &tb, int srows,
-                               int want_nbuf, cudaStream_t st);
-cudaError_t launch_contract_tc_wide(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, cudaStream_t st);
-bool contract_tc_wide_fits(int srows);
+cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int nchunks, const TcTables &tb,
+                               int srows, int want_nbuf, cudaStream_t st);
+cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks, const TcTables &tb, int srows,
+                                    cudaStream_t st);
 int contract_tc_nbuf(int rb, int gs, int srows, int want_nbuf);
 size_t contract_tc_smem(int rb, int gs, int srows, int want_nbuf);
 int contract_tc_modes();

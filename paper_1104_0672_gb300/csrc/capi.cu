@@ -662,14 +662,11 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
                            bool basic, bool shift_fix, bool tf32, cudaStream_t st, const Shape &sh = Shape{},
                            bool polar_table = true, int64_t kdiv = 0)
 {
-    const int H = contract_ring_block();
-    int maxband = 0, maxunion = 0, maxunion2 = 0, maxunion4 = 0;
+    int maxunion2 = 0, maxunion4 = 0;
     int srows[2][2] = {{0, 0}, {0, 0}}, wrows = 0;  // [16-ring blocks][groups of four]; wide form
     int maxfree = 0;  // most samples of a pair without tabulated coefficients
     for (int64_t k = 0; k < nk; ++k) {
         const Kernel &K = ks[k]->k;
-        maxband = std::max(maxband, K.maxband);
-        maxunion = std::max(maxunion, K.max_union8);
         maxunion2 = std::max(maxunion2, K.max_union2);
         maxunion4 = std::max(maxunion4, K.max_union4);
         srows[0][0] = std::max(srows[0][0], K.max_stage_rows);
@@ -679,25 +676,30 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
         wrows = std::max(wrows, K.max_win_rows);
         maxfree = std::max(maxfree, K.max_free_taps);
     }
-    // the register-resident fast path covers bands of up to contract_band_limit() rings
-    const bool fast = maxband <= contract_band_limit() && 2 * maxunion * 64 * 16 <= 200 * 1024;
-    const bool tc = tf32 && maxunion2 <= contract_band_limit() && maxfree <= 32 * g.nkc_tab &&
-                    contract_tc_smem(8, 2, srows[0][0], 0) <= 200 * 1024;
-    // bands whose ring groups see more than 32 input rings, or pairs with more samples than one
-    // run of the kernel and no tabulated coefficients: the tensor-core form with the 32
-    // slots moving along the band (contraction of 77.1 -> 4.5 ms for one nside-2048 map at a degree of support
-    // against k_contract<8>, which remains for the plain FP32 form)
-    const bool tc_wide = tf32 && !tc && contract_tc_wide_fits(wrows);
-    const TcTables tb{g.d_ctab, g.d_cos2n, g.nkc_tab};
-    // tensor-core form: groups of four rings when their union bands fit the 32 slots, blocks of
-    // 16 rings when two staging buffers fit beside one CTA per SM; the autotuner's choice, else
-    // the default: for a shared beam groups of four in blocks of 16 where they fit; for per-map
-    // beams (every CTA generates its own coefficients for one map) blocks of 8, two CTAs per SM,
-    // so that one CTA's generation overlaps the other's contraction
+    const bool per_map = nk > 1 || kdiv > 0;
+    // One window of 32 input rings per ring group where the groups' union bands fit it and no pair
+    // without tabulated coefficients has more samples than a run; else the form whose window moves
+    // along the band (one nside-2048 map at a degree of support: 4.5 ms 3xTF32, 18.5 ms plain FP32;
+    // 77 ms when a thread generated each coefficient by its own recurrence).  Ring spacings differ by at most a
+    // third, so its staged rows always fit.
     const bool g4_ok = maxunion4 <= contract_band_limit();
+    const bool run_ok = maxfree <= 32 * g.nkc_tab;
+    const bool narrow = run_ok && (tf32 ? maxunion2 <= contract_band_limit() : g4_ok);
+    const TcTables tb{g.d_ctab, g.d_cos2n, g.nkc_tab};
+    // narrow form: groups of four rings when their union bands fit the 32 slots, blocks of 16 rings
+    // when two staging buffers fit beside one CTA per SM; the autotuner's choice, else the
+    // default: for a shared beam groups of four in blocks of 16 where they fit; for per-map beams
+    // (every CTA generates its own coefficients for one map) blocks of 8, two CTAs per SM, so that
+    // one CTA's generation overlaps the other's contraction, for the plain FP32 form (generation on
+    // the CUDA cores: one nside-2048 map 0.98 against 1.11 ms with blocks of 16, four maps 1.56
+    // against 1.70 ms) and for calls of less than two waves of blocks of 16 (one nside-256 map 27
+    // against 29 us; from there on 16 is as fast for one map and faster for several, four
+    // nside-2048 maps 1.00 against 1.11 ms)
     const bool b16_ok[2] = {contract_tc_nbuf(16, 2, srows[1][0], 0) == 2, contract_tc_nbuf(16, 4, srows[1][1], 0) == 2};
     int tc_rb = 8, tc_gs = g4_ok ? 4 : 2, tc_want = 0;
-    const int form = sh.tc_form != 0 ? sh.tc_form : (nk > 1 ? 4 : 5);
+    const int64_t ctas16 = (int64_t)((g.N / 2 + contract_tc_modes()) / contract_tc_modes()) * ((g.nrep + 15) / 16) *
+                           (per_map ? nmaps : 1);
+    const int form = !tf32 ? 4 : sh.tc_form != 0 ? sh.tc_form : (nk > 1 || ctas16 < 2 * device_sms() ? 4 : 5);
     switch (form) {
     case 1: case 2: tc_gs = 2; tc_want = form; break;
     case 3: if (b16_ok[0]) { tc_rb = 16; tc_gs = 2; } break;
@@ -705,14 +707,10 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
     default: if (g4_ok && b16_ok[1]) tc_rb = 16; break;
     }
     const int tc_srows = srows[tc_rb == 16][tc_gs == 4];
-    int pair_chunk = std::min(H * maxband, 192);
-    pair_chunk = std::max(pair_chunk, 1);
-    const size_t smem = (size_t)pair_chunk * kModeBlock * sizeof(float);
-    const bool per_map = nk > 1 || kdiv > 0;
     auto kof = [&](int64_t v) { return kdiv > 0 ? v % kdiv : v; };  // kernel of map v
     const int64_t groups = per_map ? (nmaps + kMaxKernelsPerLaunch - 1) / kMaxKernelsPerLaunch : 1;
     StageScope sc(ST_CONTRACT, (int)groups, st);
-    if (kdiv > 0 && polar_table && (tc || tc_wide || fast)) {
+    if (kdiv > 0 && polar_table) {
         // several maps share each kernel: its polar coefficient table is computed once
         for (int64_t k0 = 0; k0 < kdiv; k0 += kMaxKernelsPerLaunch) {
             ContractArgs a;
@@ -765,7 +763,6 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
         a.map_base = (int)base;
         a.basic = basic;
         a.shift_fix = shift_fix;
-        a.pair_chunk = pair_chunk;
         a.withhold_mma = test_withhold_mma();
         // chunks cover maps [base, base + cnt) for per-map kernels, all maps otherwise
         const int nchunks = per_map ? (int)cnt : (int)((nmaps + chunk - 1) / chunk);
@@ -781,14 +778,12 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
             a.B = (int)cnt;
             a.map_base = 0;
         }
-        if ((tc || tc_wide || fast) && polar_table && kdiv == 0 && maxpolar > 0) {
+        if (polar_table && kdiv == 0 && maxpolar > 0) {
             CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, st));
             ++sc.launches;
         }
-        if (tc) CK(launch_contract_tc(a, tc_rb, tc_gs, nchunks, tb, tc_srows, tc_want, st));
-        else if (tc_wide) CK(launch_contract_tc_wide(a, nchunks, tb, wrows, st));
-        else if (fast) CK(launch_contract_band(a, nchunks, maxunion, st));
-        else CK(launch_contract(a, nchunks, smem, st));
+        if (narrow) CK(launch_contract_tc(a, tc_rb, tc_gs, !tf32, nchunks, tb, tc_srows, tc_want, st));
+        else CK(launch_contract_tc_wide(a, !tf32, nchunks, tb, wrows, st));
     }
     return ARKCOS_OK;
 }

@@ -1,6 +1,6 @@
-// Kernel sampling and the ring-band contraction (Sec. 4.1: kernel grid centred on each output
-// ring, its ring FFT, product with the map coefficients and the sum over the n_support rings
-// in theta; Sec. 4.3: super-Nyquist periodic extension and the equatorial shift fix).
+// Kernel sampling (Sec. 4.1: kernel grid centred on each output ring) and the tabulated Fourier
+// coefficients of the ring pairs next to the poles; the other pairs' coefficients are generated
+// inside the contraction (contract_tc.cu).
 //
 // The kernel grid of ring pair (i, j) is sampled at longitudes x_k = pi (2k + f) / N with
 // f = 1 when the shift fix applies to a pair of equal-length rings with different offsets
@@ -11,10 +11,6 @@
 //
 // k_taps evaluates c_k K(u) per pair in FP64 (u is the squared chord of Eq. kernel_angle
 // in the cancellation-free form 4[B cos^2(x/2) + A sin^2(x/2)]), storing FP32 values.
-// k_contract generates rho for a block of output rings x 128 modes into shared memory (one
-// thread per mode, cosines by Reinsch's modified recurrence, restarted from exact values
-// every 64 taps) and then contracts it with the map spectra of every map of the batch.
-// N-S mirror pairs share rho, so each CTA serves ring i and ring R-1-i.
 #include <algorithm>
 
 #include "fft_engine.cuh"
@@ -22,10 +18,6 @@
 namespace arkcos {
 
 namespace {
-
-constexpr int kRingBlock = 8;   // representative output rings per CTA
-constexpr int kMapGroups = 4;   // warp groups per CTA: they split the coefficient generation
-                                // by pairs and the contraction by maps
 
 // Kernel samples K(u(x_k)) c_k / N.  u = 4 (B cos^2(x/2) + A sin^2(x/2)) is the haversine form
 // of the squared chord, so the FP64 work per sample is the offset from the knot below it,
@@ -138,229 +130,6 @@ __global__ void __launch_bounds__(kTapThreads) k_taps(const __grid_constant__ Ta
     }
     chain_wait();
 }
-
-template <int H>
-__global__ void __launch_bounds__(kModeBlock *kMapGroups) k_contract(ContractArgs a)
-{
-    extern __shared__ float rho[];  // [pair_chunk][kModeBlock]
-    const int tid = threadIdx.x & (kModeBlock - 1);
-    const int grp = threadIdx.x / kModeBlock;
-    const int m = blockIdx.x * kModeBlock + tid;
-    const bool mv = m < a.NH;
-    const int r0 = blockIdx.y * H;
-    const int nr = min(H, a.nrep - r0);
-    const int b0 = blockIdx.z * a.maps_per_chunk;
-    const int b1 = min(a.B, b0 + a.maps_per_chunk);
-    const int kid = a.per_map ? (b0 - a.map_base) : 0;
-    const KernDev &kd = a.kd[kid];
-    const float *taps = a.taps[kid];
-
-    int jlo[H], jhi[H], ps[H];
-#pragma unroll
-    for (int li = 0; li < H; ++li) {
-        if (li < nr) {
-            jlo[li] = kd.jlo[r0 + li];
-            jhi[li] = kd.jhi[r0 + li];
-            ps[li] = kd.pstart[r0 + li];
-        } else {
-            jlo[li] = 1;
-            jhi[li] = 0;
-            ps[li] = 0;
-        }
-    }
-    const int P0 = kd.pstart[r0], P1 = kd.pstart[r0 + nr];
-    const int ju0 = jlo[0];
-    int ju1 = jhi[0];
-#pragma unroll
-    for (int li = 1; li < H; ++li) ju1 = max(ju1, jhi[li]);
-
-    chain_allow_next();
-    chain_wait();  // the samples and spectra come from the kernels before
-    for (int c0 = P0; c0 < P1; c0 += a.pair_chunk) {
-        const int c1 = min(P1, c0 + a.pair_chunk);
-        // ---- generation: rho for pairs [c0, c1), this thread's mode, pairs split by group
-        for (int p = c0 + grp; p < c1; p += kMapGroups) {
-            const int f = a.shift_fix ? kd.fl[p] : 0;
-            const int S = f ? kd.S1[p] : kd.S0[p];
-            const float4 *tp4 = reinterpret_cast<const float4 *>(taps + kd.toff[p]);
-            rho[(p - c0) * kModeBlock + tid] = mv ? gen_rho(tp4, S, f, m, a.N) : 0.f;
-        }
-        __syncthreads();
-        // ---- contraction over the input rings of the band, maps split by group
-        if (mv) {
-            for (int b = b0 + grp; b < b1; b += kMapGroups) {
-                const float4 *sp4b = map_spec4(a, b);
-                float2 acc[H], acc2[H];
-#pragma unroll
-                for (int li = 0; li < H; ++li) {
-                    if (c0 == P0 || li >= nr) {
-                        acc[li] = make_float2(0.f, 0.f);
-                        acc2[li] = make_float2(0.f, 0.f);
-                    } else {
-                        const int i = r0 + li;
-                        acc[li] = a.c[((int64_t)b * a.R + i) * a.NH + m];
-                        acc2[li] = a.c[((int64_t)b * a.R + (a.R - 1 - i)) * a.NH + m];
-                    }
-                }
-                for (int j = ju0; j <= ju1; ++j) {
-                    // skip rings no pair of this chunk uses
-                    bool used = false;
-#pragma unroll
-                    for (int li = 0; li < H; ++li) {
-                        const int p = ps[li] + j - jlo[li];
-                        used |= (j >= jlo[li] && j <= jhi[li] && p >= c0 && p < c1);
-                    }
-                    if (!used) continue;
-                    const float4 v = paired_coeff(sp4b, j, a.R, a.NH, m);
-                    const float2 aj = make_float2(v.x, v.y), ajm = make_float2(v.z, v.w);
-#pragma unroll
-                    for (int li = 0; li < H; ++li) {
-                        const int p = ps[li] + j - jlo[li];
-                        if (j >= jlo[li] && j <= jhi[li] && p >= c0 && p < c1) {
-                            const float r = rho[(p - c0) * kModeBlock + tid];
-                            acc[li].x = fmaf(r, aj.x, acc[li].x);
-                            acc[li].y = fmaf(r, aj.y, acc[li].y);
-                            acc2[li].x = fmaf(r, ajm.x, acc2[li].x);
-                            acc2[li].y = fmaf(r, ajm.y, acc2[li].y);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int li = 0; li < H; ++li) {
-                    if (li < nr) {
-                        const int i = r0 + li, im = a.R - 1 - i;
-                        a.c[((int64_t)b * a.R + i) * a.NH + m] = acc[li];
-                        if (im != i) a.c[((int64_t)b * a.R + im) * a.NH + m] = acc2[li];
-                    }
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// Fast path of the contraction for bands of at most kBand2 input rings per output ring.
-// Thread = (mode m, representative output ring r0 + li); its kBand2 ring-pair coefficients
-// live in registers (generated through a per-thread shared-memory column).  For every map
-// the CTA stages the extended spectra a_m(j) and a_m(R-1-j) of the union band as float4 in
-// shared memory (one coalesced pass), then each thread sums its band with one 16-byte
-// shared load and four FMAs per ring pair, predicate-free in the common case.
-constexpr int kBand2 = 32;    // ring pairs per output ring held in registers
-constexpr int kModes2 = 64;   // modes per CTA
-constexpr int kRings2 = 8;    // representative output rings per CTA
-
-
-__global__ void __launch_bounds__(kModes2 *kRings2, 2) k_contract_band(ContractArgs a, int max_union)
-{
-    extern __shared__ float4 sh4[];  // staging [max_union][kModes2] (aliased by the rho columns)
-    float *rho_col = reinterpret_cast<float *>(sh4);
-    const int tm = threadIdx.x & (kModes2 - 1);
-    const int li = threadIdx.x / kModes2;
-    const int m = blockIdx.x * kModes2 + tm;
-    const bool mv = m < a.NH;
-    const int r0 = blockIdx.y * kRings2;
-    const int nr = min(kRings2, a.nrep - r0);
-    const bool lv = li < nr;
-    const int b0 = blockIdx.z * a.maps_per_chunk;
-    const int b1 = min(a.B, b0 + a.maps_per_chunk);
-    const int kid = a.per_map ? (b0 - a.map_base) : 0;
-    const KernDev &kd = a.kd[kid];
-    const float *taps = a.taps[kid];
-    const int i = r0 + (lv ? li : 0);
-    const int jl = kd.jlo[i], ps = kd.pstart[i];
-    const int blen = lv ? kd.jhi[i] - jl + 1 : 0;
-    const int ju0 = kd.jlo[r0];
-    const int nu = kd.jhi[r0 + nr - 1] - ju0 + 1;
-
-    chain_allow_next();
-    chain_wait();  // the samples and spectra come from the kernels before
-    // ---- coefficient generation into this thread's shared column, then registers
-    for (int s = 0; s < blen; ++s) {
-        const int p = ps + s;
-        const int f = a.shift_fix ? kd.fl[p] : 0;
-        const int S = f ? kd.S1[p] : kd.S0[p];
-        const float4 *tp4 = reinterpret_cast<const float4 *>(taps + kd.toff[p]);
-        float r = 0.f;
-        if (mv) r = p < kd.polar_pairs ? __ldg(&a.prho[kid][(int64_t)p * a.NH + m]) : gen_rho(tp4, S, f, m, a.N);
-        rho_col[s * blockDim.x + threadIdx.x] = r;
-    }
-    float rho[kBand2];
-#pragma unroll
-    for (int s = 0; s < kBand2; ++s) rho[s] = s < blen ? rho_col[s * blockDim.x + threadIdx.x] : 0.f;
-    const int joff = jl - ju0;  // this ring's first input ring within the union band
-    __syncthreads();
-
-    // rows of southern rings hold (a(R-1-j), a(j)); only ring blocks whose union band crosses
-    // the middle ring see them, so the swap is a block-uniform branch
-    const int mid = (a.R - 1) / 2;
-    const bool crosses = ju0 + nu - 1 > mid;
-    const int sstar = mid - jl + 1;  // first slot of this ring's band that is a southern ring
-    const size_t bufsz = (size_t)nu * kModes2;
-    const int m0 = blockIdx.x * kModes2;
-    if (b0 < b1) stage_band_async(sh4, map_spec4(a, b0), ju0, nu, m0, kModes2, a.R, a.NH);
-    for (int b = b0; b < b1; ++b) {
-        const int cur = (b - b0) & 1;
-        if (b + 1 < b1)
-            stage_band_async(sh4 + (cur ^ 1) * bufsz, map_spec4(a, b + 1), ju0, nu, m0,
-                             kModes2, a.R, a.NH);
-        else
-            cp_async_commit();
-        cp_async_wait1();
-        __syncthreads();
-        if (lv && mv) {
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 *col = sh4 + cur * bufsz + joff * kModes2 + tm;
-            if (!crosses) {
-#pragma unroll
-                for (int s = 0; s < kBand2; ++s) {
-                    if (s < blen) {
-                        const float4 v = col[s * kModes2];
-                        acc.x = fmaf(rho[s], v.x, acc.x);
-                        acc.y = fmaf(rho[s], v.y, acc.y);
-                        acc.z = fmaf(rho[s], v.z, acc.z);
-                        acc.w = fmaf(rho[s], v.w, acc.w);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int s = 0; s < kBand2; ++s) {
-                    if (s < blen) {
-                        float4 v = col[s * kModes2];
-                        if (s >= sstar) v = make_float4(v.z, v.w, v.x, v.y);
-                        acc.x = fmaf(rho[s], v.x, acc.x);
-                        acc.y = fmaf(rho[s], v.y, acc.y);
-                        acc.z = fmaf(rho[s], v.z, acc.z);
-                        acc.w = fmaf(rho[s], v.w, acc.w);
-                    }
-                }
-            }
-            const int im = a.R - 1 - i;
-            a.c[((int64_t)b * a.R + i) * a.NH + m] = make_float2(acc.x, acc.y);
-            if (im != i) a.c[((int64_t)b * a.R + im) * a.NH + m] = make_float2(acc.z, acc.w);
-        }
-        __syncthreads();
-    }
-}
-
-}  // namespace
-
-int contract_ring_block() { return kRingBlock; }
-
-int contract_band_limit() { return kBand2; }
-int contract_band_rings() { return kRings2; }
-
-cudaError_t launch_contract_band(const ContractArgs &a, int nchunks, int max_union, cudaStream_t st)
-{
-    const size_t smem = std::max(2 * (size_t)max_union * kModes2 * sizeof(float4),
-                                 (size_t)kBand2 * kModes2 * kRings2 * sizeof(float));
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_band,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((a.NH + kModes2 - 1) / kModes2, (a.nrep + kRings2 - 1) / kRings2, nchunks);
-    return launch_chained(k_contract_band, grid, kModes2 * kRings2, smem, st, true, 1, a, max_union);
-}
-
-namespace {
 
 // Coefficients rho_m of the pairs next to the poles.  Those pairs have up to N/2 + 1 samples,
 // so generating them inside the contraction would leave a few CTAs running long after the
@@ -481,15 +250,6 @@ cudaError_t launch_taps(const TapArgs &a, int nk, int64_t maxtaps, cudaStream_t 
     const int64_t want = (maxtaps + 128 * (kTapThreads / 32) - 1) / (128 * (kTapThreads / 32));
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, (device_sms() + nk - 1) / nk));
     return launch_chained(k_taps, dim3(blocks, nk), kTapThreads, smem, st, after_prev, 1, a);
-}
-
-cudaError_t launch_contract(const ContractArgs &a, int nchunks, size_t smem, cudaStream_t st)
-{
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract<kRingBlock>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((a.NH + kModeBlock - 1) / kModeBlock, (a.nrep + kRingBlock - 1) / kRingBlock, nchunks);
-    return launch_chained(k_contract<kRingBlock>, grid, kModeBlock * kMapGroups, smem, st, true, 1, a);
 }
 
 }  // namespace arkcos

@@ -9,6 +9,10 @@
 // loads in flight, and one thread issues tcgen05.mma kind::tf32 with the accumulator in tensor
 // memory:
 //     D = C_hi T_hi + C_hi T_lo + C_lo T_hi      (3xTF32, FP32 accumulation).
+// The plain FP32 form (F32) is the same kernel with the sums on the CUDA cores: the samples in
+// shared memory, a thread's cosine times broadcast samples into 64 register sums by packed FMAs,
+// and the coefficients stored to tensor memory (it replaces one recurrence per pair and mode; one
+// nside-2048 map 2.52 -> 0.98 ms, six nside-4096 maps of an 8' support 15.0 -> 7.9 ms).
 // The rings of the block go in groups of G (2 or 4) consecutive rings; slot u of ring l holds
 // the pair of that ring with input ring jlo(first ring of its group) + u (zero when that ring is
 // outside its band), so the rings of a group index one common run of 32 input rings.  On the
@@ -52,6 +56,7 @@ using namespace tc;
 constexpr int kTcModes = 128;          // M of the MMA: modes per CTA (TMEM lanes)
 constexpr int kTcBand = 32;            // input-ring slots per group (columns per ring)
 constexpr int kTcK = 16;               // samples per pass (2 MMA K-steps of 8)
+constexpr int kF32K = 32;              // samples per pass of the plain FP32 form
 constexpr int kTcRun = 128;            // samples per generated run (longest tensor-core sum)
 constexpr uint32_t kTcSBO = 4 * kLBO;  // row octets of an operand of 16 samples
 
@@ -67,8 +72,17 @@ struct TcShape {
     static constexpr uint32_t kA = kTcModes / 8 * kTcSBO;  // one cosine operand (hi or lo)
     static constexpr uint32_t kB = kN / 8 * kTcSBO;        // the samples (hi or lo) of every column
     static constexpr uint32_t kStage = 4 * kA + 2 * kB;
+    static_assert((uint32_t)kF32K * kN * sizeof(float) <= kStage, "the FP32 form's samples fit a stage");
     static constexpr int kStages = RB / 8;
 };
+
+// (a, b) += c v, v as two packed pairs
+__device__ __forceinline__ void fma4(float2 &a, float2 &b, float c, const float4 &v)
+{
+    const float2 cc = make_float2(c, c);
+    a = __ffma2_rn(cc, make_float2(v.x, v.y), a);
+    b = __ffma2_rn(cc, make_float2(v.z, v.w), b);
+}
 
 // acc += c v for the four lanes of v, as two packed two-lane FMAs (each lane rounds as fmaf)
 __device__ __forceinline__ void fma4(float4 &acc, float c, const float4 &v)
@@ -87,6 +101,7 @@ __device__ __forceinline__ void stage_rows(float4 *dst, const float4 *__restrict
 {
     const int c = threadIdx.x % kTcModes, mm = m0 + c;
     const bool mv = mm < NH;
+    if (m0 + (c & ~31) >= NH) rows = 0;  // nobody reads this warp's modes
     const float4 *src = sp4b + (mv ? mm : 0);
     for (int jj = threadIdx.x / kTcModes; jj < rows; jj += THREADS / kTcModes) {
         const int j = j0 + jj;
@@ -95,7 +110,7 @@ __device__ __forceinline__ void stage_rows(float4 *dst, const float4 *__restrict
     cp_async_commit();
 }
 
-template <int RB, int G, bool WIDE>
+template <int RB, int G, bool WIDE, bool F32>
 __global__ void __launch_bounds__(TcShape<RB, G>::kThreads, 16 / RB)
 k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__restrict__ cos2n, int nkc_tab, int srows,
               int nbuf, uint32_t rows0, uint32_t ctl)
@@ -135,6 +150,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
     // run starts at input ring jg0
     const int i0 = r0 + G * grp;
     const bool v0 = G * grp < nr;
+    const bool wv = v0 && m0 + q4 * 32 < a.NH;  // some mode of the warp exists (N/2 + 1 modes: one in the last block)
     const int jg0 = v0 ? kd.jlo[i0] : 0;
     const int ju0 = kd.jlo[r0];
     const int jlast = kd.jhi[r0 + nr - 1];
@@ -266,11 +282,108 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                 // accumulator truncates each addition at the size of the running sum, so what is
                 // small comes first: the last samples of a run (a beam's tail) before the first,
                 // and the cross terms of a pass before its hi x hi products
+                constexpr int kK = F32 ? kF32K : kTcK;
                 const int kb = run * kTcRun;
                 auto cap = [&](int k) { return max(0, min(kTcRun, k - kb)); };
-                const int n0 = single ? (cap(kall) + kTcK - 1) / kTcK : (cap(max(k00, k10)) + kTcK - 1) / kTcK;
-                const int np = single ? n0 : n0 + (cap(max(k01, k11)) + kTcK - 1) / kTcK;
+                const int n0 = single ? (cap(kall) + kK - 1) / kK : (cap(max(k00, k10)) + kK - 1) / kK;
+                const int np = single ? n0 : n0 + (cap(max(k01, k11)) + kK - 1) / kK;
                 early = rows0 != 0 && np == 1 && b0 < b1;
+                if constexpr (F32) {
+                    // plain FP32 form: the samples of every column in shared memory, sample-major;
+                    // a thread sums two of its rings at a time in registers (packed two-lane FMAs of
+                    // its mode's cosine with broadcast samples), tensor memory holding the sums
+                    float *ts = reinterpret_cast<float *>(smem);  // [kF32K][kTcN]
+                    for (int i = 0; i < np; ++i) {
+                        const bool second = !single && i >= n0;
+                        const int k0 = kb + (second ? np - 1 - i : n0 - 1 - i) * kK;
+                        const int fA = single ? f0s : (int)second, fB = single ? f1s : (int)second;
+                        const int krem = (single ? kall : (second ? max(k01, k11) : max(k00, k10))) - k0;
+                        const int nq = (min(kK, krem) + 3) / 4;  // groups of four samples
+                        if (i > 0) __syncthreads();
+                        for (int c = tid; c < kTcN; c += Sh::kThreads) {
+                            const int sf = s_S[c], S = (sf & 1) == (c < kTile ? fA : fB) ? sf >> 1 : -1;
+                            const float *tp = taps + s_toff[c] + k0;
+                            for (int q = 0; q < nq; ++q) {
+                                const float4 v = k0 + 4 * q <= S ? __ldg(reinterpret_cast<const float4 *>(tp + 4 * q))
+                                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+                                ts[(4 * q) * kTcN + c] = v.x;  // (slots past the last sample hold zeros)
+                                ts[(4 * q + 1) * kTcN + c] = v.y;
+                                ts[(4 * q + 2) * kTcN + c] = v.z;
+                                ts[(4 * q + 3) * kTcN + c] = v.w;
+                            }
+                        }
+                        if (early) issue(w, b0, 0);
+                        __syncthreads();
+                        // cosines of four samples from k for offset f (hi + lo of the tables: the
+                        // FP32 value)
+                        auto cosines = [&](int k, int f, float (&c)[4]) {
+                            if (!WIDE || k < nkc_tab * 32) {
+                                const float4 *t4 = reinterpret_cast<const float4 *>(
+                                    ctab + ((((size_t)blockIdx.x * 2 + f) * nkc_tab + (k >> 5)) * 2) * 4096) +
+                                    (mrow >> 3) * 64 + ((k & 31) >> 2) * 8 + (mrow & 7);
+                                const float4 h = __ldg(t4), l = __ldg(t4 + 1024);
+                                c[0] = h.x + l.x;
+                                c[1] = h.y + l.y;
+                                c[2] = h.z + l.z;
+                                c[3] = h.w + l.w;
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    const float2 v = __ldg(&cos2n[m * (2 * (k + j) + f) % (2 * a.N)]);
+                                    c[j] = v.x + v.y;
+                                }
+                            }
+                        };
+#pragma unroll 1
+                        for (int rp = 0; rp < (wv ? G / 2 : 0); ++rp) {
+                            float2 sum[2][2][8];  // [ring][tile][column pair]
+                            const int l0 = G * grp + 2 * rp;
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) {
+                                uint32_t old[16];
+                                if (i > 0) {
+                                    tmem_ld_async(lane_base + (uint32_t)((x & 1) * kTile + (l0 + x / 2) * 16), old);
+                                    tmem_wait_ld();
+                                }
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    sum[x / 2][x & 1][j] = i > 0 ? make_float2(__uint_as_float(old[2 * j]), __uint_as_float(old[2 * j + 1]))
+                                                                 : make_float2(0.f, 0.f);
+                            }
+#pragma unroll 1
+                            for (int q = nq - 1; q >= 0; --q) {
+                                float cA[4], cB[4];
+                                cosines(k0 + 4 * q, fA, cA);
+                                if (fA != fB) cosines(k0 + 4 * q, fB, cB);
+                                else
+#pragma unroll
+                                    for (int j = 0; j < 4; ++j) cB[j] = cA[j];
+#pragma unroll
+                                for (int j = 3; j >= 0; --j) {
+#pragma unroll
+                                    for (int x = 0; x < 4; ++x) {
+                                        const float c = x & 1 ? cB[j] : cA[j];
+                                        const float4 *t4 = reinterpret_cast<const float4 *>(
+                                            ts + (4 * q + j) * kTcN + (x & 1) * kTile + (l0 + x / 2) * 16);
+#pragma unroll
+                                        for (int y = 0; y < 4; ++y) fma4(sum[x / 2][x & 1][2 * y], sum[x / 2][x & 1][2 * y + 1], c, t4[y]);
+                                    }
+                                }
+                            }
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) {
+                                float out[16];
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) {
+                                    out[2 * j] = sum[x / 2][x & 1][j].x;
+                                    out[2 * j + 1] = sum[x / 2][x & 1][j].y;
+                                }
+                                tmem_st16(lane_base + (uint32_t)((x & 1) * kTile + (l0 + x / 2) * 16), out);
+                            }
+                        }
+                    }
+                    __syncthreads();
+                } else {
                 // a thread takes 8 samples of a column, loaded four at a time (tap offsets are
                 // multiples of 4 and each pair's slots are padded to 4, so a float4 that starts at
                 // or before the last sample stays inside the pair); others read as zero
@@ -405,6 +518,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                 ok = __syncthreads_and(ok);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 have = ok;
+                }
             } else {
                 // blocks next to the poles have more samples per pair than the cosine tables hold:
                 // their coefficients were tabulated before this launch; they go to the same
@@ -476,7 +590,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                         }
                     }
                 }
-                if (v0 && have) {  // warp-uniform: the tensor-memory loads are warp-collective
+                if (wv && have) {  // warp-uniform: the tensor-memory loads are warp-collective
                     const float4 *col = reinterpret_cast<const float4 *>(smem + (cur ? off1 : off0)) + joff * kTcModes + mrow;
                     // CH slots at a time, in the order of the input rings (whatever the groups): the
                     // coefficients of the G rings (a ring's even and odd slots lie in different
@@ -759,40 +873,43 @@ size_t contract_tc_smem(int rb, int gs, int srows, int want_nbuf)
     return tc_ctl(rb, contract_tc_nbuf(rb, gs, srows, want_nbuf), srows) + 32;
 }
 
-// Whether blocks of 16 rings with moving windows of srows staged rows fit an SM.
-bool contract_tc_wide_fits(int srows) { return contract_tc_smem(16, 4, srows, 0) <= kTcSmemLimit; }
+int contract_band_limit() { return kTcBand; }
 
 namespace {
 
-template <int RB, int G, bool WIDE>
+template <int RB, int G, bool WIDE, bool F32>
 cudaError_t launch_tc(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, int nbuf, cudaStream_t st)
 {
     const size_t ctl = tc_ctl(RB, nbuf, srows), smem = ctl + 32;
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_tc<RB, G, WIDE>,
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_tc<RB, G, WIDE, F32>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.NH + kTcModes - 1) / kTcModes, (a.nrep + RB - 1) / RB, nchunks);
-    return launch_chained(k_contract_tc<RB, G, WIDE>, grid, TcShape<RB, G>::kThreads, smem, st, true, 1, a, tb.ctab,
+    return launch_chained(k_contract_tc<RB, G, WIDE, F32>, grid, TcShape<RB, G>::kThreads, smem, st, true, 1, a, tb.ctab,
                           tb.cos2n, tb.nkc, srows, nbuf, tc_rows0(RB, srows), (uint32_t)ctl);
 }
 
 }  // namespace
 
-cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, int nchunks, const TcTables &tb, int srows,
-                               int want_nbuf, cudaStream_t st)
+cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int nchunks, const TcTables &tb,
+                               int srows, int want_nbuf, cudaStream_t st)
 {
     const int nbuf = contract_tc_nbuf(rb, gs, srows, want_nbuf);
+    if (f32) return launch_tc<8, 4, false, true>(a, nchunks, tb, srows, nbuf, st);
     if (rb == 16)
-        return gs == 4 ? launch_tc<16, 4, false>(a, nchunks, tb, srows, nbuf, st)
-                       : launch_tc<16, 2, false>(a, nchunks, tb, srows, nbuf, st);
-    return gs == 4 ? launch_tc<8, 4, false>(a, nchunks, tb, srows, nbuf, st)
-                   : launch_tc<8, 2, false>(a, nchunks, tb, srows, nbuf, st);
+        return gs == 4 ? launch_tc<16, 4, false, false>(a, nchunks, tb, srows, nbuf, st)
+                       : launch_tc<16, 2, false, false>(a, nchunks, tb, srows, nbuf, st);
+    return gs == 4 ? launch_tc<8, 4, false, false>(a, nchunks, tb, srows, nbuf, st)
+                   : launch_tc<8, 2, false, false>(a, nchunks, tb, srows, nbuf, st);
 }
 
 // Bands of any width: blocks of 16 rings in groups of four, the 32 slots moving along the band.
-cudaError_t launch_contract_tc_wide(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, cudaStream_t st)
+cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks, const TcTables &tb, int srows,
+                                    cudaStream_t st)
 {
-    return launch_tc<16, 4, true>(a, nchunks, tb, srows, contract_tc_nbuf(16, 4, srows, 0), st);
+    const int nbuf = contract_tc_nbuf(16, 4, srows, 0);
+    return f32 ? launch_tc<16, 4, true, true>(a, nchunks, tb, srows, nbuf, st)
+               : launch_tc<16, 4, true, false>(a, nchunks, tb, srows, nbuf, st);
 }
 
 // Knot-gradient projection of pairs [pfirst, npairs) into X [npairs - pfirst][128] (rows of

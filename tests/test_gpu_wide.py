@@ -1,5 +1,5 @@
-"""Bands wider than 32 input rings in the tensor-core form (the 32 slots move along the band),
-against the FP64 oracle: one window past the narrow form, several windows, bands over most of
+"""Bands wider than 32 input rings (the 32 slots of the contraction move along the band), in both
+forms, against the FP64 oracle: one window past the narrow form, several windows, bands over most of
 the sphere, partial ring blocks, kernel grids that are no power of two, rings of more than 128
 samples with and without tabulated coefficients.  Tolerance: the method's fractional RMS, 1e-5,
 as in test_gpu_parity.py."""
@@ -37,9 +37,10 @@ def _setup(spec, supports, nmaps):
     (("ecp", 61, 720), [60.0], 1, False, None),               # over 128 samples in every pair near a pole
     (("healpix", 512), [6.0], 1, False, [0, 1, 15, 16, 40, 170, 186, 511, 512, 1023, 1900, 2046]),  # untabulated
 ])
-def test_wide_band_tensor_core(spec, supports, nmaps, basic, rings):
+@pytest.mark.parametrize("form", ["tf32", "fp32"])
+def test_wide_band(spec, supports, nmaps, basic, rings, form):
     ark, g, prof, ks, x, xt = _setup(spec, supports, nmaps)
-    flags = ark.FLAG_3XTF32 | (ark.FLAG_BASIC if basic else 0)
+    flags = (ark.FLAG_3XTF32 if form == "tf32" else 0) | (ark.FLAG_BASIC if basic else 0)
     y = ark.convolve(g, ks[0] if len(ks) == 1 else ks, xt, flags).cpu().numpy()
     _, _, _, n, off = oracle.geometry(spec)
     at = slice(None) if rings is None else np.concatenate([np.arange(off[r], off[r] + n[r]) for r in rings])
