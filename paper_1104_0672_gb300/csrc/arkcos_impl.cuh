@@ -15,8 +15,7 @@ constexpr int kMaxKernelsPerLaunch = 32;  // per-map beams handled per contracti
 constexpr int kMaxPolarPairs = 16384;      // most pairs whose coefficients are tabulated per call
 constexpr int kModeBlock = 128;           // modes per CTA of the generic knot-gradient kernel
 constexpr int kMaxFftM = 8192;            // largest in-shared-memory ring FFT buffer (complex pairs)
-constexpr int kMaxSplitM = 8192;          // buffer of the quarter transforms of split rings
-constexpr int kSplitClass = 15;           // FFT class index of the split rings
+constexpr int kBluMin = 9, kBluMax = 12;  // log2 buffer of the split Bluestein classes (ring_blu.cuh)
 
 // Ring table on the device (structure of arrays, R entries each).
 struct RingDev {
@@ -37,7 +36,7 @@ struct FftClass {
     int threads = 0;
     int count = 0;
     int stage_c = 0;      // some ring of the class is shorter than N / 4
-    int split = 0;        // rings of n = 4q pixels transformed as four q-point Bluestein DFTs
+    int blu = 0;          // a split Bluestein class (ring_blu.cuh)
     int tab = 0;          // largest chirp + phase table of the class (complex words)
     int *reps = nullptr;  // device array of representative (northern) ring indices
 };
@@ -158,7 +157,6 @@ struct FftFwdArgs {
     int weight;         // multiply spectra by the ring weight
     int zero_poles;     // treat rings 0 and R-1 as zero (adjoint input)
     int tab;            // shared-memory words for the per-ring chirp and phase tables
-    int split;          // the class holds split rings (n = 4q, see FftClass)
 };
 
 struct FftInvArgs {
@@ -247,16 +245,19 @@ __device__ __forceinline__ float4 paired_coeff(const float4 *__restrict__ sp4, i
 cudaError_t launch_taps(const TapArgs &a, int nk, int64_t maxtaps, cudaStream_t st, bool after_prev);
 cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs, const float2 *tw, int twM,
                              cudaStream_t st);
-size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads, bool split);  // shared memory of a ring FFT class
+size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads);  // shared memory of a ring FFT class
 cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int threads, cudaStream_t st);
 // Ring FFT class launches.  after_prev: the previous kernel on the stream is the previous class
 // of the same stage, and this launch may begin while it still runs (ring_common.cuh
 // stage_allow_next / stage_wait_prev).
 cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
-cudaError_t launch_fft_fwd_split(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
+cudaError_t launch_blu_fwd(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev);
+cudaError_t launch_blu_inv(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev);
+cudaError_t launch_blu_spectra(const FftFwdArgs &a, float2 *fb, int count, cudaStream_t st);  // a.logM, rd, reps, tw
+int blu_table_words(int h);                // words of the per-ring tables of a ring of n = 2h pixels
+size_t blu_smem_bytes(int M, int tab);
 int fft_map_chunk(int count, int nmaps, int split_mult);  // maps per CTA of a ring FFT launch over `count` ring pairs
 cudaError_t launch_fft_inv(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
-cudaError_t launch_fft_inv_split(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
 
 // Launch of kernel(args...) in clusters of `cluster` CTAs along x, with the
 // programmatic-serialization attribute when after_prev: the kernel may then begin while the

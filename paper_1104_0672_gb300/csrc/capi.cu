@@ -191,10 +191,10 @@ arkcos_status finish_grid(Grid &g)
     if ((st = upload(&g.d_theta, g.theta)) != ARKCOS_OK) return st;
     // FFT launch classes by buffer size.  A ring of n pixels is transformed as the complex
     // sequence of its h = n/2 pixel pairs, two mirror rings at a time: buffer h (a power of
-    // two) or the Bluestein size >= 2h - 1; buffers up to 1024 share one launch.  Rings whose
-    // buffer would exceed kMaxFftM are split as n = 4q into four q-point Bluestein transforms
-    // (class kSplitClass)
-    std::vector<std::vector<int>> cls(kSplitClass + 1);
+    // two) or, for short rings, the Bluestein size >= 2h - 1 (buffers up to 1024 share one
+    // launch).  Longer Bluestein rings go through the split convolutions of ring_blu.cuh: l = h/2
+    // points (h for odd h) in buffers of >= l.
+    std::vector<std::vector<int>> cls(14), blu(kBluMax + 1);
     int maxM = 2, maxpow2 = 2;
     auto buffer_of = [](int64_t l) {  // power-of-two buffer of an l-point transform (>= 2)
         if (l >= 2 && is_pow2(l)) return l;
@@ -202,51 +202,51 @@ arkcos_status finish_grid(Grid &g)
     };
     auto bluestein = [](int64_t l) { return l < 2 || !is_pow2(l); };
     for (int j = 0; j < g.nrep; ++j) {
-        const int n = g.n[j];
-        const int64_t M = buffer_of(n / 2);
+        const int n = g.n[j], h = n / 2, l = (h & 1) ? h : h / 2;
         if (is_pow2(n)) maxpow2 = std::max(maxpow2, n);
-        if (M <= kMaxFftM) {
-            cls[std::max(ilog2(M), 10)].push_back(j);
-            maxM = std::max<int>(maxM, (int)M);
-        } else if (n % 4 == 0 && !is_pow2(n / 4) && buffer_of(n / 4) <= kMaxSplitM) {
-            cls[kSplitClass].push_back(j);
-            maxM = std::max<int>(maxM, (int)buffer_of(n / 4));
+        if (bluestein(h) && l > (1 << (kBluMin - 1)) && l <= (1 << kBluMax)) {
+            blu[ilog2(l)].push_back(j);
+            maxM = std::max(maxM, 2 << ilog2(l));
+        } else if (buffer_of(h) <= kMaxFftM && (!bluestein(h) || buffer_of(h) <= 1024)) {
+            cls[std::max(ilog2(buffer_of(h)), 10)].push_back(j);
+            maxM = std::max<int>(maxM, (int)buffer_of(h));
         } else {
             return fail(ARKCOS_EUNSUPPORTED, "ring of %d pixels needs an FFT buffer of %lld > %d",
-                        n, (long long)M, kMaxFftM);
+                        n, (long long)buffer_of(h), kMaxFftM);
         }
     }
-    for (int l = 0; l <= kSplitClass; ++l) {
-        if (cls[l].empty()) continue;
+    // (in order of the work per CTA: a stage launches its classes from the last to the first)
+    for (auto [l, b] : {std::pair<int, bool>{10, false}, {9, true}, {11, false}, {10, true}, {12, false}, {13, false},
+                        {11, true}, {12, true}}) {
+        const std::vector<int> &reps = b ? blu[l] : cls[l];
+        if (reps.empty()) continue;
         FftClass c;
         int mx = 0;
-        for (int j : cls[l]) {
+        for (int j : reps) {
             const int n = g.n[j];
-            if (l == kSplitClass) {
-                // buffer of the q-point transforms | the n-point spectrum | the chirp of q
-                mx = std::max(mx, (int)buffer_of(n / 4));
-                c.tab = std::max(c.tab, n + n / 8 + 1);
+            if (b) {
+                mx = 1 << l;
+                c.tab = std::max(c.tab, blu_table_words(n / 2));
                 continue;
             }
-            const int M = (int)buffer_of(n / 2);
-            mx = std::max(mx, M);
+            mx = std::max(mx, (int)buffer_of(n / 2));
             if (4 * n < g.N) c.stage_c = 1;
             // the chirp of h (h/2 + 1, Bluestein rings) and exp(-+ i pi m / n), m <= n/2
             c.tab = std::max(c.tab, (bluestein(n / 2) ? (n / 2) / 2 + 1 : 0) + n / 2 + 1);
         }
-        c.split = l == kSplitClass;
+        c.blu = b;
         c.M = mx;
         c.logM = ilog2(mx);
-        c.threads = std::min(512, std::max(c.split ? 64 : 256, c.M / 16));  // as ring::ClassShape
-        c.count = (int)cls[l].size();
+        c.threads = std::min(512, std::max(256, c.M / 16));  // as ring::ClassShape
+        c.count = (int)reps.size();
         // staging the coefficients of short rings is an optimisation: drop it where it does not
         // fit beside the transform buffer (long kernel grids)
-        if (c.stage_c && fft_smem_bytes(c.M, g.N, true, c.tab, c.threads, c.split) > 227 * 1024) c.stage_c = 0;
-        const size_t smem = fft_smem_bytes(c.M, g.N, c.stage_c != 0, c.tab, c.threads, c.split);
+        if (c.stage_c && fft_smem_bytes(c.M, g.N, true, c.tab, c.threads) > 227 * 1024) c.stage_c = 0;
+        const size_t smem = b ? blu_smem_bytes(c.M, c.tab) : fft_smem_bytes(c.M, g.N, c.stage_c != 0, c.tab, c.threads);
         if (smem > 227 * 1024)
             return fail(ARKCOS_EUNSUPPORTED, "ring FFT class of buffer %d needs %zu bytes of shared memory",
                         c.M, smem);
-        if ((st = upload(&c.reps, cls[l])) != ARKCOS_OK) return st;
+        if ((st = upload(&c.reps, reps)) != ARKCOS_OK) return st;
         g.fft.push_back(c);
     }
     // stage twiddles tw[h + p] = exp(-2 pi i p / (2h)): the transform passes, the kernel-grid
@@ -271,11 +271,9 @@ arkcos_status finish_grid(Grid &g)
             if (cudaMemcpy(reps.data(), c.reps, c.count * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
                 return fail(ARKCOS_ECUDA, "reading the FFT class table");
             for (int j : reps) {
-                // the chirp of the ring's pair sequence, or of its quarter for split rings
-                const int64_t l = c.split ? g.n[j] / 4 : g.n[j] / 2;
-                if (!bluestein(l)) continue;
+                if (!bluestein(g.n[j] / 2)) continue;
                 fboff[j] = (int)tot;
-                tot += buffer_of(l);
+                tot += c.blu ? 2 * c.M : buffer_of(g.n[j] / 2);
             }
         }
         if (tot > (int64_t)0x7fffffff) return fail(ARKCOS_EUNSUPPORTED, "chirp spectra too large");
@@ -290,8 +288,9 @@ arkcos_status finish_grid(Grid &g)
                 a.tw = g.d_tw;
                 a.reps = c.reps;
                 a.M = c.M;
-                a.split = c.split;
-                e = launch_chirp_spectra(a, g.d_fb, c.count, c.threads, 0);
+                a.logM = c.logM;
+                e = c.blu ? launch_blu_spectra(a, g.d_fb, c.count, 0)
+                          : launch_chirp_spectra(a, g.d_fb, c.count, c.threads, 0);
                 if (e != cudaSuccess) return cuda_fail(e, "chirp spectra");
             }
             e = cudaStreamSynchronize(0);
@@ -612,8 +611,7 @@ arkcos_status run_fft_fwd(const Grid &g, const float *map, float2 *spec, float4 
         a.weight = weight;
         a.zero_poles = zero_poles;
         a.tab = c.tab;
-        a.split = c.split;
-        if (c.split) CK(launch_fft_fwd_split(a, c.count, c.threads, st, after_prev));
+        if (c.blu) CK(launch_blu_fwd(a, c.count, st, after_prev));
         else CK(launch_fft_fwd(a, c.count, c.threads, st, after_prev));
     }
     return ARKCOS_OK;
@@ -647,7 +645,7 @@ arkcos_status run_fft_inv(const Grid &g, const float2 *cbuf, float *map, int64_t
         a.skip_poles = skip_poles;
         a.stage_c = c.stage_c;
         a.tab = c.tab;
-        if (c.split) CK(launch_fft_inv_split(a, c.count, c.threads, st, after_prev));
+        if (c.blu) CK(launch_blu_inv(a, c.count, st, after_prev));
         else CK(launch_fft_inv(a, c.count, c.threads, st, after_prev));
     }
     return ARKCOS_OK;

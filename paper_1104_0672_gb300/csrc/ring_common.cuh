@@ -9,13 +9,12 @@
 // (fft_engine.cuh):
 //   - h a power of two (M = h): one forward DIF transform (digit-reversed spectrum) or, on the
 //     inverse side, the adjoint transform from digit-reversed input;
-//   - other h: Bluestein's chirp-z algorithm (1970) with M >= 2h - 1: DIF of the chirped
-//     sequence, pointwise product with the chirp spectrum (precomputed per grid) fused with
-//     the last DIF and first adjoint pass, adjoint back to natural order.
+//   - other h with buffers up to 1024: Bluestein's chirp-z algorithm (1970) with M >= 2h - 1:
+//     DIF of the chirped sequence, pointwise product with the chirp spectrum (precomputed per
+//     grid) fused with the last DIF and first adjoint pass, adjoint back to natural order;
+//   - longer ones: the split convolutions of ring_blu.cuh, in classes of their own.
 // The buffer size is a compile-time parameter of the per-ring code: a launch covers rings of
-// one or several sizes and each CTA branches once to the code for its own size.  Rings too
-// long for the largest buffer (n = 4q, 2h - 1 > 8192) go through four q-point transforms
-// instead (the split path, one ring pair packed as one complex sequence).
+// one or several sizes and each CTA branches once to the code for its own size.
 #pragma once
 #include "fft_engine.cuh"
 
@@ -47,13 +46,6 @@ __device__ __forceinline__ void tables(float2 *chirp, float2 *phase, int n, int 
             phase[m] = sgn < 0 ? w : make_float2(w.x, -w.y);
         }
     }
-    __syncthreads();
-}
-
-// Per-CTA chirp table of the split path: chirp[k] = exp(sgn i pi k^2 / q), k <= q/2.
-__device__ __forceinline__ void chirp_table(float2 *chirp, int q, int sgn)
-{
-    for (int k = threadIdx.x; 2 * k <= q; k += blockDim.x) chirp[k] = expipi_ratio(sgn * k * k, q);
     __syncthreads();
 }
 

@@ -15,8 +15,8 @@ using fft::cpair;
 using ring::chirp_at;
 
 // DIF spectrum (digit-reversed positions) of the Bluestein sequence b_k = exp(+i pi k^2 / l),
-// |k| < l, circular in M, for the l-point transform of every Bluestein ring of a class
-// (l = n/2, or n/4 for split rings): computed once per grid.
+// |k| < l, circular in M, for the l = n/2-point transform of every Bluestein ring of the class of
+// short rings: computed once per grid.
 struct ChirpCta {
     float2 *buf, *fb;
     const float2 *tw;
@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(512) k_chirp_spectra(FftFwdArgs a, float2 *fb_
 {
     extern __shared__ float2 buf[];
     const int j = a.reps[blockIdx.x];
-    const int l = a.split ? a.rd.n[j] / 4 : a.rd.n[j] / 2;
+    const int l = a.rd.n[j] / 2;
     if (!ring::bluestein(l)) return;  // power-of-two transform: no chirp
     ChirpCta c{buf, fb_all + a.rd.fboff[j], a.tw, l};
     ring::dispatch(ring::log2_buffer(l), c);
@@ -56,7 +56,7 @@ struct FwdCta {
     const float2 *chirp, *phase;  // chirp of h (Bluestein rings), exp(-i pi m / n) for m <= n/2
     const float2 *fb;
     int j, j2, n, h, hs;
-    bool pair, blu, zero;
+    bool pair, blu, zero;  // (blu: classes up to 2^10 only)
     float wsc;
 
     // exp(-i pi m / n), 0 <= m <= n/2
@@ -170,6 +170,7 @@ struct FwdCta {
     __device__ void run()
     {
         constexpr int M = 1 << L;
+        const bool blu = L <= 10 && this->blu;
         const fft::Smem<L, cpair> sm{buf};
         const float inv_m = 1.0f / (float)M;
         const int bend = min(a.B, (int)(blockIdx.y + 1) * a.mchunk);
@@ -195,7 +196,7 @@ struct FwdCta {
                 }
                 return v;
             };
-            if (blu) {
+            if (L <= 10 && blu) {
                 fft::convolve<L, false>(buf, a.tw, fb, ld, sm);
                 epilogue<L>(
                     b, [&](int k) { return fft::e_mul(sm(k), cscalef(chirp_at(chirp, k, h), inv_m)); },
@@ -207,120 +208,6 @@ struct FwdCta {
         }
     }
 };
-
-// Rings of n = 4q pixels too long for one Bluestein buffer: decimation in time by 4,
-//   X[k' + t q] = sum_p W_n^{p k'} W_4^{p t} Y_p[k'],   Y_p = DFT_q(z[4 s + p]),
-// with the ring pair packed as one complex sequence z = x_j + i x_j2, the four q-point DFTs by
-// Bluestein one after the other into the spectrum area X of shared memory, then the radix-4
-// combination in place and the split of the two rings.
-struct FwdSplitCta {
-    const FftFwdArgs &a;
-    float2 *buf, *X;
-    const float2 *chirp, *fb;  // chirp exp(-i pi k^2 / q), k <= q/2
-    int j, j2, n, hs;
-    bool pair, zero;
-    float wsc;
-
-    __device__ __forceinline__ float2 phase_at(int m) const
-    {
-        return hs ? expipi_ratio(-m, n) : make_float2(1.f, 0.f);
-    }
-
-    template <int L>
-    __device__ void run()
-    {
-        const int q = n / 4;
-        const float inv_m = 1.0f / (float)(1 << L);
-        const int bend = min(a.B, (int)(blockIdx.y + 1) * a.mchunk);
-        for (int b = blockIdx.y * a.mchunk; b < bend; ++b) {
-            const float *m1 = a.map + (int64_t)b * a.npix + a.rd.poff[j];
-            const float *m2 = a.map + (int64_t)b * a.npix + a.rd.poff[j2];
-            for (int p = 0; p < 4; ++p) {
-                auto ld = [&](int s) {
-                    float2 v = make_float2(0.f, 0.f);
-                    if (s < q && !zero) {
-                        v.x = __ldg(&m1[4 * s + p]);
-                        v.y = pair ? __ldg(&m2[4 * s + p]) : 0.f;
-                        v = cmulf(v, chirp_at(chirp, s, q));
-                    }
-                    return v;
-                };
-                float2 *Y = X + p * q;
-                auto st = [&](int s, float2 v) {
-                    if (s < q) Y[s] = cscalef(cmulf(v, chirp_at(chirp, s, q)), inv_m);
-                };
-                fft::convolve<L, false>(buf, a.tw, fb, ld, st);
-            }
-            for (int k = threadIdx.x; k < q; k += blockDim.x) {
-                float2 y0 = X[k], y1 = X[q + k], y2 = X[2 * q + k], y3 = X[3 * q + k];
-                const float2 w1 = expipi_ratio(-2 * k, n), w2 = cmulf(w1, w1), w3 = cmulf(w1, w2);
-                y1 = cmulf(y1, w1);
-                y2 = cmulf(y2, w2);
-                y3 = cmulf(y3, w3);
-                fft::dft4<false>(y0, y1, y2, y3);
-                X[k] = y0;
-                X[q + k] = y1;
-                X[2 * q + k] = y2;
-                X[3 * q + k] = y3;
-            }
-            __syncthreads();
-            // split of the packed ring pair, phase, weight and the extension (as FwdCta)
-            if (!a.ext4) {
-                float2 *s1 = a.spec + (int64_t)b * a.nspec + a.rd.soff[j];
-                float2 *s2 = a.spec + (int64_t)b * a.nspec + a.rd.soff[j2];
-                for (int m = threadIdx.x; m <= n / 2; m += blockDim.x) {
-                    const int mn = m == 0 ? 0 : n - m;
-                    const float2 zm = X[m], zn = X[mn];
-                    const float2 ph = phase_at(m);
-                    s1[m] = cscalef(cmulf(make_float2(0.5f * (zm.x + zn.x), 0.5f * (zm.y - zn.y)), ph), wsc);
-                    if (pair) s2[m] = cscalef(cmulf(make_float2(0.5f * (zm.y + zn.y), -0.5f * (zm.x - zn.x)), ph), wsc);
-                }
-            } else {
-                float4 *o4 = a.spec4 + ((int64_t)b * a.nrep + j) * a.NH;
-                for (int m = threadIdx.x; m < a.NH; m += blockDim.x) {
-                    const int qq = m / n, mm = m - qq * n;
-                    const bool up = 2 * mm > n;
-                    const int mb = up ? n - mm : mm;
-                    const int mn = mb == 0 ? 0 : n - mb;
-                    const float2 zm = X[mb], zn = X[mn];
-                    const float2 ph = phase_at(mb);
-                    float2 ea = cmulf(make_float2(0.5f * (zm.x + zn.x), 0.5f * (zm.y - zn.y)), ph);
-                    float2 eb = pair ? cmulf(make_float2(0.5f * (zm.y + zn.y), -0.5f * (zm.x - zn.x)), ph) : ea;
-                    float sc = wsc;
-                    if (a.basic) {
-                        if (qq > 0 || up) sc = 0.f;
-                        else if (2 * mm == n && n < a.N) sc *= 0.5f;
-                    } else {
-                        if (up) {
-                            ea.y = -ea.y;
-                            eb.y = -eb.y;
-                        }
-                        if (hs && ((qq + (up ? 1 : 0)) & 1)) sc = -sc;
-                    }
-                    o4[m] = make_float4(sc * ea.x, sc * ea.y, sc * eb.x, sc * eb.y);
-                }
-            }
-            __syncthreads();
-        }
-    }
-};
-
-__global__ void __launch_bounds__(512) k_fft_fwd_split(FftFwdArgs a)
-{
-    // [buffer_words(a.M)] quarter-transform buffer | [n] spectrum | chirp of the quarter
-    extern __shared__ float2 sbuf[];
-    chain_allow_next();
-    const int j = a.reps[blockIdx.x];
-    const int n = a.rd.n[j], q = n / 4;
-    float2 *X = sbuf + fft::buffer_words(a.M);
-    float2 *chirp = X + n;
-    ring::chirp_table(chirp, q, -1);
-    const int j2 = a.R - 1 - j;
-    FwdSplitCta c{a, sbuf, X, chirp, a.rd.fb + a.rd.fboff[j], j, j2, n, a.rd.hs[j], j2 != j,
-                  a.zero_poles && j == 0, a.weight ? a.rd.w[j] : 1.0f};
-    c.run<13>();  // split rings have 2048 < q < 4096: quarter buffer 8192 (kMaxSplitM)
-    chain_wait();
-}
 
 template <int LMAX>
 __global__ void __launch_bounds__(ring::ClassShape<LMAX>::kThreads, ring::ClassShape<LMAX>::kMinBlocks)
@@ -372,21 +259,11 @@ cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_fft_fwd_split(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev)
-{
-    if (count <= 0) return cudaSuccess;
-    const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, threads, true);
-    cudaError_t e = set_smem((const void *)k_fft_fwd_split, smem);
-    if (e != cudaSuccess) return e;
-    return launch_chained(k_fft_fwd_split, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), threads, smem, st,
-                          after_prev, 1, a);
-}
-
 template <int LMAX>
 cudaError_t launch_fwd_class(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev)
 {
     constexpr int T = ring::ClassShape<LMAX>::kThreads;
-    const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, T, false);
+    const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, T);
     cudaError_t e = set_smem((const void *)k_fft_fwd<LMAX>, smem);
     if (e != cudaSuccess) return e;
     return launch_chained(k_fft_fwd<LMAX>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), T, smem, st,

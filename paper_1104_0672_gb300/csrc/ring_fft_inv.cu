@@ -140,7 +140,8 @@ struct InvCta {
     float4 *part;
     const float2 *chirp, *phase, *fb;  // chirp of h (Bluestein rings), exp(+i pi m / n) for m <= n/2
     int i, i2, n, h, hs;
-    bool pair, blu, stage;
+    bool pair, stage;
+    bool blu;  // (classes above 2^10 hold power-of-two transforms only)
     float wsc;
 
     // exp(+i pi m / n), 0 <= m <= n/2
@@ -152,6 +153,7 @@ struct InvCta {
     __device__ void run()
     {
         constexpr int M = 1 << L;
+        const bool blu = L <= 10 && this->blu;
         const fft::Smem<L, cpair> sm{buf};
         const float inv_m = 1.0f / (float)M;
         const int bend = min(a.B, (int)(blockIdx.y + 1) * a.mchunk);
@@ -281,7 +283,7 @@ struct InvCta {
                     if (pair) o2[q] = make_float2(z.re.y, z.im.y);
                 }
             };
-            if (blu) {
+            if (L <= 10 && blu) {
                 // Bluestein takes natural order; the inverse chirp is the conjugate of the
                 // forward one, and so is its spectrum (the chirp sequence is even)
                 fill([&](int k, cpair v) { sm(k, v); });
@@ -294,93 +296,6 @@ struct InvCta {
         }
     }
 };
-
-// Rings of n = 4q pixels too long for one Bluestein buffer (the transpose of the forward
-// split), the ring pair packed as one complex sequence: the n folded coefficients X go to
-// shared memory, the radix-4 step
-//   Z_p[k'] = W_n^{-p k'} sum_t W_4^{-p t} X[k' + t q]
-// runs in place, then four q-point inverse DFTs by Bluestein write pixels 4 s + p.
-struct InvSplitCta {
-    const FftInvArgs &a;
-    float2 *buf, *X;
-    const float2 *chirp, *fb;  // chirp exp(+i pi k^2 / q), k <= q/2
-    int i, i2, n, hs;
-    bool pair;
-    float wsc;
-    template <int L>
-    __device__ void run()
-    {
-        const int q = n / 4;
-        const float inv_m = 1.0f / (float)(1 << L);
-        const int bend = min(a.B, (int)(blockIdx.y + 1) * a.mchunk);
-        for (int b = blockIdx.y * a.mchunk; b < bend; ++b) {
-            const float2 *c1 = a.c + ((int64_t)b * a.R + i) * a.NH;
-            const float2 *c2 = a.c + ((int64_t)b * a.R + i2) * a.NH;
-            for (int k = threadIdx.x; k < n; k += blockDim.x) {
-                const bool up = 2 * k > n;
-                const int mm = up ? n - k : k;
-                const float2 ph = hs ? expipi_ratio(mm, n) : make_float2(1.f, 0.f);
-                float2 d1 = folded_coeff(c1, mm, n, hs, ph, a.N, a.basic);
-                float2 d2 = pair ? folded_coeff(c2, mm, n, hs, ph, a.N, a.basic) : make_float2(0.f, 0.f);
-                if (up) {
-                    d1.y = -d1.y;
-                    d2.y = -d2.y;
-                }
-                X[k] = make_float2(wsc * (d1.x - d2.y), wsc * (d1.y + d2.x));
-            }
-            __syncthreads();
-            for (int k = threadIdx.x; k < q; k += blockDim.x) {
-                float2 v0 = X[k], v1 = X[q + k], v2 = X[2 * q + k], v3 = X[3 * q + k];
-                fft::dft4<true>(v0, v1, v2, v3);
-                const float2 w1 = expipi_ratio(2 * k, n), w2 = cmulf(w1, w1), w3 = cmulf(w1, w2);
-                X[k] = v0;
-                X[q + k] = cmulf(v1, w1);
-                X[2 * q + k] = cmulf(v2, w2);
-                X[3 * q + k] = cmulf(v3, w3);
-            }
-            __syncthreads();
-            float *o1 = a.map + (int64_t)b * a.npix + a.rd.poff[i];
-            float *o2 = a.map + (int64_t)b * a.npix + a.rd.poff[i2];
-            for (int p = 0; p < 4; ++p) {
-                const float2 *Z = X + p * q;
-                auto ld = [&](int k) { return k < q ? cmulf(Z[k], chirp_at(chirp, k, q)) : make_float2(0.f, 0.f); };
-                auto st = [&](int s, float2 z) {
-                    if (s < q) {
-                        z = cscalef(cmulf(z, chirp_at(chirp, s, q)), inv_m);
-                        o1[4 * s + p] = z.x;
-                        if (pair) o2[4 * s + p] = z.y;
-                    }
-                };
-                fft::convolve<L, true>(buf, a.tw, fb, ld, st);
-            }
-        }
-    }
-};
-
-__global__ void __launch_bounds__(512) k_fft_inv_split(FftInvArgs a)
-{
-    // [buffer_words(a.M)] quarter-transform buffer | [n] coefficients | chirp of the quarter
-    extern __shared__ float2 sbuf[];
-    if (!a.first) chain_allow_next();
-    const int i = a.reps[blockIdx.x];
-    if (a.skip_poles && i == 0) {
-        chain_wait();
-        return;
-    }
-    const int n = a.rd.n[i], q = n / 4;
-    float2 *X = sbuf + fft::buffer_words(a.M);
-    float2 *chirp = X + n;
-    ring::chirp_table(chirp, q, +1);
-    if (a.first) {
-        chain_wait();
-        chain_allow_next();
-    }
-    const int i2 = a.R - 1 - i;
-    InvSplitCta c{a, sbuf, X, chirp, a.rd.fb + a.rd.fboff[i], i, i2, n, a.rd.hs[i], i2 != i,
-                  a.weight ? a.rd.w[i] : 1.0f};
-    c.run<13>();  // split rings have 2048 < q < 4096: quarter buffer 8192 (kMaxSplitM)
-    chain_wait();
-}
 
 template <int LMAX>
 __global__ void __launch_bounds__(ring::ClassShape<LMAX>::kThreads, ring::ClassShape<LMAX>::kMinBlocks)
@@ -414,40 +329,28 @@ k_fft_inv(FftInvArgs a)
     }
     const int i2 = a.R - 1 - i;
     InvCta c{a, buf, D1, D2, part, chirp, phase, blu ? a.rd.fb + a.rd.fboff[i] : nullptr,
-             i, i2, n, h, hs, i2 != i, blu, stage, a.weight ? a.rd.w[i] : 1.0f};
+             i, i2, n, h, hs, i2 != i, stage, blu, a.weight ? a.rd.w[i] : 1.0f};
     ring::dispatch_upto<LMAX>(logM, c);
     chain_wait();
 }
 
 }  // namespace
 
-// Shared memory of a ring FFT class: the transform buffer (pairs of complex values, or single
-// ones for the split path), the short-ring fold's bins and partial sums, and the per-ring
-// tables.
-size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads, bool split)
+// Shared memory of a ring FFT class: the transform buffer, the short-ring fold's bins and partial
+// sums, and the per-ring tables.
+size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads)
 {
-    size_t bytes = (size_t)fft::buffer_words(M) * (split ? sizeof(float2) : sizeof(cpair));
+    size_t bytes = (size_t)fft::buffer_words(M) * sizeof(cpair);
     size_t words = (size_t)tab;
     if (stage_c) words += 2 * (size_t)(N / 8 + 1) + 4 * (size_t)threads;
     return bytes + words * sizeof(float2);
-}
-
-cudaError_t launch_fft_inv_split(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev)
-{
-    if (count <= 0) return cudaSuccess;
-    const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, threads, true);
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_fft_inv_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_chained(k_fft_inv_split, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), threads, smem, st,
-                          after_prev, 1, a);
 }
 
 template <int LMAX>
 cudaError_t launch_inv_class(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev)
 {
     constexpr int T = ring::ClassShape<LMAX>::kThreads;
-    const size_t smem = fft_smem_bytes(a.M, a.N, a.stage_c != 0, a.tab, T, false);
+    const size_t smem = fft_smem_bytes(a.M, a.N, a.stage_c != 0, a.tab, T);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_fft_inv<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
