@@ -124,7 +124,9 @@ struct Kernel {
     int max_win_rows = 0;      // rows of a 32-slot window over a block of 16 in groups of four
     int polar_pairs = 0;       // leading pairs whose coefficients are tabulated per call
     int knot_fft_pairs = 0;    // leading pairs whose knot-gradient projection runs by FFT
-    bool proj_tc_ok = false;   // the other pairs have at most 128 samples (tensor-core projection)
+    bool proj_tc_ok = false;   // the other pairs have at most 128 samples (projection by table)
+    int proj_cut[5] = {};      // their blocks of 128 pairs by samples (KnotGradArgs::cut)
+    int proj_taps = 0;         // most samples of one of them
     int64_t sum_taps_fix = 0;  // in-support tap count with the shift fix (for reporting)
     void *dmem = nullptr;      // one device allocation holding every table
     KernDev kd{};
@@ -213,15 +215,26 @@ struct PoleArgs {
     double wsum[kMaxKernelsPerLaunch];  // wsum[k] x the direct sum of kd[k] over input map b
 };
 
+// Knot gradients of up to kMaxKernelsPerLaunch kernels (blockIdx.z or .y of the launches): kernel
+// b of the batch has its own Q rows, projections and partial sums.
 struct KnotGradArgs {
     RingDev rd;
-    KernDev kd;
+    KernDev kd[kMaxKernelsPerLaunch];
+    int fft_pairs[kMaxKernelsPerLaunch];  // leading pairs projected by FFT
+    int cut[kMaxKernelsPerLaunch][5];     // tensor-core projection: first block of 128 pairs (past those) of
+                                          // at most 128, 64, 32 and 16 samples, and their number
     const float4 *spec4;  // weighted extended spectra of the input maps [B][nrep][NH]
     const float4 *gspec4; // extended spectra of the output gradients [B][nrep][NH]
     const double *s2;
     const float2 *tw;    // stage twiddles of the grid (FFT projection of the polar pairs)
-    double *partial;     // [rows][T] per-CTA partial sums
-    int R, N, NH, nrep, B, map0, nmaps;
+    float *Q, *X;        // [pairs][NH] and [pairs past the FFT ones][128] per kernel
+    double *partial;     // [rows][T] partial sums per kernel: deposit CTAs, FFT pairs, pole rings
+    int64_t qstride, xstride, pstride;  // elements from a kernel to the next
+    int nk;              // kernels of the launch
+    int row_fft, row_pole;              // first rows of the FFT pairs and the pole rings
+    int pole_split[kMaxKernelsPerLaunch];  // CTAs sharing a pole pixel's sum
+    int R, N, NH, nrep, B, map0, nmaps; // kernel b sums maps [map0 + b * per_map, + nmaps)
+    int per_map;
     int64_t nspec;
     int basic, shift_fix;
     int pole_fix;        // pole rings' hybrid outputs are replaced (skip their g)
@@ -244,7 +257,7 @@ __device__ __forceinline__ float4 paired_coeff(const float4 *__restrict__ sp4, i
 // after_prev: may begin while the kernel before it on the stream still runs.
 cudaError_t launch_taps(const TapArgs &a, int nk, int64_t maxtaps, cudaStream_t st, bool after_prev);
 cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs, const float2 *tw, int twM,
-                             cudaStream_t st);
+                             const float2 *cos2n, cudaStream_t st);
 size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads);  // shared memory of a ring FFT class
 cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int threads, cudaStream_t st);
 // Ring FFT class launches.  after_prev: the previous kernel on the stream is the previous class
@@ -292,19 +305,24 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t 
 // band_pixels: pixels of the rings inside the support of a pole
 cudaError_t launch_pole_fwd(const PoleArgs &a, int64_t band_pixels, cudaStream_t st, bool after_prev);
 cudaError_t launch_pole_adj(const PoleArgs &a, int max_band_rings, cudaStream_t st);
-cudaError_t launch_knot_grad_q(const KnotGradArgs &a, float *Q, int max_band, int max_union, int max_union2,
-                               int srows, cudaStream_t st);
-cudaError_t launch_knot_grad_proj(const KnotGradArgs &a, const float *Q, const float *X, int pfirst,
+cudaError_t launch_knot_grad_q(const KnotGradArgs &a, int max_band, int max_union, int max_union2, int srows,
+                               cudaStream_t st);
+// The cosine sums of the pairs past the FFT ones into X (all of at most 128 samples): tensor cores
+// or plain FP32
+cudaError_t launch_knot_proj_tc(const KnotGradArgs &a, const float *ctabP, int nmc, int maxblocks, cudaStream_t st);
+cudaError_t launch_knot_proj_f32(const KnotGradArgs &a, const float *ctabP, int nmc, int maxpairs, int maxtaps,
+                                 cudaStream_t st);
+// Deposits of those pairs (have_x), or projection and deposits where a pair has more samples
+cudaError_t launch_knot_grad_proj(const KnotGradArgs &a, bool have_x, int T, cudaStream_t st);
+cudaError_t launch_knot_grad_proj_fft(const KnotGradArgs &a, int maxpairs, int T, cudaStream_t st);
+cudaError_t launch_knot_grad_pole(const KnotGradArgs &a, const float *map, const float *gout, int64_t npix, int T,
                                   cudaStream_t st);
-cudaError_t launch_knot_proj_tc(const KnotGradArgs &a, const float *Q, const float *ctabP, int nmc, int pfirst,
-                                float *X, cudaStream_t st);
-cudaError_t launch_knot_grad_proj_fft(const KnotGradArgs &a, const float *Q, int npairs, int row0, cudaStream_t st);
-cudaError_t launch_knot_grad_pole(const KnotGradArgs &a, const float *map, const float *gout,
-                                  int64_t npix, int row0, cudaStream_t st);
 int knot_proj_blocks();
 int knot_proj_taps();
-cudaError_t launch_knot_reduce(const double *partial, int nrows, int T, double *out,
-                               cudaStream_t st);
+int knot_pole_split(int64_t band_pixels);  // CTAs sharing a pole pixel's sum
+cudaError_t launch_knot_reduce(const KnotGradArgs &a, double *out, int T, cudaStream_t st);
+// Which of the Q kernels serves bands like these (kernels of one launch agree on it)
+int knot_q_form(int max_band, int max_union, int max_union2, int srows);
 void set_last_error(const char *msg);  // sets the message arkcos_last_error() returns
 int contract_band_limit();
 // tensor-core contraction over blocks of rb (8 or 16) representative rings, a thread taking

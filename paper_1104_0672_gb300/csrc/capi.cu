@@ -377,9 +377,14 @@ struct StageScope {
     }
 };
 
+constexpr size_t kKnotBatchBytes = 256u << 20;
+
 struct Layout {
     size_t taps_off[kMaxKernelsPerLaunch * 8];
     size_t spec = 0, gspec = 0, cbuf = 0, q = 0, xproj = 0, partial = 0, total = 0;
+    // knot gradients: elements per kernel of a batch of kbatch, first rows of partial sums
+    int64_t qstride = 0, xstride = 0, pstride = 0, kbatch = 1;
+    int row_fft = 0, row_pole = 0;
     size_t prho = 0, prho_stride = 0;  // tabulated polar coefficients, per kernel
 };
 
@@ -414,14 +419,26 @@ bool layout_for(const Grid &g, const arkcos_kernel *ks, int64_t nk, int64_t nmap
             maxT = std::max(maxT, ks[k]->k.T);
         }
         L.q = off;
-        off = align256(off + (size_t)maxpairs * (g.N / 2 + 1) * sizeof(float));
+        // per-map kernels go in batches whose rows of Q stay within kKnotBatchBytes (at least one)
+        L.qstride = (int64_t)maxpairs * (g.N / 2 + 1);
+        L.xstride = (int64_t)maxpairs * 128;
+        L.kbatch = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(nk, kMaxKernelsPerLaunch),
+                                                          (int64_t)(kKnotBatchBytes / (L.qstride * sizeof(float)))));
+        off = align256(off + (size_t)L.kbatch * L.qstride * sizeof(float));
         L.xproj = off;
-        off = align256(off + (size_t)maxpairs * 128 * sizeof(float));
+        off = align256(off + (size_t)L.kbatch * L.xstride * sizeof(float));
         int maxfft = 0;
-        for (int64_t k = 0; k < nk; ++k) maxfft = std::max(maxfft, ks[k]->k.knot_fft_pairs);
+        int64_t pole_pixels = 0;
+        for (int64_t k = 0; k < nk; ++k) {
+            maxfft = std::max(maxfft, ks[k]->k.knot_fft_pairs);
+            pole_pixels = std::max(pole_pixels, ks[k]->k.pole_pixels);
+        }
         L.partial = off;
-        const int64_t rows = knot_proj_blocks() + 8 * nmaps + maxfft;
-        off = align256(off + (size_t)rows * maxT * sizeof(double));
+        L.row_fft = knot_proj_blocks();
+        L.row_pole = L.row_fft + (maxfft + 1) / 2;
+        const int64_t rows = L.row_pole + 8 * (nk > 1 ? 1 : nmaps) * knot_pole_split(pole_pixels);
+        L.pstride = rows * maxT;
+        off = align256(off + (size_t)L.kbatch * L.pstride * sizeof(double));
     }
     L.total = off;
     return true;
@@ -728,7 +745,7 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
             a.nrep = g.nrep;
             a.shift_fix = shift_fix;
             if (maxpolar > 0) {
-                CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, st));
+                CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, g.d_cos2n, st));
                 ++sc.launches;
             }
         }
@@ -777,7 +794,7 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
             a.map_base = 0;
         }
         if (polar_table && kdiv == 0 && maxpolar > 0) {
-            CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, st));
+            CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, g.d_cos2n, st));
             ++sc.launches;
         }
         if (narrow) CK(launch_contract_tc(a, tc_rb, tc_gs, !tf32, nchunks, tb, tc_srows, tc_want, st));
@@ -1136,6 +1153,19 @@ arkcos_status arkcos_set_kernel(arkcos_grid grid, const double *knots, int64_t n
         int mx = 0;
         for (int p = K.knot_fft_pairs; p < K.npairs; ++p) mx = std::max(mx, std::max(S0[p], S1[p]) + 1);
         K.proj_tc_ok = mx <= 128;
+        K.proj_taps = mx;
+        // blocks of 128 pairs, from the first whose own and later pairs all have at most 64, 32 and 16
+        // samples
+        const int nb = (K.npairs - K.knot_fft_pairs + 127) / 128;
+        for (int c = 1; c < 5; ++c) K.proj_cut[c] = nb;
+        int later = 0;
+        for (int b = nb - 1; b >= 0; --b) {
+            for (int p = K.knot_fft_pairs + 128 * b; p < std::min(K.npairs, K.knot_fft_pairs + 128 * (b + 1)); ++p)
+                later = std::max(later, std::max(S0[p], S1[p]) + 1);
+            if (later <= 64) K.proj_cut[1] = b;
+            if (later <= 32) K.proj_cut[2] = b;
+            if (later <= 16) K.proj_cut[3] = b;
+        }
         for (int p = K.polar_pairs; p < K.npairs; ++p)
             K.max_free_taps = std::max(K.max_free_taps, std::max(S0[p], S1[p]) + 1);
     }
@@ -1685,62 +1715,89 @@ arkcos_status arkcos_convolve_backward(arkcos_grid grid, const arkcos_kernel *ke
     if (grad_knots) {
         if ((st = run_fft_fwd(g, map_in, nullptr, aspec, nmaps, true, false, basic, s)) != ARKCOS_OK)
             return st;
-        float *Q = (float *)(ws + L.q);
-        double *partial = (double *)(ws + L.partial);
-        for (int64_t k = 0; k < nkernels; ++k) {
-            const int64_t map0 = per_map ? k : 0;
+        // batches of kernels that go through the same launches as alone (bit for bit the same result)
+        auto like = [](const Kernel &K) {
+            return std::make_tuple(K.T, K.proj_tc_ok, knot_q_form(K.maxband, K.max_union8, K.max_union2, K.max_stage_rows));
+        };
+        for (int64_t k0 = 0; k0 < nkernels;) {
+            const int T = kernels[k0]->k.T;
+            int64_t cnt = 1;
+            while (cnt < L.kbatch && k0 + cnt < nkernels && like(kernels[k0 + cnt]->k) == like(kernels[k0]->k)) ++cnt;
             const int64_t nm = per_map ? 1 : nmaps;
             KnotGradArgs a;
             memset(&a, 0, sizeof(a));
             a.rd = g.dev();
-            a.kd = kernels[k]->k.kd;
             a.spec4 = aspec;
             a.gspec4 = gspec;
             a.s2 = g.d_s2;
             a.tw = g.d_tw;
-            a.partial = partial;
+            a.Q = (float *)(ws + L.q);
+            a.X = (float *)(ws + L.xproj);
+            a.partial = (double *)(ws + L.partial);
+            a.qstride = L.qstride;
+            a.xstride = L.xstride;
+            a.pstride = L.pstride;
+            a.nk = (int)cnt;
+            a.row_fft = L.row_fft;
+            a.row_pole = L.row_pole;
             a.R = g.R;
             a.N = g.N;
             a.NH = g.N / 2 + 1;
             a.nrep = g.nrep;
             a.B = (int)nmaps;
-            a.map0 = (int)map0;
+            a.map0 = (int)(per_map ? k0 : 0);
+            a.per_map = per_map;
             a.nmaps = (int)nm;
             a.nspec = g.nspec;
             a.basic = basic;
             a.shift_fix = shift_fix;
             a.pole_fix = pole_fix;
             a.withhold_mma = test_withhold_mma();
-            const Kernel &K = kernels[k]->k;
+            int maxband = 0, union8 = 0, union2 = 0, srows = 0, maxfft = 0, maxrest = 0, maxblocks = 0, maxtaps = 0;
+            bool table = true;  // every pair past the FFT ones has at most 128 samples
+            for (int64_t k = 0; k < cnt; ++k) {
+                const Kernel &K = kernels[k0 + k]->k;
+                a.kd[k] = K.kd;
+                a.fft_pairs[k] = K.knot_fft_pairs;
+                a.pole_split[k] = knot_pole_split(K.pole_pixels);
+                memcpy(a.cut[k], K.proj_cut, sizeof(K.proj_cut));
+                maxband = std::max(maxband, K.maxband);
+                union8 = std::max(union8, K.max_union8);
+                union2 = std::max(union2, K.max_union2);
+                srows = std::max(srows, K.max_stage_rows);
+                maxfft = std::max(maxfft, K.knot_fft_pairs);
+                maxrest = std::max(maxrest, K.npairs - K.knot_fft_pairs);
+                maxblocks = std::max(maxblocks, K.proj_cut[4]);
+                maxtaps = std::max(maxtaps, K.proj_taps);
+                table = table && K.proj_tc_ok;
+            }
             {
                 StageScope sc(ST_KNOT_Q, 1, s);
-                CK(launch_knot_grad_q(a, Q, K.maxband, K.max_union8, K.max_union2, K.max_stage_rows, s));
+                CK(launch_knot_grad_q(a, maxband, union8, union2, srows, s));
             }
             {
-                // 3xTF32 form: the cosine sums of the pairs past the FFT-projected ones as one
-                // tensor-core product, then the deposits; otherwise both on the CUDA cores
+                // the cosine sums of the pairs past the FFT-projected ones as one product against the
+                // cosine table (3xTF32 form: tensor cores), then the deposits; pairs of more samples
+                // than the table by phasors
                 StageScope sc(ST_KNOT_PROJ, 1, s);
-                const bool tc = (flags & ARKCOS_FLAG_3XTF32) && K.proj_tc_ok;
-                float *X = (float *)(ws + L.xproj);
-                if (tc) {
-                    CK(launch_knot_proj_tc(a, Q, g.d_ctabP, g.nmc_p, K.knot_fft_pairs, X, s));
+                if (table) {
+                    if (flags & ARKCOS_FLAG_3XTF32) CK(launch_knot_proj_tc(a, g.d_ctabP, g.nmc_p, maxblocks, s));
+                    else CK(launch_knot_proj_f32(a, g.d_ctabP, g.nmc_p, maxrest, maxtaps, s));
                     ++sc.launches;
                 }
-                CK(launch_knot_grad_proj(a, Q, tc ? X : nullptr, K.knot_fft_pairs, s));
-            }
-            int rows = knot_proj_blocks();
-            if (kernels[k]->k.knot_fft_pairs > 0) {
-                StageScope sc(ST_KNOT_PROJ, 1, s);
-                CK(launch_knot_grad_proj_fft(a, Q, kernels[k]->k.knot_fft_pairs, rows, s));
-                rows += kernels[k]->k.knot_fft_pairs;
+                CK(launch_knot_grad_proj(a, table, T, s));
+                if (maxfft > 0) {
+                    CK(launch_knot_grad_proj_fft(a, maxfft, T, s));
+                    ++sc.launches;
+                }
             }
             if (pole_fix) {
                 StageScope sc(ST_KNOT_POLE, 1, s);
-                CK(launch_knot_grad_pole(a, map_in, grad_out, g.npix, rows, s));
-                rows += 8 * (int)nm;
+                CK(launch_knot_grad_pole(a, map_in, grad_out, g.npix, T, s));
             }
             StageScope sc(ST_KNOT_REDUCE, 1, s);
-            CK(launch_knot_reduce(partial, rows, kernels[k]->k.T, grad_knots + k * kernels[k]->k.T, s));
+            CK(launch_knot_reduce(a, grad_knots + k0 * T, T, s));
+            k0 += cnt;
         }
     }
     return ARKCOS_OK;

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(1024) k_polar_rho_fft(ContractArgs a, const fl
 }
 
 // The same coefficients one thread per (pair, mode), for kernel grids without the FFT form.
-__global__ void __launch_bounds__(256) k_polar_rho(ContractArgs a)
+__global__ void __launch_bounds__(256) k_polar_rho(const __grid_constant__ ContractArgs a, const float2 *__restrict__ cos2n)
 {
     chain_allow_next();
     chain_wait();
@@ -214,13 +214,13 @@ __global__ void __launch_bounds__(256) k_polar_rho(ContractArgs a)
     const int f = a.shift_fix ? kd.fl[p] : 0;
     const int S = f ? kd.S1[p] : kd.S0[p];
     const float4 *tp4 = reinterpret_cast<const float4 *>(a.taps[kid] + kd.toff[p]);
-    const_cast<float *>(a.prho[kid])[(int64_t)p * a.NH + m] = gen_rho(tp4, S, f, m, a.N);
+    const_cast<float *>(a.prho[kid])[(int64_t)p * a.NH + m] = gen_rho(tp4, S, f, m, a.N, cos2n);
 }
 
 }  // namespace
 
 cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs, const float2 *tw, int twM,
-                             cudaStream_t st)
+                             const float2 *cos2n, cudaStream_t st)
 {
     if (max_polar_pairs <= 0 || nk <= 0) return cudaSuccess;
     int logN = 0;
@@ -234,7 +234,7 @@ cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs,
         return launch_chained(k_polar_rho_fft, grid, a.N / 16, smem, st, true, 1, a, tw, logN);
     }
     dim3 grid((a.NH + 255) / 256, max_polar_pairs, nk);
-    return launch_chained(k_polar_rho, grid, 256, 0, st, true, 1, a);
+    return launch_chained(k_polar_rho, grid, 256, 0, st, true, 1, a, cos2n);
 }
 
 cudaError_t launch_taps(const TapArgs &a, int nk, int64_t maxtaps, cudaStream_t st, bool after_prev)

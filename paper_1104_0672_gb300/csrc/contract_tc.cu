@@ -652,33 +652,56 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
 // Knot-gradient projection on the tensor cores (the 3xTF32 form of the backward pass):
 //     X[p][k] = sum_m Q_m(p) cos(pi m (2k + f) / N),   k < 128, f = 0 and 1,
 // a dense product of the Q rows of 128 ring pairs (A, M = 128, split hi/lo on the fly) and a
-// per-grid table of the cosines of 128 taps of each flavour (B, N = 256, K = 32 modes per
-// chunk, hi/lo in the core layout).  The sum over the modes is long (N/2 + 1 terms) and the
+// per-grid table of the cosines of NT taps of each flavour (B, N = 2 NT, K = 32 modes per
+// chunk, hi/lo in the core layout), NT = 16, 32, 64 or 128 >= the most samples of a block's pairs
+// (most blocks hold pairs of at most 16: one nside-2048 kernel 0.42 ms, the other classes beside
+// it, bound by the loads of the Q rows; 1.14 ms with 128 for all, bound by the table copies and
+// products).  The sum over the modes is long (N/2 + 1 terms) and the
 // cosines make it cancel, so it is not left to the tensor core's accumulator, whose additions
-// do not round to nearest: every chunk's twelve MMAs start from zero in one of two 256-column
-// accumulators, and once a chunk is complete its 128 x 256 partial sums are added in FP32
+// do not round to nearest: every chunk's twelve MMAs start from zero in one of two 2 NT-column
+// accumulators, and once a chunk is complete its 128 x 2 NT partial sums are added in FP32
 // (round to nearest) into registers of the epilogue threads while the next chunk's MMAs fill
 // the other accumulator.  Two stages of shared memory: chunk c + 1 is staged while the MMAs of
 // chunk c run, each stage (and its accumulator) released by its own completion barrier
-// (bounded waits).  Each pair's row of its own flavour's 128 values goes to X; the hat-weight
-// deposits follow in k_knot_proj.
+// (bounded waits).  Each pair's row of its own flavour's NT values goes to X; the hat-weight
+// deposits follow in k_knot_deposit.
 constexpr int kPjPairs = 128, kPjThreads = 256;
-constexpr uint32_t kPjA = 16384, kPjB = 32768, kPjStage = 2 * kPjA + 2 * kPjB;  // 96 KiB per stage
-constexpr uint32_t kPjCols = 256;                                              // per accumulator
+constexpr uint32_t kPjA = 16384;
+template <int NT>
+struct PjShape {
+    static constexpr uint32_t kB = 2 * NT * 128, kStage = 2 * kPjA + 2 * kB;  // 40 to 96 KiB per stage
+    static constexpr uint32_t kCols = 2 * NT;                                 // per accumulator
+    static constexpr uint32_t kAlloc = 2 * kCols < 32 ? 32 : 2 * kCols;
+};
 
-__global__ void __launch_bounds__(kPjThreads, 1)
-k_knot_proj_tc(KnotGradArgs a, const float *__restrict__ Q, const float *__restrict__ ctabP, int nmc, int pfirst,
-               float *X)
+// cls: the class of blocks (KnotGradArgs::cut); first: the launch that follows the Q rows (the
+// other classes start beside it and only end after it)
+template <int NT>
+__global__ void __launch_bounds__(kPjThreads, NT <= 32 ? 2 : 1)
+k_knot_proj_tc(const __grid_constant__ KnotGradArgs a, const float *__restrict__ ctabP, int nmc, int cls, int first)
 {
+    using Sh = PjShape<NT>;
+    constexpr uint32_t kPjStage = Sh::kStage, kPjB = Sh::kB, kPjCols = Sh::kCols;
+    const int kb = blockIdx.y, blk = a.cut[kb][cls] + blockIdx.x;
+    if (first) chain_wait();
+    chain_allow_next();
+    if (blk >= a.cut[kb][cls + 1]) {
+        chain_wait();
+        return;
+    }
+    const KernDev &kd = a.kd[kb];
+    const float *Q = a.Q + kb * a.qstride;
+    const int pfirst = a.fft_pairs[kb];
+    float *X = a.X + kb * a.xstride;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + 2 * kPjStage);  // [2] stage barriers
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + 2 * kPjStage + 16);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int pbase = pfirst + blockIdx.x * kPjPairs;
-    const int npairs = a.kd.npairs;
+    const int pbase = pfirst + blk * kPjPairs;
+    const int npairs = kd.npairs;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"((uint32_t)__cvta_generic_to_shared(tslot)), "r"(2 * kPjCols));
+                     ::"r"((uint32_t)__cvta_generic_to_shared(tslot)), "r"(Sh::kAlloc));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
@@ -696,20 +719,20 @@ k_knot_proj_tc(KnotGradArgs a, const float *__restrict__ Q, const float *__restr
     ok = __syncthreads_and(ok);
     uint32_t ph = 0;    // bit s: parity of the next completion of stage s
     uint32_t pend = 0;  // bit s: stage s has an issued commit not yet seen complete
-    const uint32_t idesc = tf32_idesc(kTcModes, 2 * kTcModes);
+    const uint32_t idesc = tf32_idesc(kTcModes, 2 * NT);
     // epilogue role of the thread: warp (lane quarter, column half), lane = pair, columns =
-    // the half's 128 taps; it sums every chunk's partials of those columns in registers
+    // the half's NT taps; it sums every chunk's partials of those columns in registers
     const int er = (warp & 3) * 32 + lane, ehalf = warp >> 2;
-    float acc[128];
+    float acc[NT];
 #pragma unroll
-    for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+    for (int j = 0; j < NT; ++j) acc[j] = 0.f;
     // adds the completed partial sums of accumulator `buf` (after its completion wait)
     auto drain = [&](int buf) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)buf * kPjCols +
-                              (uint32_t)(ehalf * 128);
+                              (uint32_t)(ehalf * NT);
 #pragma unroll
-        for (int h = 0; h < 128; h += 16) {
+        for (int h = 0; h < NT; h += 16) {
             uint32_t v[16];
             tmem_ld_async(base + (uint32_t)h, v);
             tmem_wait_ld();
@@ -747,9 +770,12 @@ k_knot_proj_tc(KnotGradArgs a, const float *__restrict__ Q, const float *__restr
             ph ^= 1u << st;
             if (ok) drain(st);
         }
-        // B: the chunk's cosine tile (hi then lo, 64 KiB)
+        // B: the first NT rows of each flavour of the chunk's cosine tile (hi then lo)
         const float *src = ctabP + (size_t)c * 2 * 8192;
-        for (int e = tid; e < 4096; e += kPjThreads) cp_async16(Bhi + 16 * e, src + 4 * e, 16);
+        for (int e = tid; e < 4 * NT * 8; e += kPjThreads) {
+            const int unit = e % (NT * 8), f = e / (NT * 8) & 1, part = e / (NT * 16);
+            cp_async16(Bhi + part * kPjB + f * NT * 128 + unit * 16, src + part * 8192 + f * 4096 + unit * 4, 16);
+        }
         cp_async_commit();
         // A: the Q rows of the block's pairs at the chunk's 32 modes, split hi / lo
 #pragma unroll
@@ -815,11 +841,11 @@ k_knot_proj_tc(KnotGradArgs a, const float *__restrict__ Q, const float *__restr
     {
         const int p = pbase + er;
         const bool pv = ok && p < npairs;
-        const int f = pv && a.shift_fix ? a.kd.fl[p] : 0;
+        const int f = pv && a.shift_fix ? kd.fl[p] : 0;
         if (pv && f == ehalf) {
             float *xr = X + (int64_t)(p - pfirst) * 128;
 #pragma unroll
-            for (int j = 0; j < 128; j += 4)
+            for (int j = 0; j < NT; j += 4)
                 *reinterpret_cast<float4 *>(xr + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
         }
     }
@@ -827,7 +853,8 @@ k_knot_proj_tc(KnotGradArgs a, const float *__restrict__ Q, const float *__restr
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kPjCols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Sh::kAlloc));
+    chain_wait();
 }
 
 }  // namespace
@@ -912,19 +939,42 @@ cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks
                : launch_tc<16, 4, true, false>(a, nchunks, tb, srows, nbuf, st);
 }
 
-// Knot-gradient projection of pairs [pfirst, npairs) into X [npairs - pfirst][128] (rows of
-// 128 taps of each pair's own flavour); ctabP holds nmc chunks of 32 modes.
-cudaError_t launch_knot_proj_tc(const KnotGradArgs &a, const float *Q, const float *ctabP, int nmc, int pfirst,
-                                float *X, cudaStream_t st)
+namespace {
+
+template <int NT>
+cudaError_t launch_pj(const KnotGradArgs &a, const float *ctabP, int nmc, int cls, bool first, cudaStream_t st)
 {
-    const int n = a.kd.npairs - pfirst;
-    if (n <= 0) return cudaSuccess;
-    const size_t smem = 2 * (size_t)kPjStage + 32;
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_proj_tc,
+    int blocks = 0;
+    for (int k = 0; k < a.nk; ++k) blocks = std::max(blocks, a.cut[k][cls + 1] - a.cut[k][cls]);
+    if (blocks <= 0) return cudaSuccess;
+    const size_t smem = 2 * (size_t)PjShape<NT>::kStage + 32;
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_proj_tc<NT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_knot_proj_tc<<<(n + kPjPairs - 1) / kPjPairs, kPjThreads, smem, st>>>(a, Q, ctabP, nmc, pfirst, X);
-    return cudaGetLastError();
+    return launch_chained(k_knot_proj_tc<NT>, dim3(blocks, a.nk), kPjThreads, smem, st, true, 1, a, ctabP, nmc, cls,
+                          (int)first);
+}
+
+}  // namespace
+
+// Knot-gradient projection of the pairs past the FFT ones into X (rows of 128 taps of each pair's
+// own flavour); ctabP holds nmc chunks of 32 modes.
+cudaError_t launch_knot_proj_tc(const KnotGradArgs &a, const float *ctabP, int nmc, int maxblocks, cudaStream_t st)
+{
+    if (maxblocks <= 0) return cudaSuccess;
+    bool first = true;
+    for (int cls = 3; cls >= 0; --cls) {
+        int blocks = 0;
+        for (int k = 0; k < a.nk; ++k) blocks = std::max(blocks, a.cut[k][cls + 1] - a.cut[k][cls]);
+        if (blocks <= 0) continue;
+        const cudaError_t e = cls == 3   ? launch_pj<16>(a, ctabP, nmc, cls, first, st)
+                              : cls == 2 ? launch_pj<32>(a, ctabP, nmc, cls, first, st)
+                              : cls == 1 ? launch_pj<64>(a, ctabP, nmc, cls, first, st)
+                                         : launch_pj<128>(a, ctabP, nmc, cls, first, st);
+        if (e != cudaSuccess) return e;
+        first = false;
+    }
+    return cudaSuccess;
 }
 
 // Host-side reset/readout of the device error word (bounded waits that expired).

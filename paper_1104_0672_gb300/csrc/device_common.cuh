@@ -72,7 +72,8 @@ __device__ __forceinline__ double profile_eval(double u, const double *ut, const
 // Reinsch's recurrence: for cos(2 alpha) >= 0 the difference D_k = C_k - C_{k-1} obeys
 // D_{k+1} = D_k - lam C_k (lam = 4 sin^2 alpha); otherwise the sum E_k = C_k + C_{k-1}
 // obeys E_{k+1} = mu C_k - E_k (mu = 4 cos^2 alpha).  Rounding error grows linearly in k;
-// the state is re-seeded from exact values every 64 taps.
+// the state is re-seeded every 64 taps from exact values: cos2n[t] = cos(pi t / N) (hi, lo), t < 2N,
+// N even, whose entry t - N/2 is the sine.
 #define REC_STEP()                 \
     do {                           \
         if (low) {                 \
@@ -84,7 +85,8 @@ __device__ __forceinline__ double profile_eval(double u, const double *ut, const
         }                          \
     } while (0)
 
-__device__ __forceinline__ float gen_rho(const float4 *__restrict__ tp4, int S, int f, int m, int N)
+__device__ __forceinline__ float gen_rho(const float4 *__restrict__ tp4, int S, int f, int m, int N,
+                                         const float2 *__restrict__ cos2n)
 {
     if (S < 0) return 0.f;
     float sa, ca;
@@ -103,11 +105,10 @@ __device__ __forceinline__ float gen_rho(const float4 *__restrict__ tp4, int S, 
             if ((q & 15) == 0) {
                 // exact C_k at k = 4q and its recurrence partner (angles (2k+f) alpha and
                 // (2k-1+f) alpha, reduced exactly modulo 2N)
-                const int k = 4 * q;
-                const float2 e1 = expipi_ratio((2 * k + f) * m, N);
-                const float2 e2 = expipi_ratio((2 * k - 1 + f) * m, N);
-                C = e1.x;
-                G = low ? -2.f * e2.y * sa : 2.f * e2.x * ca;
+                const int k = 4 * q, t1 = (2 * k + f) * m % (2 * N), t2 = (2 * k - 1 + f) * m % (2 * N);
+                const float2 c1 = __ldg(&cos2n[t1]), c2 = __ldg(&cos2n[low ? (t2 < N / 2 ? t2 + 3 * (N / 2) : t2 - N / 2) : t2]);
+                C = c1.x + c1.y;
+                G = low ? -2.f * (c2.x + c2.y) * sa : 2.f * (c2.x + c2.y) * ca;
             } else {
                 REC_STEP();
             }

@@ -7,8 +7,11 @@
 // gradients, so dJ/dK_k(i,j) = c_k sum_m cos(m x_k) Q_m(i,j), and K_k depends on the knots
 // through the hat weights of the linear-in-u lookup.  N-S mirror pairs share their taps and
 // contribute Q(i,j) + Q(R-1-i, R-1-j).  The pole rings add the derivative of their true-
-// profile direct sum.  All reductions over pairs and pixels are staged per CTA and summed in
-// a fixed order, so the result is bitwise reproducible.
+// profile direct sum.  Every warp adds its deposits in a fixed order into bins of its own, a CTA's
+// bins are summed in order, and the CTAs' rows too, so the result is bitwise reproducible.  Each
+// launch serves several kernels.
+#include <algorithm>
+
 #include "fft_engine.cuh"
 
 namespace arkcos {
@@ -20,14 +23,18 @@ constexpr int kQRing = 8;  // representative rings per Q CTA
 
 // Q[p][m] for all pairs p of a block of representative rings and 128 modes (grid x: mode
 // blocks, y: ring blocks).  Q is written to global memory, pairs-major.
-__global__ void __launch_bounds__(kModeBlock) k_knot_q(KnotGradArgs a, float *Q)
+__global__ void __launch_bounds__(kModeBlock) k_knot_q(const __grid_constant__ KnotGradArgs a)
 {
+    chain_allow_next();
+    chain_wait();
+    const int kb = blockIdx.z;
+    float *Q = a.Q + kb * a.qstride;
     const int tid = threadIdx.x;
     const int m = blockIdx.x * kModeBlock + tid;
     if (m >= a.NH) return;
     const int r0 = blockIdx.y * kQRing;
     const int nr = min(kQRing, a.nrep - r0);
-    const KernDev &kd = a.kd;
+    const KernDev &kd = a.kd[kb];
     const float eta = (m == 0 || 2 * m == a.N) ? 1.f : 2.f;
     for (int li = 0; li < nr; ++li) {
         const int i = r0 + li;
@@ -38,9 +45,10 @@ __global__ void __launch_bounds__(kModeBlock) k_knot_q(KnotGradArgs a, float *Q)
             const int j = jl + (p - p0);
             float q = 0.f;
             if (!pole) {
+                const int map0 = a.map0 + kb * a.per_map;
                 for (int b = 0; b < a.nmaps; ++b) {
-                    const float4 *sa = a.spec4 + (int64_t)(a.map0 + b) * a.nrep * a.NH;
-                    const float4 *sg = a.gspec4 + (int64_t)(a.map0 + b) * a.nrep * a.NH;
+                    const float4 *sa = a.spec4 + (int64_t)(map0 + b) * a.nrep * a.NH;
+                    const float4 *sg = a.gspec4 + (int64_t)(map0 + b) * a.nrep * a.NH;
                     const float4 x = paired_coeff(sa, j, a.R, a.NH, m);   // a(j), a(R-1-j)
                     const float4 y = paired_coeff(sg, i, a.R, a.NH, m);   // g(i), g(R-1-i)
                     q = fmaf(x.x, y.x, fmaf(x.y, y.y, q));
@@ -57,8 +65,12 @@ __global__ void __launch_bounds__(kModeBlock) k_knot_q(KnotGradArgs a, float *Q)
 // shared memory (double-buffered cp.async), and one accumulator per ring pair of the band.
 constexpr int kQBand = 32, kQModes = 64, kQRings = 8;
 
-__global__ void __launch_bounds__(kQModes *kQRings, 2) k_knot_q_band(KnotGradArgs a, float *Q)
+__global__ void __launch_bounds__(kQModes *kQRings, 2) k_knot_q_band(const __grid_constant__ KnotGradArgs a)
 {
+    chain_allow_next();
+    chain_wait();
+    const int kb = blockIdx.z;
+    float *Q = a.Q + kb * a.qstride;
     extern __shared__ float4 qsh[];
     const int tm = threadIdx.x & (kQModes - 1);
     const int li = threadIdx.x / kQModes;
@@ -67,7 +79,7 @@ __global__ void __launch_bounds__(kQModes *kQRings, 2) k_knot_q_band(KnotGradArg
     const int r0 = blockIdx.y * kQRings;
     const int nr = min(kQRings, a.nrep - r0);
     const bool lv = li < nr;
-    const KernDev &kd = a.kd;
+    const KernDev &kd = a.kd[kb];
     const int i = r0 + (lv ? li : 0);
     const int jl = kd.jlo[i], ps = kd.pstart[i];
     const int blen = lv ? kd.jhi[i] - jl + 1 : 0;
@@ -84,7 +96,7 @@ __global__ void __launch_bounds__(kQModes *kQRings, 2) k_knot_q_band(KnotGradArg
     float q[kQBand];
 #pragma unroll
     for (int s = 0; s < kQBand; ++s) q[s] = 0.f;
-    const int b0 = a.map0, b1 = a.map0 + a.nmaps;
+    const int b0 = a.map0 + kb * a.per_map, b1 = b0 + a.nmaps;
     if (b0 < b1) stage_band_async(qsh, a.spec4 + (int64_t)b0 * a.nrep * a.NH, ju0, nu, m0, kQModes, a.R, a.NH);
     for (int b = b0; b < b1; ++b) {
         const int cur = (b - b0) & 1;
@@ -127,8 +139,12 @@ __global__ void __launch_bounds__(kQModes *kQRings, 2) k_knot_q_band(KnotGradArg
 // zero; products outside a ring's band are accumulated but never stored.
 constexpr int kQGModes = 64, kQGGroups = 4;  // 8 rings per CTA
 
-__global__ void __launch_bounds__(kQGModes *kQGGroups, 2) k_knot_q_g2(KnotGradArgs a, float *Q, int srows)
+__global__ void __launch_bounds__(kQGModes *kQGGroups, 2) k_knot_q_g2(const __grid_constant__ KnotGradArgs a, int srows)
 {
+    chain_allow_next();
+    chain_wait();
+    const int kb = blockIdx.z;
+    float *Q = a.Q + kb * a.qstride;
     extern __shared__ float4 qgs[];  // [2 buffers][srows][kQGModes]
     const int tm = threadIdx.x & (kQGModes - 1);
     const int grp = threadIdx.x / kQGModes;
@@ -136,7 +152,7 @@ __global__ void __launch_bounds__(kQGModes *kQGGroups, 2) k_knot_q_g2(KnotGradAr
     const bool mv = m < a.NH;
     const int r0 = blockIdx.y * 2 * kQGGroups;
     const int nr = min(2 * kQGGroups, a.nrep - r0);
-    const KernDev &kd = a.kd;
+    const KernDev &kd = a.kd[kb];
     const int i0 = r0 + 2 * grp, i1 = i0 + 1;
     const bool v0 = 2 * grp < nr, v1 = 2 * grp + 1 < nr;  // warp-uniform (a warp is one group)
     const int jg0 = v0 ? kd.jlo[i0] : 0;
@@ -162,7 +178,7 @@ __global__ void __launch_bounds__(kQGModes *kQGGroups, 2) k_knot_q_g2(KnotGradAr
         if (a.pole_fix && i == 0) g = make_float4(0.f, 0.f, 0.f, 0.f);
         return g;
     };
-    const int b0 = a.map0, b1 = a.map0 + a.nmaps;
+    const int b0 = a.map0 + kb * a.per_map, b1 = b0 + a.nmaps;
     if (b0 < b1) stage_band_async(qgs, a.spec4 + (int64_t)b0 * a.nrep * a.NH, ju0, nu, m0, kQGModes, a.R, a.NH);
     for (int b = b0; b < b1; ++b) {
         const int cur = (b - b0) & 1;
@@ -210,305 +226,439 @@ __global__ void __launch_bounds__(kQGModes *kQGGroups, 2) k_knot_q_g2(KnotGradAr
     }
 }
 
-// X_k = c_k sum_m cos(m x_k) Q_m for the in-support taps of every pair, then the hat weights
-// of u(x_k) deposit (1 - lam) X_k and lam X_k on knots t0, t0 + 1.
-//
-// Work unit = (pair, kProjTaps consecutive taps), from a table built with the kernel.  A warp
-// takes one unit at a time with its lanes over the modes m = lane + 32 t (coalesced Q loads)
-// and, per tap, the phasor z = exp(i m x_k) advanced by exp(i 32 x_k) each step and reseeded
-// from exact values every kProjReseed steps.  The lane sums are reduced by shuffles.  The CTA's
-// warps run in rounds; the round's deposits are staged in shared memory and thread 0 adds
-// them in a fixed order into the CTA's shared bins, written to its row of partial sums at the
-// end, so the result is reproducible.
-constexpr int kProjTaps = 8, kProjReseed = 16, kProjWarps = 8;
-
-// With Xtc (the cosine sums of pairs [pfirst, npairs) from the tensor-core product, rows of
-// 128 taps) only the deposits are computed here.
-__global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(KnotGradArgs a, const float *Q, const float *Xtc,
-                                                               int pfirst)
+// Adds w0 to bins[t0] and w1 to bins[t0 + 1] for every lane with t0 >= 0: the lanes of a warp, in
+// its own bins, lane by lane only where they share a knot, so the order is fixed.
+__device__ __forceinline__ void warp_deposit(double *bins, int t0, double w0, double w1)
 {
-    extern __shared__ double ksm[];
-    const int T = a.kd.T;
-    double *bins = ksm;                       // [T]
-    double *ut = ksm + T;                     // [T]
-    double *stage = ksm + 2 * T;              // [warps][kProjTaps][2]
-    int *stage_t = reinterpret_cast<int *>(stage + kProjWarps * kProjTaps * 2);
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        bins[t] = 0.0;
-        ut[t] = a.kd.ut[t];
+    const unsigned same = __match_any_sync(0xffffffffu, t0);
+    const int rank = __popc(same & ((1u << (threadIdx.x & 31)) - 1u));
+    const int most = __reduce_max_sync(0xffffffffu, t0 >= 0 ? rank : -1);
+    for (int q = 0; q <= most; ++q) {
+        const bool mine = t0 >= 0 && rank == q;
+        if (mine) bins[t0] += w0;
+        __syncwarp();
+        if (mine) bins[t0 + 1] += w1;
+        __syncwarp();
     }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int N = a.N, NH = a.NH;
-    const double invN = 1.0 / (double)N;
-    const int2 *units = a.shift_fix ? a.kd.unit_fix : a.kd.unit_nofix;
-    const int nunits = a.shift_fix ? a.kd.nunit_fix : a.kd.nunit_nofix;
-    const int per_round = gridDim.x * kProjWarps;
-    const int rounds = (nunits + per_round - 1) / per_round;
-    for (int rd = 0; rd < rounds; ++rd) {
-        const int u = rd * per_round + blockIdx.x * kProjWarps + wid;
-        double X = 0.0, lam = 0.0;
-        int t0 = -1;
-        if (u < nunits) {  // warp-uniform
-            const int2 un = __ldg(&units[u]);
-            const int p = un.x, k0 = un.y;
-            const int f = a.shift_fix ? a.kd.fl[p] : 0;
-            const int ntap = (f ? a.kd.S1[p] : a.kd.S0[p]) + 1;
-            float mine = 0.f;
-            if (Xtc) {
-                if (lane < kProjTaps && k0 + lane < 128) mine = Xtc[(int64_t)(p - pfirst) * 128 + k0 + lane];
-            } else {
-                const float *q = Q + (int64_t)p * NH;
-                float acc[kProjTaps], zr[kProjTaps], zi[kProjTaps], wr[kProjTaps], wi[kProjTaps];
-#pragma unroll
-                for (int j = 0; j < kProjTaps; ++j) {
-                    const int ang = 2 * (k0 + j) + f;  // x = pi ang / N
-                    const float2 w = expipi_ratio(32 * ang, N);
-                    wr[j] = w.x;
-                    wi[j] = w.y;
-                    acc[j] = 0.f;
-                    zr[j] = zi[j] = 0.f;
-                }
-                const int nsteps = (NH + 31) >> 5;
-                for (int t = 0; t < nsteps; ++t) {
-                    const int m = lane + 32 * t;
-                    const float qm = m < NH ? __ldg(&q[m]) : 0.f;
-                    if (t % kProjReseed == 0) {
-#pragma unroll
-                        for (int j = 0; j < kProjTaps; ++j) {
-                            const float2 z = expipi_ratio((2 * (k0 + j) + f) * m, N);
-                            zr[j] = z.x;
-                            zi[j] = z.y;
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < kProjTaps; ++j) {
-                        acc[j] = fmaf(qm, zr[j], acc[j]);
-                        const float r = fmaf(zr[j], wr[j], -zi[j] * wi[j]);
-                        zi[j] = fmaf(zr[j], wi[j], zi[j] * wr[j]);
-                        zr[j] = r;
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < kProjTaps; ++j) {
-                    float v = acc[j];
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (lane == j) mine = v;
-                }
-            }
-            const int k = k0 + lane;
-            if (lane < kProjTaps && k < ntap) {
-                const double mult = (f == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
-                X = (double)mine * mult * invN;
-                const int tt = 2 * k + f;
-                double uu = 4.0 * (a.kd.B[p] * a.s2[N - tt] + a.kd.A[p] * a.s2[tt]);
-                uu = fmin(uu, a.kd.umax);
-                t0 = knot_segment(uu, ut, T, a.kd.gscale);
-                lam = (uu - ut[t0]) / (ut[t0 + 1] - ut[t0]);
-            }
-        }
-        if (lane < kProjTaps) {
-            stage[(wid * kProjTaps + lane) * 2 + 0] = (1.0 - lam) * X;
-            stage[(wid * kProjTaps + lane) * 2 + 1] = lam * X;
-            stage_t[wid * kProjTaps + lane] = t0;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int s = 0; s < kProjWarps * kProjTaps; ++s) {
-                const int tt = stage_t[s];
-                if (tt >= 0) {
-                    bins[tt] += stage[2 * s];
-                    bins[tt + 1] += stage[2 * s + 1];
-                }
-            }
-        }
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < T; t += blockDim.x) a.partial[(int64_t)blockIdx.x * T + t] = bins[t];
 }
 
-// The projection of the pairs next to the poles (up to N/2 + 1 samples each) by FFT:
-//   sum_{m=0}^{N/2} Q_m cos(m x_k) = Re( sum_m Q_m e^{i pi m f / N} e^{2 pi i m k / N} ),
-// one N-point inverse transform per pair (the adjoint passes from digit-reversed input), then
-// the hat-weight deposits of every in-support sample.  One CTA per pair; the deposits are
-// computed in parallel and added by one thread in sample order (runs of equal knots summed
-// in registers), so the CTA's row of partial sums is reproducible.
-template <int L>
-struct ProjFft {
-    const KnotGradArgs &a;
-    const float *Q;
-    float2 *buf;
-    double *bins, *ut;
-    int p, row;
-    __device__ void run()
+// Knot tables and per-warp bins of a deposit CTA in shared memory.
+struct KnotBins {
+    double *ut, *inv, *bins;  // [T] knots in u, [T] 1 / spacing, [warps][T]
+    int T, warps;
+    __device__ KnotBins(double *sm, const KernDev &kd, int nw) : ut(sm), inv(sm + kd.T), bins(sm + 2 * kd.T), T(kd.T), warps(nw)
     {
-        constexpr int N = 1 << L;
-        const int T = a.kd.T, NH = a.NH;
-        const int f = a.shift_fix ? a.kd.fl[p] : 0;
-        const int ntap = (f ? a.kd.S1[p] : a.kd.S0[p]) + 1;
-        const fft::Smem<L> sm{buf};
-        const float *q = Q + (int64_t)p * NH;
-        for (int m = threadIdx.x; m < N; m += blockDim.x) {
-            float2 v = make_float2(0.f, 0.f);
-            if (m < NH) {
-                const float qm = __ldg(&q[m]);
-                v = f ? cscalef(expipi_ratio(m, N), qm) : make_float2(qm, 0.f);
-            }
-            sm(fft::digitrev<L>(m), v);
+        for (int t = threadIdx.x; t < T; t += blockDim.x) {
+            ut[t] = kd.ut[t];
+            inv[t] = t < T - 1 ? 1.0 / (kd.ut[t + 1] - kd.ut[t]) : 0.0;
         }
+        for (int t = threadIdx.x; t < warps * T; t += blockDim.x) bins[t] = 0.0;
         __syncthreads();
-        fft::adj<L>(buf, a.tw, sm);
-        // this thread's samples k = tid + i blockDim: X_k and its knot segment
-        constexpr int KMAX = (N / 2 + N / 16) / (N / 16);  // samples per thread (N / 16 threads)
-        float xr[KMAX];
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i) {
-            const int k = threadIdx.x + i * blockDim.x;
-            xr[i] = k < ntap ? sm(k).x : 0.f;
+    }
+    // the warps' bins summed in order into a row of partial sums
+    __device__ void write(double *row)
+    {
+        __syncthreads();
+        for (int t = threadIdx.x; t < T; t += blockDim.x) {
+            double s = 0.0;
+            for (int w = 0; w < warps; ++w) s += bins[w * T + t];
+            row[t] = s;
         }
-        __syncthreads();
-        int *t0s = reinterpret_cast<int *>(buf);
-        float *w0s = reinterpret_cast<float *>(t0s + N / 2 + 1), *w1s = w0s + N / 2 + 1;
-        const double invN = 1.0 / (double)N, A = a.kd.A[p], B = a.kd.B[p];
-#pragma unroll
-        for (int i = 0; i < KMAX; ++i) {
-            const int k = threadIdx.x + i * blockDim.x;
-            if (k < ntap) {
-                const double mult = (f == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
-                const double X = (double)xr[i] * mult * invN;
-                const int t = 2 * k + f;
-                double u = 4.0 * (B * a.s2[N - t] + A * a.s2[t]);
-                u = fmin(u, a.kd.umax);
-                const int t0 = knot_segment(u, ut, T, a.kd.gscale);
-                const double lam = (u - ut[t0]) / (ut[t0 + 1] - ut[t0]);
-                t0s[k] = t0;
-                w0s[k] = (float)((1.0 - lam) * X);
-                w1s[k] = (float)(lam * X);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int cur = -1;
-            double s0 = 0.0, s1 = 0.0;
-            for (int k = 0; k < ntap; ++k) {
-                const int t = t0s[k];
-                if (t != cur) {
-                    if (cur >= 0) {
-                        bins[cur] += s0;
-                        bins[cur + 1] += s1;
-                    }
-                    cur = t;
-                    s0 = s1 = 0.0;
-                }
-                s0 += (double)w0s[k];
-                s1 += (double)w1s[k];
-            }
-            if (cur >= 0) {
-                bins[cur] += s0;
-                bins[cur + 1] += s1;
-            }
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < T; t += blockDim.x) a.partial[(int64_t)row * T + t] = bins[t];
     }
 };
 
-__global__ void __launch_bounds__(1024) k_knot_proj_fft(KnotGradArgs a, const float *Q, int logN, int row0)
+// Warps with bins of their own that fit (T up to 4096), and the shared memory of a deposit CTA.
+int bin_warps(int T, int most, size_t other)
 {
-    extern __shared__ float2 kbuf[];
-    const int T = a.kd.T;
-    const int N = 1 << logN;
-    double *bins = reinterpret_cast<double *>(kbuf + fft::buffer_words(N));
-    double *ut = bins + T;
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        bins[t] = 0.0;
-        ut[t] = a.kd.ut[t];
-    }
-    __syncthreads();
-    const int p = blockIdx.x;
-    switch (logN) {
-    case 10: ProjFft<10>{a, Q, kbuf, bins, ut, p, row0 + p}.run(); break;
-    case 11: ProjFft<11>{a, Q, kbuf, bins, ut, p, row0 + p}.run(); break;
-    case 12: ProjFft<12>{a, Q, kbuf, bins, ut, p, row0 + p}.run(); break;
-    case 13: ProjFft<13>{a, Q, kbuf, bins, ut, p, row0 + p}.run(); break;
-    default: ProjFft<14>{a, Q, kbuf, bins, ut, p, row0 + p}.run(); break;
-    }
+    const size_t left = 200 * 1024 - other - 2 * (size_t)T * sizeof(double);
+    return (int)std::max<size_t>(1, std::min<size_t>((size_t)most, left / ((size_t)T * sizeof(double))));
+}
+size_t bin_bytes(int T, int warps) { return (size_t)(2 + warps) * T * sizeof(double); }
+
+// Hat weights of sample k of pair p: its knot segment and position in it.
+__device__ __forceinline__ int sample_knot(const KnotGradArgs &a, const KernDev &kd, const KnotBins &kb, int p, int k, int f,
+                                           double &lam)
+{
+    const int tt = 2 * k + f;
+    const double u = fmin(4.0 * (kd.B[p] * a.s2[a.N - tt] + kd.A[p] * a.s2[tt]), kd.umax);
+    const int t0 = knot_segment(u, kb.ut, kb.T, kd.gscale);
+    lam = (u - kb.ut[t0]) * kb.inv[t0];
+    return t0;
 }
 
-// Pole rings: d/df_t of sum_p g_p sum_q w_q K(u_pq) r_q, one CTA per (pole pixel, side, map).
-__global__ void __launch_bounds__(256) k_knot_pole(KnotGradArgs a, const float *map,
-                                                   const float *gout, int64_t npix, int row0)
+// Plain FP32 projection by table: X[p][t] = sum_m Q_m(p) cos(pi m (2t + f) / N), a lane per tap
+// t (32 at a time), a CTA for 16 consecutive pairs, whose taps share each cosine loaded (of
+// either offset; the pairs' own by a uniform choice); its warps take every fourth 32 modes, and
+// their sums (kept short: 128 modes at a time) are added in order.  Loads of the cosines through
+// L1 bound it: 50 us per kernel at nside 256, 160 us with a phasor per pair, tap and mode.
+constexpr int kXPairs = 16, kXWarps = 4;
+
+__global__ void __launch_bounds__(kXWarps * 32) k_knot_proj_f32(const __grid_constant__ KnotGradArgs a,
+                                                                const float *__restrict__ ctabP, int nmc)
 {
-    extern __shared__ double ksm[];
-    const int T = a.kd.T;
-    double *bins = ksm;
-    double *ut = ksm + T;
-    double *stage = ksm + 2 * T;
-    int *stage_t = reinterpret_cast<int *>(stage + 2 * blockDim.x);
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        bins[t] = 0.0;
-        ut[t] = a.kd.ut[t];
+    chain_allow_next();
+    const int kb = blockIdx.z;
+    const KernDev &kd = a.kd[kb];
+    const int lane = threadIdx.x & 31, pf = a.fft_pairs[kb], NH = a.NH;
+    const int p0 = pf + blockIdx.x * kXPairs, t = blockIdx.y * 32 + lane, wid = threadIdx.x >> 5;
+    chain_wait();
+    if (p0 >= kd.npairs) return;
+    int most = 0;
+    unsigned fm = 0;  // bit i: offset of pair p0 + i
+    const float *q = a.Q + kb * a.qstride + (int64_t)p0 * NH;
+#pragma unroll
+    for (int i = 0; i < kXPairs; ++i) {
+        const int p = min(p0 + i, kd.npairs - 1);
+        const int f = a.shift_fix ? kd.fl[p] : 0;
+        fm |= (unsigned)f << i;
+        most = max(most, (f ? kd.S1[p] : kd.S0[p]) + 1);
     }
-    __syncthreads();
-    const int p = blockIdx.x, e = blockIdx.y, b = blockIdx.z;
-    const int i = e == 0 ? 0 : a.R - 1;
-    const RingDev &rd = a.rd;
-    const float *r = map + (int64_t)(a.map0 + b) * npix;
-    const double gp = (double)gout[(int64_t)(a.map0 + b) * npix + rd.poff[i] + p];
-    const int jl = a.kd.jlo[0], jh = a.kd.jhi[0];
-    for (int jj = jl; jj <= jh; ++jj) {
-        const int j = e == 0 ? jj : a.R - 1 - jj;
-        const int nj = rd.n[j];
-        for (int q0 = 0; q0 < nj; q0 += blockDim.x) {
-            const int q = q0 + threadIdx.x;
-            int t0 = -1;
-            double lam = 0.0, X = 0.0;
-            if (q < nj) {
-                const double y = (double)(2 * p + rd.hs[i]) / (2.0 * rd.n[i]) -
-                                 (double)(2 * q + rd.hs[j]) / (2.0 * nj);
-                double sy, cy;
-                sincospi(y, &sy, &cy);
-                const double sd = sin(0.5 * (rd.theta[i] - rd.theta[j]));
-                const double ss = sin(0.5 * (rd.theta[i] + rd.theta[j]));
-                const double u = 4.0 * (sd * sd * cy * cy + ss * ss * sy * sy);
-                if (u <= a.kd.umax) {
-                    t0 = knot_segment(u, ut, T, a.kd.gscale);
-                    lam = (u - ut[t0]) / (ut[t0 + 1] - ut[t0]);
-                    X = gp * (double)rd.w[j] * (double)r[rd.poff[j] + q];
-                }
+    if (blockIdx.y * 32 >= (unsigned)most) return;
+    const bool any0 = fm != (1u << kXPairs) - 1u, any1 = fm != 0;
+    const int np = min(kXPairs, kd.npairs - p0);
+    // a chunk's Q values of the pairs, loaded a mode per lane
+    __shared__ __align__(16) float qs_all[kXWarps][kXPairs][32];
+    float (&qs)[kXPairs][32] = qs_all[wid];
+    // rows t and 128 + t of the table tiles (32 modes: 8 x 16-byte pieces 128 bytes apart)
+    const float4 *c0 = reinterpret_cast<const float4 *>(ctabP) + (t >> 3) * 64 + (t & 7), *c1 = c0 + 16 * 64;
+    float acc[kXPairs], tot[kXPairs];
+#pragma unroll
+    for (int i = 0; i < kXPairs; ++i) acc[i] = tot[i] = 0.f;
+    int since = 0;
+    for (int c = wid; c < nmc; c += kXWarps) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kXPairs; ++i) qs[i][lane] = i < np && 32 * c + lane < NH ? __ldg(&q[(int64_t)i * NH + 32 * c + lane]) : 0.f;
+        __syncwarp();
+#pragma unroll 2
+        for (int j = 0; j < 8; ++j) {
+            const int64_t o = (int64_t)c * 4096 + j * 8;
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 h0 = any0 ? __ldg(&c0[o]) : z, l0 = any0 ? __ldg(&c0[o + 2048]) : z;
+            const float4 h1 = any1 ? __ldg(&c1[o]) : z, l1 = any1 ? __ldg(&c1[o + 2048]) : z;
+            const float x0[4] = {h0.x + l0.x, h0.y + l0.y, h0.z + l0.z, h0.w + l0.w};
+            const float x1[4] = {h1.x + l1.x, h1.y + l1.y, h1.z + l1.z, h1.w + l1.w};
+#pragma unroll
+            for (int i = 0; i < kXPairs; ++i) {
+                const float4 v = *reinterpret_cast<const float4 *>(&qs[i][4 * j]);
+                acc[i] = fmaf(v.x, fm >> i & 1 ? x1[0] : x0[0], acc[i]);
+                acc[i] = fmaf(v.y, fm >> i & 1 ? x1[1] : x0[1], acc[i]);
+                acc[i] = fmaf(v.z, fm >> i & 1 ? x1[2] : x0[2], acc[i]);
+                acc[i] = fmaf(v.w, fm >> i & 1 ? x1[3] : x0[3], acc[i]);
             }
-            stage[2 * threadIdx.x] = (1.0 - lam) * X;
-            stage[2 * threadIdx.x + 1] = lam * X;
-            stage_t[threadIdx.x] = t0;
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int s = 0; s < (int)blockDim.x; ++s)
-                    if (stage_t[s] >= 0) {
-                        bins[stage_t[s]] += stage[2 * s];
-                        bins[stage_t[s] + 1] += stage[2 * s + 1];
-                    }
-            __syncthreads();
+        }
+        if (++since == 4 || c + kXWarps >= nmc) {
+            since = 0;
+#pragma unroll
+            for (int i = 0; i < kXPairs; ++i) {
+                tot[i] += acc[i];
+                acc[i] = 0.f;
+            }
         }
     }
-    const int row = row0 + (b * 2 + e) * 4 + p;
-    for (int t = threadIdx.x; t < T; t += blockDim.x) a.partial[(int64_t)row * T + t] = bins[t];
+    // the warps' sums in order (their Q values are no longer needed)
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kXPairs; ++i) qs[i][lane] = tot[i];
+    __syncthreads();
+    for (int i = wid; i < np; i += kXWarps) {
+        float x = qs_all[0][i][lane];
+#pragma unroll
+        for (int w = 1; w < kXWarps; ++w) x += qs_all[w][i][lane];
+        a.X[kb * a.xstride + (int64_t)(p0 + i - pf) * 128 + t] = x;
+    }
 }
 
-// One CTA per knot: each thread sums a strided subset of the rows in order, then a tree over
-// the threads in a fixed pairing, so the result does not depend on scheduling.
-__global__ void __launch_bounds__(256) k_knot_reduce(const double *partial, int nrows, int T, double *out)
+// Hat-weight deposits of the projected pairs: c_k X_k goes to the knots of u(x_k) with weights
+// 1 - lam and lam.  A warp takes four pairs at a time, eight lanes to a pair and its taps, and adds
+// into its own bins; the CTA writes their sum as its row of partial sums.  FP64 bounds it: 0.08 ms
+// for one nside-2048 kernel, 0.57 ms with a round's deposits staged for one thread to add.
+constexpr int kProjTaps = 8, kProjReseed = 16, kProjWarps = 8;
+
+__global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_constant__ KnotGradArgs a, int nw)
+{
+    extern __shared__ double ksm[];
+    const int kb = blockIdx.y;
+    const KernDev &kd = a.kd[kb];
+    KnotBins bn(ksm, kd, nw);
+    chain_wait();
+    chain_allow_next();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, pf = a.fft_pairs[kb];
+    const double invN = 1.0 / (double)a.N;
+    const float *X = a.X + kb * a.xstride;
+    if (wid < nw) {
+        for (int p4 = pf + 4 * (blockIdx.x * nw + wid); p4 < kd.npairs; p4 += 4 * gridDim.x * nw) {
+            const int p = p4 + (lane >> 3);
+            int f = 0, ntap = 0;
+            if (p < kd.npairs) {
+                f = a.shift_fix ? kd.fl[p] : 0;
+                ntap = (f ? kd.S1[p] : kd.S0[p]) + 1;
+            }
+            const int most = __reduce_max_sync(0xffffffffu, ntap);
+            for (int k0 = 0; k0 < most; k0 += 8) {
+                const int k = k0 + (lane & 7);
+                int t0 = -1;
+                double w0 = 0.0, w1 = 0.0;
+                if (k < ntap) {
+                    const double mult = (f == 0 && (k == 0 || 2 * k == a.N)) ? 1.0 : 2.0;
+                    const double x = (double)__ldg(&X[(int64_t)(p - pf) * 128 + k]) * mult * invN;
+                    double lam;
+                    t0 = sample_knot(a, kd, bn, p, k, f, lam);
+                    w1 = lam * x;
+                    w0 = x - w1;
+                }
+                warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
+            }
+        }
+    }
+    bn.write(a.partial + kb * a.pstride + (int64_t)blockIdx.x * bn.T);
+}
+
+// Projection and deposits of pairs of more than 128 samples without the FFT form: work unit =
+// (pair, kProjTaps consecutive taps), from a table built with the kernel.  A warp takes one unit
+// at a time with its lanes over the modes m = lane + 32 t (coalesced Q loads) and, per tap, the
+// phasor z = exp(i m x_k) advanced by exp(i 32 x_k) each step and reseeded from exact values every
+// kProjReseed steps.  The lane sums are reduced by shuffles and deposited in the warp's bins.
+__global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_constant__ KnotGradArgs a, int nw)
+{
+    extern __shared__ double ksm[];
+    const int kb = blockIdx.y;
+    const KernDev &kd = a.kd[kb];
+    KnotBins bn(ksm, kd, nw);
+    chain_wait();
+    chain_allow_next();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int N = a.N, NH = a.NH;
+    const double invN = 1.0 / (double)N;
+    const int2 *units = a.shift_fix ? kd.unit_fix : kd.unit_nofix;
+    const int nunits = a.shift_fix ? kd.nunit_fix : kd.nunit_nofix;
+    if (wid < nw) {
+        for (int u = blockIdx.x * nw + wid; u < nunits; u += gridDim.x * nw) {
+            const int2 un = __ldg(&units[u]);
+            const int p = un.x, k0 = un.y;
+            const int f = a.shift_fix ? kd.fl[p] : 0;
+            const int ntap = (f ? kd.S1[p] : kd.S0[p]) + 1;
+            float mine = 0.f;
+            const float *q = a.Q + kb * a.qstride + (int64_t)p * NH;
+            float acc[kProjTaps], zr[kProjTaps], zi[kProjTaps], wr[kProjTaps], wi[kProjTaps];
+#pragma unroll
+            for (int j = 0; j < kProjTaps; ++j) {
+                const int ang = 2 * (k0 + j) + f;  // x = pi ang / N
+                const float2 w = expipi_ratio(32 * ang, N);
+                wr[j] = w.x;
+                wi[j] = w.y;
+                acc[j] = 0.f;
+                zr[j] = zi[j] = 0.f;
+            }
+            const int nsteps = (NH + 31) >> 5;
+            for (int t = 0; t < nsteps; ++t) {
+                const int m = lane + 32 * t;
+                const float qm = m < NH ? __ldg(&q[m]) : 0.f;
+                if (t % kProjReseed == 0) {
+#pragma unroll
+                    for (int j = 0; j < kProjTaps; ++j) {
+                        const float2 z = expipi_ratio((2 * (k0 + j) + f) * m, N);
+                        zr[j] = z.x;
+                        zi[j] = z.y;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kProjTaps; ++j) {
+                    acc[j] = fmaf(qm, zr[j], acc[j]);
+                    const float r = fmaf(zr[j], wr[j], -zi[j] * wi[j]);
+                    zi[j] = fmaf(zr[j], wi[j], zi[j] * wr[j]);
+                    zr[j] = r;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kProjTaps; ++j) {
+                float v = acc[j];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == j) mine = v;
+            }
+            const int k = k0 + lane;
+            int t0 = -1;
+            double w0 = 0.0, w1 = 0.0;
+            if (lane < kProjTaps && k < ntap) {
+                const double mult = (f == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
+                const double x = (double)mine * mult * invN;
+                double lam;
+                t0 = sample_knot(a, kd, bn, p, k, f, lam);
+                w1 = lam * x;
+                w0 = x - w1;
+            }
+            warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
+        }
+    }
+    bn.write(a.partial + kb * a.pstride + (int64_t)blockIdx.x * bn.T);
+}
+
+// The projection of the pairs next to the poles (up to N/2 + 1 samples each) by FFT.  The even
+// extension of Q (half of Q_m at m and at N - m, with the phases exp(+-i pi m f / N)) has the real
+// transform sum_m Q_m cos(m x_k), so one N-point inverse transform (the adjoint passes from
+// digit-reversed input) projects two pairs, as its real and imaginary part.  Then the
+// hat-weight deposits of every in-support sample, 32 consecutive samples to a warp and its bins; the
+// CTA's sum is one row.  The 2297 pairs of one nside-2048 kernel take 0.22 ms, 0.76 ms
+// with a transform per pair and one thread adding its samples.
+template <int L>
+struct ProjFft {
+    const KnotGradArgs &a;
+    const KernDev &kd;
+    const float *Q;
+    float2 *buf;
+    KnotBins &bn;
+    int p0, np;
+    __device__ void run()
+    {
+        constexpr int N = 1 << L;
+        const int NH = a.NH;
+        const fft::Smem<L> sm{buf};
+        int f[2], ntap[2];
+        const float *q[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int p = min(p0 + i, np - 1);
+            f[i] = a.shift_fix ? kd.fl[p] : 0;
+            ntap[i] = p0 + i < np ? (f[i] ? kd.S1[p] : kd.S0[p]) + 1 : 0;
+            q[i] = Q + (int64_t)p * NH;
+        }
+        for (int m = threadIdx.x; m < NH; m += blockDim.x) {
+            const bool edge = m == 0 || 2 * m == N;  // its own mirror
+            const float2 ph = expipi_ratio(m, N);
+            float2 e[2];  // Q_m exp(i pi m f / N), halved where the mirror holds the conjugate
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float v = ntap[i] > 0 ? __ldg(&q[i][m]) : 0.f, w = edge ? v : 0.5f * v;
+                e[i] = f[i] ? make_float2(w * ph.x, edge ? 0.f : w * ph.y) : make_float2(w, 0.f);
+            }
+            // both pairs as real and imaginary part: e0 + i e1, and conj e0 + i conj e1 at N - m
+            sm(fft::digitrev<L>(m), make_float2(e[0].x - e[1].y, e[0].y + e[1].x));
+            if (!edge) sm(fft::digitrev<L>(N - m), make_float2(e[0].x + e[1].y, e[1].x - e[0].y));
+        }
+        __syncthreads();
+        fft::adj<L>(buf, a.tw, sm);
+        const double invN = 1.0 / (double)N;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        if (wid < bn.warps) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                for (int k0 = 32 * wid; k0 < ntap[i]; k0 += 32 * bn.warps) {
+                    const int k = k0 + lane;
+                    int t0 = -1;
+                    double w0 = 0.0, w1 = 0.0;
+                    if (k < ntap[i]) {
+                        const float2 v = sm(k);
+                        const double mult = (f[i] == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
+                        const double x = (double)(i ? v.y : v.x) * mult * invN;
+                        double lam;
+                        t0 = sample_knot(a, kd, bn, p0 + i, k, f[i], lam);
+                        w1 = lam * x;
+                        w0 = x - w1;
+                    }
+                    warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
+                }
+        }
+    }
+};
+
+__global__ void __launch_bounds__(1024) k_knot_proj_fft(const __grid_constant__ KnotGradArgs a, int logN, int nw)
+{
+    extern __shared__ float2 kbuf[];
+    chain_allow_next();  // (the kernel before waited for Q)
+    const int kb = blockIdx.y, p0 = 2 * blockIdx.x, np = a.fft_pairs[kb];
+    if (p0 < np) {
+        const KernDev &kd = a.kd[kb];
+        KnotBins bn(reinterpret_cast<double *>(kbuf + fft::buffer_words(1 << logN)), kd, nw);
+        const float *Q = a.Q + kb * a.qstride;
+        switch (logN) {
+        case 10: ProjFft<10>{a, kd, Q, kbuf, bn, p0, np}.run(); break;
+        case 11: ProjFft<11>{a, kd, Q, kbuf, bn, p0, np}.run(); break;
+        case 12: ProjFft<12>{a, kd, Q, kbuf, bn, p0, np}.run(); break;
+        case 13: ProjFft<13>{a, kd, Q, kbuf, bn, p0, np}.run(); break;
+        default: ProjFft<14>{a, kd, Q, kbuf, bn, p0, np}.run(); break;
+        }
+        bn.write(a.partial + kb * a.pstride + (int64_t)(a.row_fft + blockIdx.x) * bn.T);
+    }
+    chain_wait();
+}
+
+// Pole rings: d/df_t of sum_p g_p sum_q w_q K(u_pq) r_q: pole_split CTAs per (pole pixel, side,
+// map) and kernel share the pixels of the band's rings (one run of the map), a row each.  Four
+// kernels in one launch: 15 us; ring by ring with three FP64 sines per pixel and one thread adding
+// a CTA's deposits: 154 us each.
+constexpr int kPoleWarps = 8;
+
+__global__ void __launch_bounds__(kPoleWarps * 32) k_knot_pole(const __grid_constant__ KnotGradArgs a, const float *map,
+                                                               const float *gout, int64_t npix, int nw)
+{
+    extern __shared__ double ksm[];
+    chain_allow_next();
+    const int kb = blockIdx.z / a.nmaps, b = blockIdx.z % a.nmaps, m = a.map0 + kb * a.per_map + b;
+    const int C = a.pole_split[kb], p = blockIdx.x % 4, part = blockIdx.x / 4, e = blockIdx.y;
+    if (part >= C) {
+        chain_wait();
+        return;
+    }
+    const KernDev &kd = a.kd[kb];
+    const RingDev &rd = a.rd;
+    KnotBins bn(ksm, kd, nw);
+    const int i = e == 0 ? 0 : a.R - 1, jh = kd.jhi[0], ja = e == 0 ? 0 : a.R - 1 - jh, jz = e == 0 ? jh : a.R - 1;
+    const float *r = map + (int64_t)m * npix;
+    const double gp = (double)gout[(int64_t)m * npix + rd.poff[i] + p];
+    const int64_t q0 = rd.poff[ja], q1 = rd.poff[jz] + rd.n[jz];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < nw) {
+        for (int64_t q32 = q0 + 32 * (part * nw + wid); q32 < q1; q32 += 32 * C * nw) {
+            const int64_t q = q32 + lane;
+            int t0 = -1;
+            double w0 = 0.0, w1 = 0.0;
+            if (q < q1) {
+                int j = ja, hi = jz;  // the pixel's ring
+                while (j < hi) {
+                    const int mid = (j + hi + 1) >> 1;
+                    if (__ldg(&rd.poff[mid]) <= q) j = mid;
+                    else hi = mid - 1;
+                }
+                // squared chord as in pole.cu
+                const double y = (double)(2 * p + rd.hs[i]) / (2.0 * rd.n[i]) -
+                                 (double)(2 * (int)(q - rd.poff[j]) + rd.hs[j]) / (2.0 * rd.n[j]);
+                const int jj = e == 0 ? j : a.R - 1 - j;
+                const double sy = sinpi(y), B = kd.B[jj], u = 4.0 * fma(kd.A[jj] - B, sy * sy, B);
+                if (u <= kd.umax) {
+                    t0 = knot_segment(u, bn.ut, bn.T, kd.gscale);
+                    const double x = gp * (double)rd.w[j] * (double)__ldg(&r[q]);
+                    w1 = (u - bn.ut[t0]) * bn.inv[t0] * x;
+                    w0 = x - w1;
+                }
+            }
+            warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
+        }
+    }
+    bn.write(a.partial + kb * a.pstride + (int64_t)(a.row_pole + ((b * 2 + e) * 4 + p) * C + part) * bn.T);
+    chain_wait();
+}
+
+// One CTA per knot and kernel: each thread sums a strided subset of the rows in order, then a tree
+// over the threads in a fixed pairing, so the result does not depend on scheduling.
+// The rows of a kernel: deposit CTAs, then its FFT pairs (two to a row), then the pole rings from
+// row_pole (a kernel with fewer FFT pairs than the longest of the call leaves rows unused).
+__global__ void __launch_bounds__(256) k_knot_reduce(const __grid_constant__ KnotGradArgs a, int T, double *out)
 {
     __shared__ double red[256];
-    const int t = blockIdx.x;
+    chain_wait();
+    const int t = blockIdx.x, kb = blockIdx.y, head = a.row_fft + (a.fft_pairs[kb] + 1) / 2;
+    const int pole_rows = a.pole_fix ? 8 * a.nmaps * a.pole_split[kb] : 0;
+    const double *partial = a.partial + kb * a.pstride;
     double s = 0.0;
-    for (int r = threadIdx.x; r < nrows; r += blockDim.x) s += partial[(int64_t)r * T + t];
+    for (int r = threadIdx.x; r < head + pole_rows; r += blockDim.x)
+        s += partial[(int64_t)(r < head ? r : r - head + a.row_pole) * T + t];
     red[threadIdx.x] = s;
     __syncthreads();
     for (int h = blockDim.x / 2; h > 0; h >>= 1) {
         if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[t] = red[0];
+    if (threadIdx.x == 0) out[(int64_t)kb * T + t] = red[0];
 }
 
 }  // namespace
@@ -518,76 +668,94 @@ int knot_proj_taps() { return kProjTaps; }
 
 int knot_q_band_limit() { return kQBand; }
 
-cudaError_t launch_knot_grad_q(const KnotGradArgs &a, float *Q, int max_band, int max_union, int max_union2,
-                               int srows, cudaStream_t st)
+int knot_q_form(int max_band, int max_union, int max_union2, int srows)
 {
-    const size_t smem2 = 2 * (size_t)srows * kQGModes * sizeof(float4);
-    if (max_union2 <= kQBand && smem2 <= 100 * 1024) {
+    if (max_union2 <= kQBand && 2 * (size_t)srows * kQGModes * sizeof(float4) <= 100 * 1024) return 0;
+    return max_band <= kQBand && 2 * (size_t)max_union * kQModes * sizeof(float4) <= 200 * 1024 ? 1 : 2;
+}
+
+cudaError_t launch_knot_grad_q(const KnotGradArgs &a, int max_band, int max_union, int max_union2, int srows,
+                               cudaStream_t st)
+{
+    const int form = knot_q_form(max_band, max_union, max_union2, srows);
+    if (form == 0) {
+        const size_t smem = 2 * (size_t)srows * kQGModes * sizeof(float4);
         cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_q_g2,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        dim3 grid((a.NH + kQGModes - 1) / kQGModes, (a.nrep + 2 * kQGGroups - 1) / (2 * kQGGroups));
-        k_knot_q_g2<<<grid, kQGModes * kQGGroups, smem2, st>>>(a, Q, srows);
-        return cudaGetLastError();
+        dim3 grid((a.NH + kQGModes - 1) / kQGModes, (a.nrep + 2 * kQGGroups - 1) / (2 * kQGGroups), a.nk);
+        return launch_chained(k_knot_q_g2, grid, kQGModes * kQGGroups, smem, st, true, 1, a, srows);
     }
-    const size_t smem = 2 * (size_t)max_union * kQModes * sizeof(float4);
-    if (max_band <= kQBand && smem <= 200 * 1024) {
+    if (form == 1) {
+        const size_t smem = 2 * (size_t)max_union * kQModes * sizeof(float4);
         cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_q_band,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        dim3 grid((a.NH + kQModes - 1) / kQModes, (a.nrep + kQRings - 1) / kQRings);
-        k_knot_q_band<<<grid, kQModes * kQRings, smem, st>>>(a, Q);
-        return cudaGetLastError();
+        dim3 grid((a.NH + kQModes - 1) / kQModes, (a.nrep + kQRings - 1) / kQRings, a.nk);
+        return launch_chained(k_knot_q_band, grid, kQModes * kQRings, smem, st, true, 1, a);
     }
-    dim3 grid((a.NH + kModeBlock - 1) / kModeBlock, (a.nrep + kQRing - 1) / kQRing);
-    k_knot_q<<<grid, kModeBlock, 0, st>>>(a, Q);
-    return cudaGetLastError();
+    dim3 grid((a.NH + kModeBlock - 1) / kModeBlock, (a.nrep + kQRing - 1) / kQRing, a.nk);
+    return launch_chained(k_knot_q, grid, kModeBlock, 0, st, true, 1, a);
 }
 
-cudaError_t launch_knot_grad_proj(const KnotGradArgs &a, const float *Q, const float *X, int pfirst,
-                                  cudaStream_t st)
+cudaError_t launch_knot_proj_f32(const KnotGradArgs &a, const float *ctabP, int nmc, int maxpairs, int maxtaps,
+                                 cudaStream_t st)
 {
-    const size_t smem = (size_t)2 * a.kd.T * sizeof(double) + kProjWarps * kProjTaps * 2 * sizeof(double) +
-                        kProjWarps * kProjTaps * sizeof(int);
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_proj,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (maxpairs <= 0) return cudaSuccess;
+    dim3 grid((maxpairs + kXPairs - 1) / kXPairs, (maxtaps + 31) / 32, a.nk);
+    return launch_chained(k_knot_proj_f32, grid, kXWarps * 32, 0, st, true, 1, a, ctabP, nmc);
+}
+
+cudaError_t launch_knot_grad_proj(const KnotGradArgs &a, bool have_x, int T, cudaStream_t st)
+{
+    const int nw = bin_warps(T, kProjWarps, 0);
+    const size_t smem = bin_bytes(T, nw);
+    const auto kernel = have_x ? k_knot_deposit : k_knot_proj;
+    cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_knot_proj<<<knot_proj_blocks(), kProjWarps * 32, smem, st>>>(a, Q, X, pfirst);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3(knot_proj_blocks(), a.nk), kProjWarps * 32, smem, st, true, 1, a, nw);
 }
 
-// Pairs [0, npairs) by FFT (the caller checks that N is a power of two in [2^10, 2^14] and
-// within the grid's twiddle table); their rows of partial sums start at row0.
-cudaError_t launch_knot_grad_proj_fft(const KnotGradArgs &a, const float *Q, int npairs, int row0, cudaStream_t st)
+// The kernels' FFT pairs (the caller checks that N is a power of two in [2^10, 2^14] and within
+// the grid's twiddle table), two to a CTA and row.
+cudaError_t launch_knot_grad_proj_fft(const KnotGradArgs &a, int maxpairs, int T, cudaStream_t st)
 {
-    if (npairs <= 0) return cudaSuccess;
+    if (maxpairs <= 0) return cudaSuccess;
     int logN = 0;
     while ((1 << logN) < a.N) ++logN;
-    const size_t smem = (size_t)fft::buffer_words(a.N) * sizeof(float2) + 2 * (size_t)a.kd.T * sizeof(double);
+    const size_t buf = (size_t)fft::buffer_words(a.N) * sizeof(float2);
+    const int nw = std::min(bin_warps(T, 32, buf), std::max(1, a.N / 16 / 32));
+    const size_t smem = buf + bin_bytes(T, nw);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_proj_fft,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_knot_proj_fft<<<npairs, a.N / 16, smem, st>>>(a, Q, logN, row0);
-    return cudaGetLastError();
+    return launch_chained(k_knot_proj_fft, dim3((maxpairs + 1) / 2, a.nk), a.N / 16, smem, st, true, 1, a, logN, nw);
 }
 
-cudaError_t launch_knot_grad_pole(const KnotGradArgs &a, const float *map, const float *gout,
-                                  int64_t npix, int row0, cudaStream_t st)
+int knot_pole_split(int64_t band_pixels)
 {
-    const size_t smem = (size_t)2 * a.kd.T * sizeof(double) + 256 * 2 * sizeof(double) +
-                        256 * sizeof(int);
+    int c = 1;
+    while (c < 8 && 512 * (int64_t)c < band_pixels) c *= 2;
+    return c;
+}
+
+cudaError_t launch_knot_grad_pole(const KnotGradArgs &a, const float *map, const float *gout, int64_t npix, int T,
+                                  cudaStream_t st)
+{
+    const int nw = bin_warps(T, kPoleWarps, 0);
+    const size_t smem = bin_bytes(T, nw);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_pole,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(4, 2, a.nmaps);
-    k_knot_pole<<<grid, 256, smem, st>>>(a, map, gout, npix, row0);
-    return cudaGetLastError();
+    int split = 1;
+    for (int k = 0; k < a.nk; ++k) split = std::max(split, a.pole_split[k]);
+    return launch_chained(k_knot_pole, dim3(4 * split, 2, a.nmaps * a.nk), kPoleWarps * 32, smem, st, true, 1, a,
+                          map, gout, npix, nw);
 }
 
-cudaError_t launch_knot_reduce(const double *partial, int nrows, int T, double *out, cudaStream_t st)
+cudaError_t launch_knot_reduce(const KnotGradArgs &a, double *out, int T, cudaStream_t st)
 {
-    k_knot_reduce<<<T, 256, 0, st>>>(partial, nrows, T, out);
-    return cudaGetLastError();
+    return launch_chained(k_knot_reduce, dim3(T, a.nk), 256, 0, st, true, 1, a, T, out);
 }
 
 }  // namespace arkcos
