@@ -112,13 +112,16 @@ __device__ __forceinline__ void dispatch_upto(int logM, F &f)
 }
 
 // Launch shape of the class of buffers up to 2^LMAX (LMAX >= 10): one thread per radix-16
-// group of the largest buffer, at least 256 (the short rings' folds and extensions run over
-// all kernel-grid modes with the whole CTA), and two CTAs per SM below the largest buffer, so
-// that the register budget follows.
+// group of the largest buffer, at least 256, and two CTAs per SM below the largest buffer, so
+// that the register budget follows.  The short rings (LMAX = 10) have at most 64 such groups:
+// their CTAs have 64 threads, eight to an SM (four nside-512 maps, forward stage 128 -> 92 us against
+// 256 threads), but 128 for the inverse transforms of kernel grids past 2048 points, where the folds
+// run over all kernel-grid modes with the whole CTA (one nside-1024 map: 151 us with 256
+// threads, 127 with 128, 147 with 64; at nside 512 54, 49 and 40 us).
 template <int LMAX>
 struct ClassShape {
-    static constexpr int kThreads = (1 << LMAX) / 16 < 256 ? 256 : (1 << LMAX) / 16;
-    static constexpr int kMinBlocks = LMAX >= 13 ? 1 : 2;
+    static constexpr int kThreads = LMAX <= 10 ? 128 : (1 << LMAX) / 16 < 256 ? 256 : (1 << LMAX) / 16;  // (at most)
+    static constexpr int kMinBlocks = LMAX >= 13 ? 1 : 512 / kThreads;
 };
 
 // Launch order inside one transform stage.  The buffer classes of a stage write disjoint rings

@@ -262,7 +262,7 @@ cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int
 template <int LMAX>
 cudaError_t launch_fwd_class(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev)
 {
-    constexpr int T = ring::ClassShape<LMAX>::kThreads;
+    const int T = LMAX <= 10 ? 64 : ring::ClassShape<LMAX>::kThreads;
     const size_t smem = fft_smem_bytes(a.M, a.N, false, a.tab, T);
     cudaError_t e = set_smem((const void *)k_fft_fwd<LMAX>, smem);
     if (e != cudaSuccess) return e;

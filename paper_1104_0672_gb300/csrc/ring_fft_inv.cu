@@ -349,7 +349,7 @@ size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads)
 template <int LMAX>
 cudaError_t launch_inv_class(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev)
 {
-    constexpr int T = ring::ClassShape<LMAX>::kThreads;
+    const int T = LMAX <= 10 && a.N <= 2048 ? 64 : ring::ClassShape<LMAX>::kThreads;
     const size_t smem = fft_smem_bytes(a.M, a.N, a.stage_c != 0, a.tab, T);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_fft_inv<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
