@@ -237,7 +237,7 @@ arkcos_status finish_grid(Grid &g)
         c.blu = b;
         c.M = mx;
         c.logM = ilog2(mx);
-        c.threads = c.M <= 1024 ? 128 : std::min(512, std::max(256, c.M / 16));  // at most (ring::ClassShape)
+        c.threads = std::min(512, std::max(128, c.M / 16));  // at most (ring::ClassShape)
         c.count = (int)reps.size();
         // staging the coefficients of short rings is an optimisation: drop it where it does not
         // fit beside the transform buffer (long kernel grids)

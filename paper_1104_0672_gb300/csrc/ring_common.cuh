@@ -120,7 +120,7 @@ __device__ __forceinline__ void dispatch_upto(int logM, F &f)
 // threads, 127 with 128, 147 with 64; at nside 512 54, 49 and 40 us).
 template <int LMAX>
 struct ClassShape {
-    static constexpr int kThreads = LMAX <= 10 ? 128 : (1 << LMAX) / 16 < 256 ? 256 : (1 << LMAX) / 16;  // (at most)
+    static constexpr int kThreads = LMAX <= 10 ? 128 : (1 << LMAX) / 16;  // (at most)
     static constexpr int kMinBlocks = LMAX >= 13 ? 1 : 512 / kThreads;
 };
 
