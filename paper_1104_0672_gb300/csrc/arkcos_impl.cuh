@@ -37,6 +37,7 @@ struct FftClass {
     int count = 0;
     int stage_c = 0;      // some ring of the class is shorter than N / 4
     int blu = 0;          // a split Bluestein class (ring_blu.cuh)
+    int even_h = 1;       // ... whose rings all have a multiple of four pixels
     int tab = 0;          // largest chirp + phase table of the class (complex words)
     int *reps = nullptr;  // device array of representative (northern) ring indices
 };
@@ -265,7 +266,7 @@ cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int
 // stage_allow_next / stage_wait_prev).
 cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_fwd(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev);
-cudaError_t launch_blu_inv(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev);
+cudaError_t launch_blu_inv(const FftInvArgs &a, bool even_h, int count, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_spectra(const FftFwdArgs &a, float2 *fb, int count, cudaStream_t st);  // a.logM, rd, reps, tw
 int blu_table_words(int h);                // words of the per-ring tables of a ring of n = 2h pixels
 size_t blu_smem_bytes(int M, int tab);

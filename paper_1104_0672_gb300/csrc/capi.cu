@@ -227,6 +227,7 @@ arkcos_status finish_grid(Grid &g)
             if (b) {
                 mx = 1 << l;
                 c.tab = std::max(c.tab, blu_table_words(n / 2));
+                if (n % 4) c.even_h = 0;
                 continue;
             }
             mx = std::max(mx, (int)buffer_of(n / 2));
@@ -662,7 +663,7 @@ arkcos_status run_fft_inv(const Grid &g, const float2 *cbuf, float *map, int64_t
         a.skip_poles = skip_poles;
         a.stage_c = c.stage_c;
         a.tab = c.tab;
-        if (c.blu) CK(launch_blu_inv(a, c.count, st, after_prev));
+        if (c.blu) CK(launch_blu_inv(a, c.even_h != 0, c.count, st, after_prev));
         else CK(launch_fft_inv(a, c.count, c.threads, st, after_prev));
     }
     return ARKCOS_OK;

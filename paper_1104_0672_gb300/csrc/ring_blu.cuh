@@ -25,10 +25,11 @@ namespace ring {
 
 using fft::cpair;
 
-// CTA of the class of M = 2^L: two teams of M / 16 threads; 128 registers per thread.
-template <int L>
+// CTA of the class of M = 2^L: two teams of M / 16 threads, or four that run both half sequences
+// at once; 128 registers per thread.
+template <int L, bool BOTH = false>
 struct BluShape {
-    static constexpr int kM = 1 << L, kTeam = kM / 16, kThreads = 2 * kTeam;
+    static constexpr int kM = 1 << L, kTeam = kM / 16, kThreads = (BOTH ? 4 : 2) * kTeam;
     static constexpr int kMinBlocks = 512 / kThreads;
     static constexpr int kBuf = fft::buffer_words(kM);
 };
@@ -42,9 +43,9 @@ __host__ __device__ constexpr int blu_twiddle_words(int M) { return M / 4 + M / 
 
 // Shared memory of a class of lengths l <= lmax: two buffers, the chirps of s = 0 and 1 and the
 // phase table.
-inline size_t blu_smem_bytes(int M, int tab)
+inline size_t blu_smem_bytes(int M, int tab, int buffers = 2)
 {
-    return 2 * (size_t)fft::buffer_words(M) * sizeof(cpair) + (size_t)(tab + blu_twiddle_words(M)) * sizeof(float2);
+    return buffers * (size_t)fft::buffer_words(M) * sizeof(cpair) + (size_t)(tab + blu_twiddle_words(M)) * sizeof(float2);
 }
 
 // Words of the per-ring tables: chirp exp(-+ i pi t^2 / l) for t <= l/2, the same of t (t + 1)
@@ -99,13 +100,15 @@ __device__ __forceinline__ BluTables blu_tables(float2 *words, int h, int n, int
     return BluTables{ca, cb, p, l, h, sgn};
 }
 
-// Barrier of the T threads of team e (a warp when T = 32).
+// Barrier of the T threads of team e < 4 (a warp when T = 32).
 template <int T>
 __device__ __forceinline__ void team_sync(int e)
 {
     if constexpr (T <= 32) __syncwarp();
     else if (e == 0) asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
-    else asm volatile("bar.sync 2, %0;" ::"n"(T) : "memory");
+    else if (e == 1) asm volatile("bar.sync 2, %0;" ::"n"(T) : "memory");
+    else if (e == 2) asm volatile("bar.sync 3, %0;" ::"n"(T) : "memory");
+    else asm volatile("bar.sync 4, %0;" ::"n"(T) : "memory");
 }
 
 // v[k] *= w^k for k = 1..15 (conjugated when CONJ) from w, w^2, w^3 and w^4, as fft::twiddle.

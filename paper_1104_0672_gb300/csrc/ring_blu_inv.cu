@@ -15,24 +15,30 @@ using ring::BluTables;
 // would leave room for one CTA per SM).  Bounds and batching as the forward kernel; 16
 // nside-2048 maps: the rings of 2048 < n < 8192 pixels 2.8 -> 2.3 ms, the whole stage 4.28 -> 3.79
 // ms; six nside-4096 maps 10.4 -> 6.9 ms.
-template <int L>
-__global__ void __launch_bounds__(BluShape<L>::kThreads, BluShape<L>::kMinBlocks) k_blu_inv(const __grid_constant__ FftInvArgs a)
+//
+// BOTH (M <= 1024, rings of even h): four teams run both half sequences at once, with one fold for
+// both -- short transforms leave room for the four buffers (12 nside-474 maps, inverse stage
+// 485 -> 290 us, 64 nside-1024 maps 3.99 -> 3.54 ms).
+template <int L, bool BOTH>
+__global__ void __launch_bounds__(BluShape<L, BOTH>::kThreads, BluShape<L, BOTH>::kMinBlocks)
+k_blu_inv(const __grid_constant__ FftInvArgs a)
 {
-    using Sh = BluShape<L>;
+    using Sh = BluShape<L, BOTH>;
     using namespace fft;
     constexpr int M = Sh::kM;
     // two buffers | twiddles | per-ring tables
     extern __shared__ float4 smem4[];
     if (!a.first) chain_allow_next();
+    // (four with BOTH: those of s = 1 behind those of s = 0)
     cpair *buf0 = reinterpret_cast<cpair *>(smem4), *buf1 = buf0 + Sh::kBuf;
     const int i = a.reps[blockIdx.x], i2 = a.R - 1 - i, n = a.rd.n[i], h = n / 2, hs = a.rd.hs[i], nyq = a.N / 2;
-    float2 *twA = reinterpret_cast<float2 *>(buf1 + Sh::kBuf), *twB = twA + M / 4;
+    float2 *twA = reinterpret_cast<float2 *>(buf0 + (BOTH ? 4 : 2) * Sh::kBuf), *twB = twA + M / 4;
     ring::blu_twiddles<L>(twA, a.tw);
     const BluTables tb = ring::blu_tables(twA + ring::blu_twiddle_words(M), h, n, +1);
     const int S = (h & 1) ? 1 : 2, l = h / S;
     const bool pair = i2 != i;
     const float wsc = a.weight ? a.rd.w[i] : 1.0f, inv = 0.5f / (float)M;
-    const int e = threadIdx.x / Sh::kTeam, tid = threadIdx.x % Sh::kTeam;
+    const int team = threadIdx.x / Sh::kTeam, e = team & 1, tid = threadIdx.x % Sh::kTeam;
     const float2 *fb = a.rd.fb + a.rd.fboff[i] + e * M;
     if (a.first) {
         // the first class of the stage starts beside the end of the contraction; the next class
@@ -111,14 +117,23 @@ __global__ void __launch_bounds__(BluShape<L>::kThreads, BluShape<L>::kMinBlocks
         };
         float2 *o1 = reinterpret_cast<float2 *>(a.map + (int64_t)b * a.npix + a.rd.poff[i]);
         float2 *o2 = reinterpret_cast<float2 *>(a.map + (int64_t)b * a.npix + a.rd.poff[i2]);
-        for (int s = 0; s < S; ++s) {
-            // input k of both convolutions: the radix-2 step and the chirp, W^k for the odd ones
-            auto put = [&](int k, const cpair &v) {
-                const cpair x = e_mul(v, tb.chirp(s, k));
-                buf0[ring::bsp(k)] = x;
-                buf1[ring::bsp(k)] = e_mul(x, __ldg(&a.tw[M + k]));
+        for (int s = 0; s < (BOTH ? 1 : S); ++s) {
+            // input k of the convolutions from the two halves p, q of the radix-2 step: p + q (s = 0),
+            // p - q (s = 1) times the chirp, and W^k for the odd frequencies
+            auto put1 = [&](cpair *b, int half, int k, const cpair &v) {
+                const cpair x = e_mul(v, tb.chirp(half, k));
+                b[ring::bsp(k)] = x;
+                b[Sh::kBuf + ring::bsp(k)] = e_mul(x, __ldg(&a.tw[M + k]));
             };
-            if (S == 2) {
+            auto put = [&](int k, const cpair &p, const cpair &q) {
+                if (BOTH) {
+                    put1(buf0, 0, k, e_add(p, q));
+                    put1(buf0 + 2 * Sh::kBuf, 1, k, e_sub(p, q));
+                } else {
+                    put1(buf0, s, k, s ? e_sub(p, q) : e_add(p, q));
+                }
+            };
+            if (BOTH || S == 2) {
                 for (int k = threadIdx.x; 2 * k <= l; k += Sh::kThreads) {
                     // Z_k, Z_{h-k} and Z_{l-k}, Z_{l+k}: inputs k and l - k
                     cpair x[4], z0, z1, z2, z3;
@@ -127,11 +142,11 @@ __global__ void __launch_bounds__(BluShape<L>::kThreads, BluShape<L>::kMinBlocks
                     unsplit(x[0], x[1], k, z0, z1);
                     if (k == 0) {
                         unsplit(x[2], x[2], l, z2, z3);
-                        put(0, s ? e_sub(z0, z2) : e_add(z0, z2));
+                        put(0, z0, z2);
                     } else {
                         unsplit(x[2], x[3], l - k, z2, z3);
-                        put(k, s ? e_sub(z0, z3) : e_add(z0, z3));
-                        if (2 * k != l) put(l - k, s ? e_sub(z2, z1) : e_add(z2, z1));
+                        put(k, z0, z3);
+                        if (2 * k != l) put(l - k, z2, z1);
                     }
                 }
             } else {
@@ -140,16 +155,19 @@ __global__ void __launch_bounds__(BluShape<L>::kThreads, BluShape<L>::kMinBlocks
                     const int mm[2] = {k, h - k};
                     folded(mm, x);
                     unsplit(x[0], x[1], k, z0, z1);
-                    put(k, z0);
-                    if (k > 0) put(h - k, z1);
+                    put1(buf0, 0, k, z0);
+                    if (k > 0) put1(buf0, 0, h - k, z1);
                 }
             }
-            for (int k = l + threadIdx.x; k < M; k += Sh::kThreads) buf0[ring::bsp(k)] = buf1[ring::bsp(k)] = e_zero(cpair{});
+            for (int k = l + threadIdx.x; k < M; k += Sh::kThreads) {
+                buf0[ring::bsp(k)] = buf1[ring::bsp(k)] = e_zero(cpair{});
+                if (BOTH) buf0[2 * Sh::kBuf + ring::bsp(k)] = buf1[2 * Sh::kBuf + ring::bsp(k)] = e_zero(cpair{});
+            }
             __syncthreads();
-            cpair *x = e ? buf1 : buf0, v[16];
+            cpair *x = buf0 + team * Sh::kBuf, v[16];
 #pragma unroll
             for (int r = 0; r < 16; ++r) v[r] = x[ring::bsp(tid + r * Sh::kTeam)];
-            ring::blu_convolve<L, true>(v, x, twA, twB, fb, tid, e);
+            ring::blu_convolve<L, true>(v, x, twA, twB, fb, tid, team);
             ring::blu_scale<L, true>(v, a.tw, l, tid, e, inv, [&](int t) { return tb.chirp0(t); });
 #pragma unroll
             for (int r = 0; r < 16; ++r) x[ring::bsp(tid + r * Sh::kTeam)] = v[r];
@@ -157,8 +175,14 @@ __global__ void __launch_bounds__(BluShape<L>::kThreads, BluShape<L>::kMinBlocks
 #pragma unroll 4
             for (int t = threadIdx.x; t < l; t += Sh::kThreads) {
                 const cpair z = e_add(buf0[ring::bsp(t)], buf1[ring::bsp(t)]);
-                o1[S * t + s] = make_float2(z.re.x, z.im.x);
-                if (pair) o2[S * t + s] = make_float2(z.re.y, z.im.y);
+                const int o = BOTH ? 2 * t : S * t + s;
+                o1[o] = make_float2(z.re.x, z.im.x);
+                if (pair) o2[o] = make_float2(z.re.y, z.im.y);
+                if (BOTH) {
+                    const cpair w = e_add(buf0[2 * Sh::kBuf + ring::bsp(t)], buf1[2 * Sh::kBuf + ring::bsp(t)]);
+                    o1[o + 1] = make_float2(w.re.x, w.im.x);
+                    if (pair) o2[o + 1] = make_float2(w.re.y, w.im.y);
+                }
             }
             __syncthreads();
         }
@@ -166,27 +190,28 @@ __global__ void __launch_bounds__(BluShape<L>::kThreads, BluShape<L>::kMinBlocks
     chain_wait();
 }
 
-template <int L>
+template <int L, bool BOTH>
 cudaError_t launch_inv(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev)
 {
-    using Sh = BluShape<L>;
-    const size_t smem = ring::blu_smem_bytes(Sh::kM, a.tab);
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_blu_inv<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    using Sh = BluShape<L, BOTH>;
+    const size_t smem = ring::blu_smem_bytes(Sh::kM, a.tab, BOTH ? 4 : 2);
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_blu_inv<L, BOTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_blu_inv<L>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), Sh::kThreads, smem, st,
+    return launch_chained(k_blu_inv<L, BOTH>, dim3(count, (a.B + a.mchunk - 1) / a.mchunk), Sh::kThreads, smem, st,
                           after_prev, 1, a);
 }
 
 }  // namespace
 
-cudaError_t launch_blu_inv(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev)
+// even_h: every ring of the class has an even h
+cudaError_t launch_blu_inv(const FftInvArgs &a, bool even_h, int count, cudaStream_t st, bool after_prev)
 {
     if (count <= 0) return cudaSuccess;
     switch (a.logM) {
-    case 9: return launch_inv<9>(a, count, st, after_prev);
-    case 10: return launch_inv<10>(a, count, st, after_prev);
-    case 11: return launch_inv<11>(a, count, st, after_prev);
-    default: return launch_inv<12>(a, count, st, after_prev);
+    case 9: return even_h ? launch_inv<9, true>(a, count, st, after_prev) : launch_inv<9, false>(a, count, st, after_prev);
+    case 10: return even_h ? launch_inv<10, true>(a, count, st, after_prev) : launch_inv<10, false>(a, count, st, after_prev);
+    case 11: return launch_inv<11, false>(a, count, st, after_prev);
+    default: return launch_inv<12, false>(a, count, st, after_prev);
     }
 }
 
