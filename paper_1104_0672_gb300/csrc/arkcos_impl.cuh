@@ -265,7 +265,7 @@ cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int
 // of the same stage, and this launch may begin while it still runs (ring_common.cuh
 // stage_allow_next / stage_wait_prev).
 cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
-cudaError_t launch_blu_fwd(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev);
+cudaError_t launch_blu_fwd(const FftFwdArgs &a, bool even_h, int count, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_inv(const FftInvArgs &a, bool even_h, int count, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_spectra(const FftFwdArgs &a, float2 *fb, int count, cudaStream_t st);  // a.logM, rd, reps, tw
 int blu_table_words(int h);                // words of the per-ring tables of a ring of n = 2h pixels

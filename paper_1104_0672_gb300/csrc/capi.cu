@@ -629,7 +629,7 @@ arkcos_status run_fft_fwd(const Grid &g, const float *map, float2 *spec, float4 
         a.weight = weight;
         a.zero_poles = zero_poles;
         a.tab = c.tab;
-        if (c.blu) CK(launch_blu_fwd(a, c.count, st, after_prev));
+        if (c.blu) CK(launch_blu_fwd(a, c.even_h != 0, c.count, st, after_prev));
         else CK(launch_fft_fwd(a, c.count, c.threads, st, after_prev));
     }
     return ARKCOS_OK;

@@ -16,9 +16,10 @@ using ring::BluTables;
 // nside-2048 maps: the rings of 2048 < n < 8192 pixels 2.8 -> 2.3 ms, the whole stage 4.28 -> 3.79
 // ms; six nside-4096 maps 10.4 -> 6.9 ms.
 //
-// BOTH (M <= 1024, rings of even h): four teams run both half sequences at once, with one fold for
+// BOTH (M <= 2048, rings of even h): four teams run both half sequences at once, with one fold for
 // both -- short transforms leave room for the four buffers (12 nside-474 maps, inverse stage
-// 485 -> 290 us, 64 nside-1024 maps 3.99 -> 3.54 ms).
+// 485 -> 290 us, 64 nside-1024 maps 3.99 -> 3.54 ms; at M = 2048,
+// where it leaves one CTA per SM, eight nside-2048 maps 1.86 -> 1.83 ms).
 template <int L, bool BOTH>
 __global__ void __launch_bounds__(BluShape<L, BOTH>::kThreads, BluShape<L, BOTH>::kMinBlocks)
 k_blu_inv(const __grid_constant__ FftInvArgs a)
@@ -210,7 +211,7 @@ cudaError_t launch_blu_inv(const FftInvArgs &a, bool even_h, int count, cudaStre
     switch (a.logM) {
     case 9: return even_h ? launch_inv<9, true>(a, count, st, after_prev) : launch_inv<9, false>(a, count, st, after_prev);
     case 10: return even_h ? launch_inv<10, true>(a, count, st, after_prev) : launch_inv<10, false>(a, count, st, after_prev);
-    case 11: return launch_inv<11, false>(a, count, st, after_prev);
+    case 11: return even_h ? launch_inv<11, true>(a, count, st, after_prev) : launch_inv<11, false>(a, count, st, after_prev);
     default: return launch_inv<12, false>(a, count, st, after_prev);
     }
 }
