@@ -338,7 +338,6 @@ cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, 
 cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks, const TcTables &tb, int srows,
                                     cudaStream_t st);
 int contract_tc_nbuf(int rb, int gs, int srows, int want_nbuf);
-size_t contract_tc_smem(int rb, int gs, int srows, int want_nbuf);
 int contract_tc_modes();
 cudaError_t take_tc_error(int *out);
 // Failure-detection test knob, read on every call: when the environment variable

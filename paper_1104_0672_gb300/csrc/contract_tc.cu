@@ -895,11 +895,6 @@ size_t tc_ctl(int rb, int nbuf, int srows)
 
 }  // namespace
 
-size_t contract_tc_smem(int rb, int gs, int srows, int want_nbuf)
-{
-    return tc_ctl(rb, contract_tc_nbuf(rb, gs, srows, want_nbuf), srows) + 32;
-}
-
 int contract_band_limit() { return kTcBand; }
 
 namespace {

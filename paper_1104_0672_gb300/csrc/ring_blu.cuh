@@ -11,7 +11,8 @@
 // the lower half of the output is wanted, so the 2M-point convolution is two independent
 // M-point ones, the even and the odd frequencies (e = 0, 1; W = e^{-i pi / M}):
 //     y_t = ( y0_t + W^{-t} y1_t ) / 2M,   y_e = M IDFT_M( fb_e DFT_M( x_t W^{e t} ) ).
-// Half of the CTA runs each, M / 16 threads with 16 elements apiece: three radix passes forward,
+// A team of M / 16 threads with 16 elements apiece runs each (two teams, or four where the CTA takes
+// both half sequences at once): three radix passes forward,
 // the product and three back, of which the inner two on each side stay within a warp.
 // Against one 2h - 1-point buffer per ring the same rings need half the buffer (so two CTAs fit
 // an SM where one did, and one's loads and barriers overlap the other's arithmetic), four

@@ -11,8 +11,7 @@ using ring::BluShape;
 using ring::BluTables;
 
 // The two spectra (even and odd frequencies of the 2M-point DFT, each in DIF order of M points,
-// laid out as blu_convolve reads it)
-// of the Bluestein sequence b_k = exp(+i pi k^2 / l), |k| < l, circular in 2M: once per grid.
+// laid out as blu_convolve reads it) of the Bluestein sequence b_k = exp(+i pi k^2 / l), |k| < l, circular in 2M: once per grid.
 template <int L>
 __global__ void __launch_bounds__(BluShape<L>::kTeam) k_blu_spectra(RingDev rd, const int *reps, const float2 *tw,
                                                                     float2 *fb_all)
@@ -39,9 +38,9 @@ __global__ void __launch_bounds__(BluShape<L>::kTeam) k_blu_spectra(RingDev rd, 
 
 // One ring pair: see ring_blu.cuh.  What bounds it: arithmetic and exchanges at 16 warps per SM
 // (registers); the pixels, the next pass's twiddles and the chirp spectrum are asked for in whole
-// batches, as latency, not arithmetic, took most of the time before.  16 nside-2048 maps: the
-// rings of 2048 < n < 8192 pixels 2.5 -> 2.0 ms, the whole stage 3.71 -> 3.20 ms; six nside-4096
-// maps (rings up to 16380 pixels, four quarter transforms before) 7.8 -> 6.1 ms.
+// batches, as latency, not arithmetic, took most of the time before.  The forward stage of 16
+// nside-2048 maps 3.71 -> 3.06 ms (one long buffer per ring before), of six nside-4096 maps (rings
+// up to 16380 pixels, four quarter transforms before) 7.8 -> 6.1 ms.
 //
 // BOTH (M <= 1024, rings of even h): four teams run both half sequences at once and the pixels are
 // loaded once (12 nside-474 maps, forward stage 345 -> 274 us; at M = 2048, one CTA per SM, slower:
@@ -53,10 +52,9 @@ k_blu_fwd(const __grid_constant__ FftFwdArgs a)
     using Sh = BluShape<L, BOTH>;
     using namespace fft;
     constexpr int M = Sh::kM;
-    // two buffers | twiddles | per-ring tables
+    // two buffers (four with BOTH: those of s = 1 behind those of s = 0) | twiddles | per-ring tables
     extern __shared__ float4 smem4[];
     chain_allow_next();
-    // (four with BOTH: those of s = 1 behind those of s = 0)
     cpair *buf0 = reinterpret_cast<cpair *>(smem4), *buf1 = buf0 + Sh::kBuf;
     const int j = a.reps[blockIdx.x], j2 = a.R - 1 - j, n = a.rd.n[j], h = n / 2, hs = a.rd.hs[j];
     float2 *twA = reinterpret_cast<float2 *>(buf0 + (BOTH ? 4 : 2) * Sh::kBuf), *twB = twA + M / 4;

@@ -11,15 +11,15 @@ using ring::BluShape;
 using ring::BluTables;
 
 // One ring pair: see ring_blu.cuh.  The two half sequences of a ring each take every folded
-// coefficient, so the fold runs twice rather than keep one of them in shared memory (which
-// would leave room for one CTA per SM).  Bounds and batching as the forward kernel; 16
-// nside-2048 maps: the rings of 2048 < n < 8192 pixels 2.8 -> 2.3 ms, the whole stage 4.28 -> 3.79
-// ms; six nside-4096 maps 10.4 -> 6.9 ms.
+// coefficient; at M = 4096 and for odd h the fold runs once per half sequence rather than keep one
+// of them in shared memory.  Bounds and batching as the forward kernel; the inverse stage of 16
+// nside-2048 maps 4.28 -> 3.54 ms (one long buffer per ring before), of six nside-4096 maps
+// 10.4 -> 6.9 ms (four quarter transforms before).
 //
 // BOTH (M <= 2048, rings of even h): four teams run both half sequences at once, with one fold for
 // both -- short transforms leave room for the four buffers (12 nside-474 maps, inverse stage
-// 485 -> 290 us, 64 nside-1024 maps 3.99 -> 3.54 ms; at M = 2048,
-// where it leaves one CTA per SM, eight nside-2048 maps 1.86 -> 1.83 ms).
+// 485 -> 290 us, 64 nside-1024 maps 3.99 -> 3.54 ms; at M = 2048, where it leaves one CTA per SM,
+// eight nside-2048 maps 1.86 -> 1.83 ms).
 template <int L, bool BOTH>
 __global__ void __launch_bounds__(BluShape<L, BOTH>::kThreads, BluShape<L, BOTH>::kMinBlocks)
 k_blu_inv(const __grid_constant__ FftInvArgs a)
@@ -27,10 +27,9 @@ k_blu_inv(const __grid_constant__ FftInvArgs a)
     using Sh = BluShape<L, BOTH>;
     using namespace fft;
     constexpr int M = Sh::kM;
-    // two buffers | twiddles | per-ring tables
+    // two buffers (four with BOTH: those of s = 1 behind those of s = 0) | twiddles | per-ring tables
     extern __shared__ float4 smem4[];
     if (!a.first) chain_allow_next();
-    // (four with BOTH: those of s = 1 behind those of s = 0)
     cpair *buf0 = reinterpret_cast<cpair *>(smem4), *buf1 = buf0 + Sh::kBuf;
     const int i = a.reps[blockIdx.x], i2 = a.R - 1 - i, n = a.rd.n[i], h = n / 2, hs = a.rd.hs[i], nyq = a.N / 2;
     float2 *twA = reinterpret_cast<float2 *>(buf0 + (BOTH ? 4 : 2) * Sh::kBuf), *twB = twA + M / 4;
