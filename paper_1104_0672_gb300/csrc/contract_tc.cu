@@ -596,9 +596,8 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                     // coefficients of the G rings (a ring's even and odd slots lie in different
                     // tiles), then the staged values, each used by all G rings
                     constexpr int CH = 8, UNROLL = WIDE ? 1 : kTcBand / CH;  // (wide: less code, 4.5 against 5.1 ms)
-#pragma unroll(UNROLL)
-                    for (int h = 0; h < kTcBand; h += CH) {
-                        uint32_t cr[G][2][CH / 2];
+                    uint32_t cr[G][2][CH / 2];
+                    auto coeffs = [&](int h) {
 #pragma unroll
                         for (int t = 0; t < G; ++t)
 #pragma unroll
@@ -606,6 +605,10 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                                 tmem_ld_async(lane_base + (uint32_t)(((t + o) & 1) * kTile + (G * grp + t) * 16 + h / 2),
                                               cr[t][o]);
                         tmem_wait_ld();
+                    };
+#pragma unroll(UNROLL)
+                    for (int h = 0; h < kTcBand; h += CH) {
+                        coeffs(h);
                         if (!crosses && (!WIDE || inner)) {
 #pragma unroll
                             for (int u = 0; u < CH; ++u) {
@@ -622,6 +625,43 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                                 for (int t = 0; t < G; ++t)
                                     if (!WIDE || (h + u >= lo[t] && h + u <= hi[t]))
                                         fma4(acc[t], __uint_as_float(cr[t][u & 1][u >> 1]), v);
+                            }
+                        }
+                    }
+                    if constexpr (!WIDE) {
+                        // a non-finite value of a staged ring times the zero coefficient of a ring
+                        // whose band lacks it is NaN: a warp that finds such sums takes them again over
+                        // the slots of each ring's own band (the same sums otherwise).  A test of the
+                        // sums, as one of every slot costs more (one nside-256 map, plain FP32: 112 us
+                        // without a test, 114 with this one, 122 with a test of the slots; 16
+                        // nside-2048 maps, 3xTF32: 9.54, 9.55 and 9.74 ms)
+                        float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int t = 0; t < G; ++t)
+                            s = caddf(s, caddf(make_float2(acc[t].x, acc[t].y), make_float2(acc[t].z, acc[t].w)));
+                        if (__any_sync(0xffffffffu, !isfinite(s.x + s.y))) {
+                            uint32_t in[G];  // slots of the ring's band
+#pragma unroll
+                            for (int t = 0; t < G; ++t) {
+                                const int i = r0 + min(G * grp + t, nr - 1), jl = kd.jlo[i];
+                                in[t] = (0xffffffffu >> (kTcBand - 1 - (kd.jhi[i] - jl))) << (jl - jg0);
+                                acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+#pragma unroll 1
+                            for (int h = 0; h < kTcBand; h += CH) {
+                                coeffs(h);
+#pragma unroll
+                                for (int u = 0; u < CH; ++u) {
+                                    float4 v = col[(h + u) * kTcModes];
+                                    if (h + u >= sstar) v = make_float4(v.z, v.w, v.x, v.y);
+#pragma unroll
+                                    for (int t = 0; t < G; ++t) {
+                                        // (the plain form has no registers left for the masks)
+                                        const int i = r0 + min(G * grp + t, nr - 1), j = jg0 + h + u;
+                                        if (F32 ? j >= __ldg(&kd.jlo[i]) && j <= __ldg(&kd.jhi[i]) : in[t] >> (h + u) & 1)
+                                            fma4(acc[t], __uint_as_float(cr[t][u & 1][u >> 1]), v);
+                                    }
+                                }
                             }
                         }
                     }
