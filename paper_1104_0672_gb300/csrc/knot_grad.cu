@@ -242,19 +242,28 @@ __device__ __forceinline__ void warp_deposit(double *bins, int t0, double w0, do
     }
 }
 
+// Warps of a deposit CTA with bins of their own, and whether the table of reciprocal knot spacings has
+// room beside them.
+struct BinShape {
+    int warps, table;
+};
+
 // Knot tables and per-warp bins of a deposit CTA in shared memory.
 struct KnotBins {
-    double *ut, *inv, *bins;  // [T] knots in u, [T] 1 / spacing, [warps][T]
+    double *ut, *inv, *bins;  // [T] knots in u, [T] 1 / spacing (none: divided per sample), [warps][T]
     int T, warps;
-    __device__ KnotBins(double *sm, const KernDev &kd, int nw) : ut(sm), inv(sm + kd.T), bins(sm + 2 * kd.T), T(kd.T), warps(nw)
+    __device__ KnotBins(double *sm, const KernDev &kd, BinShape bs)
+        : ut(sm), inv(bs.table ? sm + kd.T : nullptr), bins(sm + (1 + bs.table) * kd.T), T(kd.T), warps(bs.warps)
     {
         for (int t = threadIdx.x; t < T; t += blockDim.x) {
             ut[t] = kd.ut[t];
-            inv[t] = t < T - 1 ? 1.0 / (kd.ut[t + 1] - kd.ut[t]) : 0.0;
+            if (inv) inv[t] = t < T - 1 ? 1.0 / (kd.ut[t + 1] - kd.ut[t]) : 0.0;
         }
         for (int t = threadIdx.x; t < warps * T; t += blockDim.x) bins[t] = 0.0;
         __syncthreads();
     }
+    // 1 / spacing of segment t < T - 1
+    __device__ __forceinline__ double spacing(int t) const { return inv ? inv[t] : 1.0 / (ut[t + 1] - ut[t]); }
     // the warps' bins summed in order into a row of partial sums
     __device__ void write(double *row)
     {
@@ -267,13 +276,18 @@ struct KnotBins {
     }
 };
 
-// Warps with bins of their own that fit (T up to 4096), and the shared memory of a deposit CTA.
-int bin_warps(int T, int most, size_t other)
+// Deposit CTA of up to `most` warps with bins of their own beside `other` bytes, T up to 4096: as many
+// as fit 200 KB with both tables, but one at least.  Beside the 16384-point transform of
+// k_knot_proj_fft (139392 bytes) that one fits the 227 KB of a CTA with both tables up to T = 3877, and
+// with the knots alone up to T = 4096.
+BinShape bin_shape(int T, int most, size_t other)
 {
-    const size_t left = 200 * 1024 - other - 2 * (size_t)T * sizeof(double);
-    return (int)std::max<size_t>(1, std::min<size_t>((size_t)most, left / ((size_t)T * sizeof(double))));
+    const int64_t row = (int64_t)T * (int64_t)sizeof(double);
+    const int64_t rows = std::max<int64_t>(0, 200 * 1024 - (int64_t)other) / row;
+    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(most, rows - 2));
+    return BinShape{warps, (int64_t)other + (2 + warps) * row <= 227 * 1024};
 }
-size_t bin_bytes(int T, int warps) { return (size_t)(2 + warps) * T * sizeof(double); }
+size_t bin_bytes(int T, BinShape bs) { return (size_t)(1 + bs.table + bs.warps) * T * sizeof(double); }
 
 // Hat weights of sample k of pair p: its knot segment and position in it.
 __device__ __forceinline__ int sample_knot(const KnotGradArgs &a, const KernDev &kd, const KnotBins &kb, int p, int k, int f,
@@ -282,7 +296,7 @@ __device__ __forceinline__ int sample_knot(const KnotGradArgs &a, const KernDev 
     const int tt = 2 * k + f;
     const double u = fmin(4.0 * (kd.B[p] * a.s2[a.N - tt] + kd.A[p] * a.s2[tt]), kd.umax);
     const int t0 = knot_segment(u, kb.ut, kb.T, kd.gscale);
-    lam = (u - kb.ut[t0]) * kb.inv[t0];
+    lam = (u - kb.ut[t0]) * kb.spacing(t0);
     return t0;
 }
 
@@ -375,12 +389,13 @@ __global__ void __launch_bounds__(kXWarps * 32) k_knot_proj_f32(const __grid_con
 // for one nside-2048 kernel, 0.57 ms with a round's deposits staged for one thread to add.
 constexpr int kProjTaps = 8, kProjReseed = 16, kProjWarps = 8;
 
-__global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_constant__ KnotGradArgs a, int nw)
+__global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_constant__ KnotGradArgs a, BinShape bs)
 {
     extern __shared__ double ksm[];
     const int kb = blockIdx.y;
     const KernDev &kd = a.kd[kb];
-    KnotBins bn(ksm, kd, nw);
+    KnotBins bn(ksm, kd, bs);
+    const int nw = bs.warps;
     chain_wait();
     chain_allow_next();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, pf = a.fft_pairs[kb];
@@ -419,12 +434,13 @@ __global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_c
 // at a time with its lanes over the modes m = lane + 32 t (coalesced Q loads) and, per tap, the
 // phasor z = exp(i m x_k) advanced by exp(i 32 x_k) each step and reseeded from exact values every
 // kProjReseed steps.  The lane sums are reduced by shuffles and deposited in the warp's bins.
-__global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_constant__ KnotGradArgs a, int nw)
+__global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_constant__ KnotGradArgs a, BinShape bs)
 {
     extern __shared__ double ksm[];
     const int kb = blockIdx.y;
     const KernDev &kd = a.kd[kb];
-    KnotBins bn(ksm, kd, nw);
+    KnotBins bn(ksm, kd, bs);
+    const int nw = bs.warps;
     chain_wait();
     chain_allow_next();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -561,14 +577,14 @@ struct ProjFft {
     }
 };
 
-__global__ void __launch_bounds__(1024) k_knot_proj_fft(const __grid_constant__ KnotGradArgs a, int logN, int nw)
+__global__ void __launch_bounds__(1024) k_knot_proj_fft(const __grid_constant__ KnotGradArgs a, int logN, BinShape bs)
 {
     extern __shared__ float2 kbuf[];
     chain_allow_next();  // (the kernel before waited for Q)
     const int kb = blockIdx.y, p0 = 2 * blockIdx.x, np = a.fft_pairs[kb];
     if (p0 < np) {
         const KernDev &kd = a.kd[kb];
-        KnotBins bn(reinterpret_cast<double *>(kbuf + fft::buffer_words(1 << logN)), kd, nw);
+        KnotBins bn(reinterpret_cast<double *>(kbuf + fft::buffer_words(1 << logN)), kd, bs);
         const float *Q = a.Q + kb * a.qstride;
         switch (logN) {
         case 10: ProjFft<10>{a, kd, Q, kbuf, bn, p0, np}.run(); break;
@@ -589,7 +605,7 @@ __global__ void __launch_bounds__(1024) k_knot_proj_fft(const __grid_constant__ 
 constexpr int kPoleWarps = 8;
 
 __global__ void __launch_bounds__(kPoleWarps * 32) k_knot_pole(const __grid_constant__ KnotGradArgs a, const float *map,
-                                                               const float *gout, int64_t npix, int nw)
+                                                               const float *gout, int64_t npix, BinShape bs)
 {
     extern __shared__ double ksm[];
     chain_allow_next();
@@ -601,7 +617,8 @@ __global__ void __launch_bounds__(kPoleWarps * 32) k_knot_pole(const __grid_cons
     }
     const KernDev &kd = a.kd[kb];
     const RingDev &rd = a.rd;
-    KnotBins bn(ksm, kd, nw);
+    KnotBins bn(ksm, kd, bs);
+    const int nw = bs.warps;
     const int i = e == 0 ? 0 : a.R - 1, jh = kd.jhi[0], ja = e == 0 ? 0 : a.R - 1 - jh, jz = e == 0 ? jh : a.R - 1;
     const float *r = map + (int64_t)m * npix;
     const double gp = (double)gout[(int64_t)m * npix + rd.poff[i] + p];
@@ -627,7 +644,7 @@ __global__ void __launch_bounds__(kPoleWarps * 32) k_knot_pole(const __grid_cons
                 if (u <= kd.umax) {
                     t0 = knot_segment(u, bn.ut, bn.T, kd.gscale);
                     const double x = gp * (double)rd.w[j] * (double)__ldg(&r[q]);
-                    w1 = (u - bn.ut[t0]) * bn.inv[t0] * x;
+                    w1 = (u - bn.ut[t0]) * bn.spacing(t0) * x;
                     w0 = x - w1;
                 }
             }
@@ -708,12 +725,12 @@ cudaError_t launch_knot_proj_f32(const KnotGradArgs &a, const float *ctabP, int 
 
 cudaError_t launch_knot_grad_proj(const KnotGradArgs &a, bool have_x, int T, cudaStream_t st)
 {
-    const int nw = bin_warps(T, kProjWarps, 0);
-    const size_t smem = bin_bytes(T, nw);
+    const BinShape bs = bin_shape(T, kProjWarps, 0);
+    const size_t smem = bin_bytes(T, bs);
     const auto kernel = have_x ? k_knot_deposit : k_knot_proj;
     cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(kernel, dim3(knot_proj_blocks(), a.nk), kProjWarps * 32, smem, st, true, 1, a, nw);
+    return launch_chained(kernel, dim3(knot_proj_blocks(), a.nk), kProjWarps * 32, smem, st, true, 1, a, bs);
 }
 
 // The kernels' FFT pairs (the caller checks that N is a power of two in [2^10, 2^14] and within
@@ -724,12 +741,12 @@ cudaError_t launch_knot_grad_proj_fft(const KnotGradArgs &a, int maxpairs, int T
     int logN = 0;
     while ((1 << logN) < a.N) ++logN;
     const size_t buf = (size_t)fft::buffer_words(a.N) * sizeof(float2);
-    const int nw = std::min(bin_warps(T, 32, buf), std::max(1, a.N / 16 / 32));
-    const size_t smem = buf + bin_bytes(T, nw);
+    const BinShape bs = bin_shape(T, std::max(1, a.N / 16 / 32), buf);
+    const size_t smem = buf + bin_bytes(T, bs);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_proj_fft,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_knot_proj_fft, dim3((maxpairs + 1) / 2, a.nk), a.N / 16, smem, st, true, 1, a, logN, nw);
+    return launch_chained(k_knot_proj_fft, dim3((maxpairs + 1) / 2, a.nk), a.N / 16, smem, st, true, 1, a, logN, bs);
 }
 
 int knot_pole_split(int64_t band_pixels)
@@ -742,15 +759,15 @@ int knot_pole_split(int64_t band_pixels)
 cudaError_t launch_knot_grad_pole(const KnotGradArgs &a, const float *map, const float *gout, int64_t npix, int T,
                                   cudaStream_t st)
 {
-    const int nw = bin_warps(T, kPoleWarps, 0);
-    const size_t smem = bin_bytes(T, nw);
+    const BinShape bs = bin_shape(T, kPoleWarps, 0);
+    const size_t smem = bin_bytes(T, bs);
     cudaError_t e = cudaFuncSetAttribute((const void *)k_knot_pole,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int split = 1;
     for (int k = 0; k < a.nk; ++k) split = std::max(split, a.pole_split[k]);
     return launch_chained(k_knot_pole, dim3(4 * split, 2, a.nmaps * a.nk), kPoleWarps * 32, smem, st, true, 1, a,
-                          map, gout, npix, nw);
+                          map, gout, npix, bs);
 }
 
 cudaError_t launch_knot_reduce(const KnotGradArgs &a, double *out, int T, cudaStream_t st)

@@ -1,0 +1,29 @@
+"""Knot gradients at the limits of a call: as many knots as a kernel may have on the longest kernel grid
+(the knot tables beside the projection's 16384-point transform), against the FP64 oracle (relative
+2-norm 1e-5, as the other knot-gradient tests)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1104_0672_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+# The transform's buffer takes 139392 of 232448 bytes; a table of T doubles 8 T: three tables fit up to
+# T = 3877, two up to the largest T = 4096.
+@pytest.mark.parametrize("T", [3877, 3878, 4096])
+def test_knot_gradient_of_many_knots_on_the_longest_grid(T):
+    import torch
+
+    import paper_1104_0672_gb300 as ark
+    assert torch.cuda.is_available()
+    spec, gmax = ("ecp", 3, 16384), 20.3 * inputs.DEG  # one pair per ring, of 920 samples or more
+    g = ark.Grid.ecp(*spec[1:])
+    knots = inputs.gaussian_knots(8.0 * inputs.DEG, gmax, T)
+    k = ark.Kernel(g, knots, gmax)
+    x, gr = (inputs.white_noise(inputs.npix(spec), 1, config=25, salt=s) for s in (0, 1))
+    _, gk = ark.convolve_backward(g, k, torch.from_numpy(x).cuda(), torch.from_numpy(gr).cuda(), False, True)
+    ref = oracle.knot_grad(spec, knots, gmax, x[0].astype(np.float64), gr[0].astype(np.float64))
+    err = float(np.linalg.norm(gk[0].cpu().numpy() - ref) / np.linalg.norm(ref))
+    assert err < 1e-5, err
