@@ -99,7 +99,9 @@ arkcos_status arkcos_kernel_update_knots(arkcos_kernel kernel, const double *kno
 arkcos_status arkcos_destroy_kernel(arkcos_kernel kernel);
 
 /* Workspace bytes needed by arkcos_convolve (backward = 0) or arkcos_convolve_backward
- * (backward = 1) for `nmaps` maps using the given kernels (nkernels == 1 or nmaps).
+ * (backward = 1) for `nmaps` maps using the given kernels (nkernels == 1 or nmaps).  The knot
+ * gradients of several kernels share launches in batches of kernels whose scratch together stays
+ * within 256 MiB (or is that of one kernel, where one needs more).
  * Errors: EINVAL. */
 arkcos_status arkcos_workspace_size(arkcos_grid grid, const arkcos_kernel *kernels,
                                     int64_t nkernels, int64_t nmaps, uint32_t flags,

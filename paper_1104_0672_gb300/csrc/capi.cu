@@ -378,7 +378,7 @@ struct StageScope {
     }
 };
 
-constexpr size_t kKnotBatchBytes = 256u << 20;
+constexpr size_t kKnotBatchBytes = 256u << 20;  // scratch of a batch of kernels' knot gradients
 
 struct Layout {
     size_t taps_off[kMaxKernelsPerLaunch * 8];
@@ -419,26 +419,28 @@ bool layout_for(const Grid &g, const arkcos_kernel *ks, int64_t nk, int64_t nmap
             maxpairs = std::max(maxpairs, ks[k]->k.npairs);
             maxT = std::max(maxT, ks[k]->k.T);
         }
-        L.q = off;
-        // per-map kernels go in batches whose rows of Q stay within kKnotBatchBytes (at least one)
-        L.qstride = (int64_t)maxpairs * (g.N / 2 + 1);
-        L.xstride = (int64_t)maxpairs * 128;
-        L.kbatch = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(nk, kMaxKernelsPerLaunch),
-                                                          (int64_t)(kKnotBatchBytes / (L.qstride * sizeof(float)))));
-        off = align256(off + (size_t)L.kbatch * L.qstride * sizeof(float));
-        L.xproj = off;
-        off = align256(off + (size_t)L.kbatch * L.xstride * sizeof(float));
         int maxfft = 0;
         int64_t pole_pixels = 0;
         for (int64_t k = 0; k < nk; ++k) {
             maxfft = std::max(maxfft, ks[k]->k.knot_fft_pairs);
             pole_pixels = std::max(pole_pixels, ks[k]->k.pole_pixels);
         }
-        L.partial = off;
+        L.qstride = (int64_t)maxpairs * (g.N / 2 + 1);
+        L.xstride = (int64_t)maxpairs * 128;
         L.row_fft = knot_proj_blocks();
         L.row_pole = L.row_fft + (maxfft + 1) / 2;
         const int64_t rows = L.row_pole + 8 * (nk > 1 ? 1 : nmaps) * knot_pole_split(pole_pixels);
         L.pstride = rows * maxT;
+        // per-map kernels go in batches whose rows of Q, projections and partial sums together stay
+        // within kKnotBatchBytes (at least one kernel)
+        const int64_t per_kernel = (L.qstride + L.xstride) * (int64_t)sizeof(float) + L.pstride * (int64_t)sizeof(double);
+        L.kbatch = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(nk, kMaxKernelsPerLaunch),
+                                                          (int64_t)kKnotBatchBytes / per_kernel));
+        L.q = off;
+        off = align256(off + (size_t)L.kbatch * L.qstride * sizeof(float));
+        L.xproj = off;
+        off = align256(off + (size_t)L.kbatch * L.xstride * sizeof(float));
+        L.partial = off;
         off = align256(off + (size_t)L.kbatch * L.pstride * sizeof(double));
     }
     L.total = off;

@@ -1,6 +1,6 @@
 """Knot gradients at the limits of a call: as many knots as a kernel may have on the longest kernel grid
 (the knot tables beside the projection's 16384-point transform), against the FP64 oracle (relative
-2-norm 1e-5, as the other knot-gradient tests)."""
+2-norm 1e-5, as the other knot-gradient tests); and the workspace of many kernels."""
 import numpy as np
 import pytest
 
@@ -27,3 +27,20 @@ def test_knot_gradient_of_many_knots_on_the_longest_grid(T):
     ref = oracle.knot_grad(spec, knots, gmax, x[0].astype(np.float64), gr[0].astype(np.float64))
     err = float(np.linalg.norm(gk[0].cpu().numpy() - ref) / np.linalg.norm(ref))
     assert err < 1e-5, err
+
+
+def test_workspace_of_many_kernels_stays_bounded():
+    """Kernels of one call share launches in batches; what a batch adds for its kernels -- rows of Q,
+    projections and FP64 partial sums together -- stays within 256 MiB, or what one kernel needs."""
+    import paper_1104_0672_gb300 as ark
+
+    def knot_bytes(g, ks):  # the backward workspace less the forward one and the gradients' spectra
+        n = len(ks)
+        spec = n * ((g.nrings + 1) // 2) * (g.nlon // 2 + 1) * 16
+        return ark.workspace_size(g, ks, n, 0, True) - ark.workspace_size(g, ks, n, 0, False) - spec
+
+    for nside, support, T in ((16, 20.0, 4096), (8, 89.0, 4096), (16, 20.0, 100), (128, 40.0, 1000)):
+        g = ark.Grid.healpix(nside)
+        knots = inputs.gaussian_knots(0.4 * support * inputs.DEG, support * inputs.DEG, T)
+        ks = [ark.Kernel(g, knots, support * inputs.DEG) for _ in range(32)]
+        assert knot_bytes(g, ks) <= max(256 << 20, knot_bytes(g, ks[:1])) + 4096, (nside, support, T)
