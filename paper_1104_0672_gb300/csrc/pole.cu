@@ -40,15 +40,34 @@ __device__ double block_sum(double v, double *red)
     return s;
 }
 
-// Direct sum of kernel kd at pixel p of the pole ring over input map mp (this thread's share: the
-// CTAs of the cluster take the pixels of the band's rings, one run of the map, in turn).
-__device__ double pole_sum(const PoleArgs &a, const KernDev &kd, const float *mp, int p, int e, int rank, int ranks)
+// A pixel's sum is taken in slices, each by the threads of one CTA and added in order, as many as its
+// kernel's band has blocks of pixels (a power of two up to kPoleSlices): the order of the sum
+// depends on the kernel alone, not on how many maps or other kernels share the launch.
+constexpr int kPoleThreads = 256, kPoleSlices = 8;
+
+__host__ __device__ inline int pole_slices(int64_t band_pixels)
+{
+    int s = 1;
+    while (s < kPoleSlices && kPoleThreads * (int64_t)s < band_pixels) s *= 2;
+    return s;
+}
+
+// Pixels of the rings of kernel kd's band about a pole.
+__device__ __forceinline__ int64_t band_pixels(const RingDev &rd, const KernDev &kd)
+{
+    const int jh = kd.jhi[0];
+    return rd.poff[jh] + rd.n[jh];
+}
+
+// Direct sum of kernel kd at pixel p of the pole ring over input map mp: this thread's share of slice
+// `slice` (the slices take the pixels of the band's rings, one run of the map, in turn).
+__device__ double pole_sum(const PoleArgs &a, const KernDev &kd, const float *mp, int p, int e, int slice, int slices)
 {
     const int jh = kd.jhi[0], ja = e == 0 ? 0 : a.R - 1 - jh, jz = e == 0 ? jh : a.R - 1;
     const int i = e == 0 ? 0 : a.R - 1;
     const int64_t q0 = a.rd.poff[ja], q1 = a.rd.poff[jz] + a.rd.n[jz];
     double acc = 0.0;
-    for (int64_t q = q0 + rank * blockDim.x + threadIdx.x; q < q1; q += ranks * blockDim.x) {
+    for (int64_t q = q0 + slice * kPoleThreads + threadIdx.x; q < q1; q += slices * kPoleThreads) {
         int j = ja, hi = jz;  // the pixel's ring
         while (j < hi) {
             const int mid = (j + hi + 1) >> 1;
@@ -62,33 +81,40 @@ __device__ double pole_sum(const PoleArgs &a, const KernDev &kd, const float *mp
     return acc;
 }
 
-// One cluster per (pixel p of the pole ring, pole e in {0: ring 0, 1: ring R-1}, map b), its CTAs'
-// sums added in order.  It reads only the input maps and the inverse transforms leave these
+// One cluster per (pixel p of the pole ring, pole e in {0: ring 0, 1: ring R-1}, map b), whose CTAs
+// take its slices in turn.  It reads only the input maps and the inverse transforms leave these
 // rings alone, so it runs beside their end.  FP64 arithmetic (two FMAs per SM and clock) bounds
 // it: the chord from the band table and one sine per pixel, spread over more SMs, 14 us for one
 // nside-2048 map with a 15' support and 21 us at a degree, launch included, against 60 and 224 us
 // with three sines per pixel and a CTA per output pixel going ring by ring.
-__global__ void __launch_bounds__(256) k_pole_fwd(const __grid_constant__ PoleArgs a)
+__global__ void __launch_bounds__(kPoleThreads) k_pole_fwd(const __grid_constant__ PoleArgs a)
 {
     namespace cg = cooperative_groups;
-    __shared__ double red[8], part;
+    __shared__ double red[kPoleThreads / 32], part[kPoleSlices];
     auto cluster = cg::this_cluster();
     const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int p = blockIdx.x / ranks, e = blockIdx.y, b = blockIdx.z;
     const int src = a.vdiv > 1 ? (a.vbase + b) / a.vdiv : b;
     const float *mp = a.map + (int64_t)src * a.npix;
-    double acc = 0.0;
-    if (a.nsum > 0) {
-        // the weighted sum over several kernels of one input map, in kernel order
-        for (int k = 0; k < a.nsum; ++k) acc += a.wsum[k] * pole_sum(a, a.kd[k], mp, p, e, rank, ranks);
-    } else {
-        acc = pole_sum(a, a.kd[a.per_map ? b - a.map_base : 0], mp, p, e, rank, ranks);
+    const int kid = a.nsum > 0 || !a.per_map ? 0 : b - a.map_base;
+    int64_t pixels = band_pixels(a.rd, a.kd[kid]);
+    for (int k = 1; k < a.nsum; ++k) pixels = max(pixels, band_pixels(a.rd, a.kd[k]));
+    const int slices = pole_slices(pixels);
+    for (int s = rank; s < slices; s += ranks) {
+        double acc = 0.0;
+        if (a.nsum > 0) {
+            // the weighted sum over several kernels of one input map, in kernel order
+            for (int k = 0; k < a.nsum; ++k) acc += a.wsum[k] * pole_sum(a, a.kd[k], mp, p, e, s, slices);
+        } else {
+            acc = pole_sum(a, a.kd[kid], mp, p, e, s, slices);
+        }
+        acc = block_sum(acc, red);
+        if (threadIdx.x == 0) part[s] = acc;
     }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) part = acc;
     cluster.sync();
     if (rank == 0 && threadIdx.x == 0) {
-        for (int r = 1; r < ranks; ++r) acc += *cluster.map_shared_rank(&part, r);
+        double acc = part[0];
+        for (int s = 1; s < slices; ++s) acc += *cluster.map_shared_rank(&part[s], s % ranks);
         a.out[(int64_t)b * a.npix + a.rd.poff[e == 0 ? 0 : a.R - 1] + p] = (float)acc;
     }
     cluster.sync();
@@ -131,10 +157,10 @@ __global__ void __launch_bounds__(256) k_pole_adj(PoleArgs a)
 
 cudaError_t launch_pole_fwd(const PoleArgs &a, int64_t band_pixels, cudaStream_t st, bool after_prev)
 {
-    // CTAs per cluster: about one pixel per thread, while the launch is not already some CTAs per SM
+    // CTAs per cluster: one per slice, while the launch is not already some CTAs per SM
     int c = 1;
-    while (c < 8 && 256 * (int64_t)c < band_pixels && 16 * (int64_t)c * a.B <= 4 * device_sms()) c *= 2;
-    return launch_chained(k_pole_fwd, dim3(4 * c, 2, a.B), 256, 0, st, after_prev, c, a);
+    while (c < pole_slices(band_pixels) && 16 * (int64_t)c * a.B <= 4 * device_sms()) c *= 2;
+    return launch_chained(k_pole_fwd, dim3(4 * c, 2, a.B), kPoleThreads, 0, st, after_prev, c, a);
 }
 
 cudaError_t launch_pole_adj(const PoleArgs &a, int max_band_rings, cudaStream_t st)
