@@ -111,7 +111,6 @@ struct Kernel {
     int npairs = 0;
     int64_t ntaps = 0;  // padded tap slots
     int maxband = 0;
-    int maxS = 0;
     int pole_band = 0;         // input rings inside the support of ring 0
     int64_t pole_pixels = 0;   // their pixels
     int max_union8 = 0;        // largest union band of 8 consecutive representative rings
@@ -262,16 +261,17 @@ cudaError_t launch_polar_rho(const ContractArgs &a, int nk, int max_polar_pairs,
 size_t fft_smem_bytes(int M, int N, bool stage_c, int tab, int threads);  // shared memory of a ring FFT class
 cudaError_t launch_chirp_spectra(const FftFwdArgs &a, float2 *fb, int count, int threads, cudaStream_t st);
 // Ring FFT class launches.  after_prev: the previous kernel on the stream is the previous class
-// of the same stage, and this launch may begin while it still runs (ring_common.cuh
-// stage_allow_next / stage_wait_prev).
-cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
+// of the same stage (or the kernel of the call before an inverse stage), and this launch may begin
+// while it still runs (launch_chained): the classes of a stage write disjoint rings and read only
+// what earlier stages wrote, so later ones fill the SMs that the last wave of one leaves idle.
+cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_fwd(const FftFwdArgs &a, bool even_h, int count, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_inv(const FftInvArgs &a, bool even_h, int count, cudaStream_t st, bool after_prev);
 cudaError_t launch_blu_spectra(const FftFwdArgs &a, float2 *fb, int count, cudaStream_t st);  // a.logM, rd, reps, tw
 int blu_table_words(int h);                // words of the per-ring tables of a ring of n = 2h pixels
 size_t blu_smem_bytes(int M, int tab);
 int fft_map_chunk(int count, int nmaps, int split_mult);  // maps per CTA of a ring FFT launch over `count` ring pairs
-cudaError_t launch_fft_inv(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev);
+cudaError_t launch_fft_inv(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev);
 
 // Launch of kernel(args...) in clusters of `cluster` CTAs along x, with the
 // programmatic-serialization attribute when after_prev: the kernel may then begin while the
@@ -337,7 +337,7 @@ cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, 
                                int srows, int want_nbuf, cudaStream_t st);
 cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks, const TcTables &tb, int srows,
                                     cudaStream_t st);
-int contract_tc_nbuf(int rb, int gs, int srows, int want_nbuf);
+int contract_tc_nbuf(int rb, int srows, int want_nbuf);
 int contract_tc_modes();
 cudaError_t take_tc_error(int *out);
 // Failure-detection test knob, read on every call: when the environment variable

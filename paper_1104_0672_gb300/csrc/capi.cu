@@ -632,7 +632,7 @@ arkcos_status run_fft_fwd(const Grid &g, const float *map, float2 *spec, float4 
         a.zero_poles = zero_poles;
         a.tab = c.tab;
         if (c.blu) CK(launch_blu_fwd(a, c.even_h != 0, c.count, st, after_prev));
-        else CK(launch_fft_fwd(a, c.count, c.threads, st, after_prev));
+        else CK(launch_fft_fwd(a, c.count, st, after_prev));
     }
     return ARKCOS_OK;
 }
@@ -666,7 +666,7 @@ arkcos_status run_fft_inv(const Grid &g, const float2 *cbuf, float *map, int64_t
         a.stage_c = c.stage_c;
         a.tab = c.tab;
         if (c.blu) CK(launch_blu_inv(a, c.even_h != 0, c.count, st, after_prev));
-        else CK(launch_fft_inv(a, c.count, c.threads, st, after_prev));
+        else CK(launch_fft_inv(a, c.count, st, after_prev));
     }
     return ARKCOS_OK;
 }
@@ -713,7 +713,7 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
     // against 1.70 ms) and for calls of less than two waves of blocks of 16 (one nside-256 map 27
     // against 29 us; from there on 16 is as fast for one map and faster for several, four
     // nside-2048 maps 1.00 against 1.11 ms)
-    const bool b16_ok[2] = {contract_tc_nbuf(16, 2, srows[1][0], 0) == 2, contract_tc_nbuf(16, 4, srows[1][1], 0) == 2};
+    const bool b16_ok[2] = {contract_tc_nbuf(16, srows[1][0], 0) == 2, contract_tc_nbuf(16, srows[1][1], 0) == 2};
     int tc_rb = 8, tc_gs = g4_ok ? 4 : 2, tc_want = 0;
     const int64_t ctas16 = (int64_t)((g.N / 2 + contract_tc_modes()) / contract_tc_modes()) * ((g.nrep + 15) / 16) *
                            (per_map ? nmaps : 1);
@@ -1069,7 +1069,6 @@ arkcos_status arkcos_set_kernel(arkcos_grid grid, const double *knots, int64_t n
             toff.push_back((int)taps);
             const int slots = (std::max(s0, s1) + 1 + 3) & ~3;
             taps += slots;
-            K.maxS = std::max(K.maxS, std::max(s0, s1));
             K.sum_taps_fix += (f ? s1 : s0) + 1;
         }
     }
@@ -1391,7 +1390,7 @@ arkcos_status arkcos_convolve_multi(arkcos_grid grid, const arkcos_kernel *kerne
     if (weighted) {
         // sum_k w_k L(f_k) = L(sum_k w_k f_k): the weighted samples of the kernels are summed over
         // the ring pairs of the widest one, and one convolution follows (ten kernels on one
-        // nside-2048 map: 1.7 ms against 9.0 ms when each kernel's coefficients were generated
+        // nside-2048 map: 1.5 ms against 9.0 ms when each kernel's coefficients were generated
         // and contracted and their outputs summed)
         const int64_t wk = widest(kernels, K);
         {

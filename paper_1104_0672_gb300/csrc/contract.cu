@@ -9,8 +9,9 @@
 //     rho_m(i,j) = sum_{k >= 0} c_k K(u(x_k)) cos(m x_k),   c_k = multiplicity(k) / N,
 // and the contraction is c_m(i) = sum_j rho_m(i,j) w_j a_m(j) (w_j folded into a).
 //
-// k_taps evaluates c_k K(u) per pair in FP64 (u is the squared chord of Eq. kernel_angle
-// in the cancellation-free form 4[B cos^2(x/2) + A sin^2(x/2)]), storing FP32 values.
+// k_taps evaluates c_k K(u) per sample (u is the squared chord of Eq. kernel_angle in the
+// cancellation-free form 4[B cos^2(x/2) + A sin^2(x/2)]): the offset of u from its knot in FP64, the
+// linear step from there in FP32.
 #include <algorithm>
 
 #include "fft_engine.cuh"

@@ -4,7 +4,7 @@
 // For a block of RB (8 or 16) representative output rings x 128 modes the coefficients are a
 // dense product  rho[m, col] = sum_k C_f[m, k] T[k, col]  with C_f[m, k] = cos(pi m (2k + f) / N)
 // (f = the pair's sample offset, see contract.cu) and T the FP32 kernel samples.  The CTA
-// stages C (exact FP64 values split into TF32 hi + lo parts, prepared per grid) and T (split
+// stages C (cosines in FP64, split into TF32 hi + lo parts of together 22 to 23 bits, prepared per grid) and T (split
 // into hi + lo on the fly) in shared memory, a pass of 16 samples at a time with the next pass's
 // loads in flight, and one thread issues tcgen05.mma kind::tf32 with the accumulator in tensor
 // memory:
@@ -314,8 +314,8 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                         }
                         if (early) issue(w, b0, 0);
                         __syncthreads();
-                        // cosines of four samples from k for offset f (hi + lo of the tables: the
-                        // FP32 value)
+                        // cosines of four samples from k for offset f (hi + lo of the tables: within
+                        // one unit in the last place of the FP32 value)
                         auto cosines = [&](int k, int f, float (&c)[4]) {
                             if (!WIDE || k < nkc_tab * 32) {
                                 const float4 *t4 = reinterpret_cast<const float4 *>(
@@ -447,7 +447,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                                        src + oct * 256 + (k0 & 16) * 8 + wi * 4, 16);
                         }
                     } else {
-                        // past the tables: the exact values of cos(pi t / N), t = m (2k + f) mod 2N
+                        // past the tables: cos(pi t / N), t = m (2k + f) mod 2N, split as they are
                         const bool pow2 = (a.N & (a.N - 1)) == 0;
                         for (int e = tid; e < ncos * kTcModes * kTcK; e += Sh::kThreads) {
                             const int x = e % (kTcModes * kTcK), tl = e / (kTcModes * kTcK);
@@ -904,12 +904,11 @@ int contract_tc_modes() { return kTcModes; }
 constexpr size_t kTcSmemLimit = 216 * 1024;  // dynamic shared memory of a one-CTA-per-SM launch
 constexpr size_t kTcRow = (size_t)kTcModes * sizeof(float4);
 
-// Staging buffers of srows rows for blocks of rb rings in groups of gs.  Two CTAs per SM
+// Staging buffers of srows rows for blocks of rb rings.  Two CTAs per SM
 // (rb == 8): one, unless `want` == 2 and two fit in 200 KiB.  One CTA per SM (rb == 16): two when
 // they fit.
-int contract_tc_nbuf(int rb, int gs, int srows, int want)
+int contract_tc_nbuf(int rb, int srows, int want)
 {
-    (void)gs;
     if (rb == 16) return 2 * srows * kTcRow + 32 <= kTcSmemLimit ? 2 : 1;
     return want == 2 && 2 * srows * kTcRow + 32 <= 200 * 1024 ? 2 : 1;
 }
@@ -956,7 +955,7 @@ cudaError_t launch_tc(const ContractArgs &a, int nchunks, const TcTables &tb, in
 cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int nchunks, const TcTables &tb,
                                int srows, int want_nbuf, cudaStream_t st)
 {
-    const int nbuf = contract_tc_nbuf(rb, gs, srows, want_nbuf);
+    const int nbuf = contract_tc_nbuf(rb, srows, want_nbuf);
     if (f32) return launch_tc<8, 4, false, true>(a, nchunks, tb, srows, nbuf, st);
     if (rb == 16)
         return gs == 4 ? launch_tc<16, 4, false, false>(a, nchunks, tb, srows, nbuf, st)
@@ -969,7 +968,7 @@ cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, 
 cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks, const TcTables &tb, int srows,
                                     cudaStream_t st)
 {
-    const int nbuf = contract_tc_nbuf(16, 4, srows, 0);
+    const int nbuf = contract_tc_nbuf(16, srows, 0);
     return f32 ? launch_tc<16, 4, true, true>(a, nchunks, tb, srows, nbuf, st)
                : launch_tc<16, 4, true, false>(a, nchunks, tb, srows, nbuf, st);
 }

@@ -72,8 +72,8 @@ __device__ __forceinline__ double profile_eval(double u, const double *ut, const
 // Reinsch's recurrence: for cos(2 alpha) >= 0 the difference D_k = C_k - C_{k-1} obeys
 // D_{k+1} = D_k - lam C_k (lam = 4 sin^2 alpha); otherwise the sum E_k = C_k + C_{k-1}
 // obeys E_{k+1} = mu C_k - E_k (mu = 4 cos^2 alpha).  Rounding error grows linearly in k;
-// the state is re-seeded every 64 taps from exact values: cos2n[t] = cos(pi t / N) (hi, lo), t < 2N,
-// N even, whose entry t - N/2 is the sine.
+// the state is re-seeded every 64 taps from the table cos2n[t] = cos(pi t / N) (hi + lo, within one unit
+// in the last place), t < 2N, N even, whose entry t - N/2 is the sine.
 #define REC_STEP()                 \
     do {                           \
         if (low) {                 \
@@ -103,7 +103,7 @@ __device__ __forceinline__ float gen_rho(const float4 *__restrict__ tp4, int S, 
         const float4 t4 = __ldg(&tp4[q]);
         if (q > 0) {
             if ((q & 15) == 0) {
-                // exact C_k at k = 4q and its recurrence partner (angles (2k+f) alpha and
+                // C_k at k = 4q and its recurrence partner (angles (2k+f) alpha and
                 // (2k-1+f) alpha, reduced exactly modulo 2N)
                 const int k = 4 * q, t1 = (2 * k + f) * m % (2 * N), t2 = (2 * k - 1 + f) * m % (2 * N);
                 const float2 c1 = __ldg(&cos2n[t1]), c2 = __ldg(&cos2n[low ? (t2 < N / 2 ? t2 + 3 * (N / 2) : t2 - N / 2) : t2]);

@@ -683,8 +683,6 @@ __global__ void __launch_bounds__(256) k_knot_reduce(const __grid_constant__ Kno
 int knot_proj_blocks() { return device_sms() * 3; }
 int knot_proj_taps() { return kProjTaps; }
 
-int knot_q_band_limit() { return kQBand; }
-
 int knot_q_form(int max_band, int max_union, int max_union2, int srows)
 {
     if (max_union2 <= kQBand && 2 * (size_t)srows * kQGModes * sizeof(float4) <= 100 * 1024) return 0;

@@ -65,30 +65,10 @@ __host__ __device__ __forceinline__ int log2_buffer(int l)
 // which runs as a 2-point buffer).
 __host__ __device__ __forceinline__ bool bluestein(int h) { return h < 2 || (h & (h - 1)) != 0; }
 
-// Calls f.template run<L>() for the runtime buffer size 2^logM (1 <= logM <= 13).
-template <class F>
-__device__ __forceinline__ void dispatch(int logM, F &f)
-{
-    switch (logM) {
-    case 1: f.template run<1>(); break;
-    case 2: f.template run<2>(); break;
-    case 3: f.template run<3>(); break;
-    case 4: f.template run<4>(); break;
-    case 5: f.template run<5>(); break;
-    case 6: f.template run<6>(); break;
-    case 7: f.template run<7>(); break;
-    case 8: f.template run<8>(); break;
-    case 9: f.template run<9>(); break;
-    case 10: f.template run<10>(); break;
-    case 11: f.template run<11>(); break;
-    case 12: f.template run<12>(); break;
-    default: f.template run<13>(); break;
-    }
-}
-
-// The same for the launch of one buffer class.  The host puts every ring whose buffer is at
-// most 2^10 into class 10 and every other ring into the class of exactly its own buffer, so a
-// class LMAX >= 11 needs the code of its own size only (the other sizes are not instantiated).
+// Calls f.template run<L>() for the runtime buffer size 2^logM of a ring in class LMAX.  The host
+// puts every ring whose buffer is at most 2^10 into class 10 and every other ring into the class
+// of exactly its own buffer, so a class LMAX >= 11 needs the code of its own size only (the other
+// sizes are not instantiated).
 template <int LMAX, class F>
 __device__ __forceinline__ void dispatch_upto(int logM, F &f)
 {
@@ -112,10 +92,10 @@ __device__ __forceinline__ void dispatch_upto(int logM, F &f)
 }
 
 // Launch shape of the class of buffers up to 2^LMAX (LMAX >= 10): one thread per radix-16
-// group of the largest buffer, at least 256, and two CTAs per SM below the largest buffer, so
-// that the register budget follows.  The short rings (LMAX = 10) have at most 64 such groups:
-// their CTAs have 64 threads, eight to an SM (four nside-512 maps, forward stage 128 -> 92 us against
-// 256 threads), but 128 for the inverse transforms of kernel grids past 2048 points, where the folds
+// group of the largest buffer, and 512 threads on an SM (four CTAs of 128 threads at 2^11, two
+// of 256 at 2^12, one of 512 at 2^13), so that a thread has 128 registers.  The short rings (LMAX = 10)
+// have at most 64 such groups: their CTAs have 64 threads, eight to an SM (four nside-512 maps, forward
+// stage 128 -> 92 us against 256 threads), but 128 for the inverse transforms of kernel grids past 2048 points, where the folds
 // run over all kernel-grid modes with the whole CTA (one nside-1024 map: 151 us with 256
 // threads, 127 with 128, 147 with 64; at nside 512 54, 49 and 40 us).
 template <int LMAX>
@@ -123,12 +103,6 @@ struct ClassShape {
     static constexpr int kThreads = LMAX <= 10 ? 128 : (1 << LMAX) / 16;  // (at most)
     static constexpr int kMinBlocks = LMAX >= 13 ? 1 : 512 / kThreads;
 };
-
-// Launch order inside one transform stage.  The buffer classes of a stage write disjoint rings
-// and read only what earlier stages wrote, so a class kernel lets the next class of the stage
-// start as soon as all of its own CTAs are running (they fill the SMs its last wave leaves
-// idle), and each CTA waits for the previous class to complete only before it exits: a stage
-// still completes in stream order.
 
 // Lane views of a packed pair: (re, im) of lane 0 (ring j) and lane 1 (ring R-1-j).
 __device__ __forceinline__ float4 lanes4(const fft::cpair &x) { return make_float4(x.re.x, x.im.x, x.re.y, x.im.y); }

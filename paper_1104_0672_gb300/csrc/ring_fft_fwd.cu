@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(512) k_chirp_spectra(FftFwdArgs a, float2 *fb_
     const int l = a.rd.n[j] / 2;
     if (!ring::bluestein(l)) return;  // power-of-two transform: no chirp
     ChirpCta c{buf, fb_all + a.rd.fboff[j], a.tw, l};
-    ring::dispatch(ring::log2_buffer(l), c);
+    ring::dispatch_upto<10>(ring::log2_buffer(l), c);
 }
 
 // One ring pair through the h-point transforms of its two rings (lanes of a cpair).
@@ -270,9 +270,8 @@ cudaError_t launch_fwd_class(const FftFwdArgs &a, int count, cudaStream_t st, bo
                           after_prev, 1, a);
 }
 
-cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, int threads, cudaStream_t st, bool after_prev)
+cudaError_t launch_fft_fwd(const FftFwdArgs &a, int count, cudaStream_t st, bool after_prev)
 {
-    (void)threads;  // the class's own launch shape (ring_common.cuh ClassShape)
     if (count <= 0) return cudaSuccess;
     if (a.logM <= 10) return launch_fwd_class<10>(a, count, st, after_prev);
     if (a.logM == 11) return launch_fwd_class<11>(a, count, st, after_prev);

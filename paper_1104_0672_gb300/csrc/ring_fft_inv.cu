@@ -358,9 +358,8 @@ cudaError_t launch_inv_class(const FftInvArgs &a, int count, cudaStream_t st, bo
                           after_prev, 1, a);
 }
 
-cudaError_t launch_fft_inv(const FftInvArgs &a, int count, int threads, cudaStream_t st, bool after_prev)
+cudaError_t launch_fft_inv(const FftInvArgs &a, int count, cudaStream_t st, bool after_prev)
 {
-    (void)threads;  // the class's own launch shape (ring_common.cuh ClassShape)
     if (count <= 0) return cudaSuccess;
     if (a.logM <= 10) return launch_inv_class<10>(a, count, st, after_prev);
     if (a.logM == 11) return launch_inv_class<11>(a, count, st, after_prev);
