@@ -538,41 +538,57 @@ struct ProjFft {
             ntap[i] = p0 + i < np ? (f[i] ? kd.S1[p] : kd.S0[p]) + 1 : 0;
             q[i] = Q + (int64_t)p * NH;
         }
-        for (int m = threadIdx.x; m < NH; m += blockDim.x) {
-            const bool edge = m == 0 || 2 * m == N;  // its own mirror
-            const float2 ph = expipi_ratio(m, N);
-            float2 e[2];  // Q_m exp(i pi m f / N), halved where the mirror holds the conjugate
+        // the input of the pairs in `which` (bit i: pair p0 + i); whether some value is not finite
+        auto fill = [&](int which) {
+            bool bad = false;
+            for (int m = threadIdx.x; m < NH; m += blockDim.x) {
+                const bool edge = m == 0 || 2 * m == N;  // its own mirror
+                const float2 ph = expipi_ratio(m, N);
+                float2 e[2];  // Q_m exp(i pi m f / N), halved where the mirror holds the conjugate
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float v = ntap[i] > 0 ? __ldg(&q[i][m]) : 0.f, w = edge ? v : 0.5f * v;
-                e[i] = f[i] ? make_float2(w * ph.x, edge ? 0.f : w * ph.y) : make_float2(w, 0.f);
+                for (int i = 0; i < 2; ++i) {
+                    const float v = (which >> i & 1) && ntap[i] > 0 ? __ldg(&q[i][m]) : 0.f, w = edge ? v : 0.5f * v;
+                    bad |= !isfinite(v);
+                    e[i] = f[i] ? make_float2(w * ph.x, edge ? 0.f : w * ph.y) : make_float2(w, 0.f);
+                }
+                // both pairs as real and imaginary part: e0 + i e1, and conj e0 + i conj e1 at N - m
+                sm(fft::digitrev<L>(m), make_float2(e[0].x - e[1].y, e[0].y + e[1].x));
+                if (!edge) sm(fft::digitrev<L>(N - m), make_float2(e[0].x + e[1].y, e[1].x - e[0].y));
             }
-            // both pairs as real and imaginary part: e0 + i e1, and conj e0 + i conj e1 at N - m
-            sm(fft::digitrev<L>(m), make_float2(e[0].x - e[1].y, e[0].y + e[1].x));
-            if (!edge) sm(fft::digitrev<L>(N - m), make_float2(e[0].x + e[1].y, e[1].x - e[0].y));
-        }
-        __syncthreads();
-        fft::adj<L>(buf, a.tw, sm);
+            return bad;
+        };
         const double invN = 1.0 / (double)N;
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        if (wid < bn.warps) {
+        // a value that is not finite would reach the other pair's samples too: a transform each then
+        const bool apart = __syncthreads_or(fill(3));
+        for (int r = 0; r < (apart ? 2 : 1); ++r) {
+            if (apart) {
+                (void)fill(1 << r);
+                __syncthreads();
+            }
+            fft::adj<L>(buf, a.tw, sm);
+            if (wid < bn.warps) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-                for (int k0 = 32 * wid; k0 < ntap[i]; k0 += 32 * bn.warps) {
-                    const int k = k0 + lane;
-                    int t0 = -1;
-                    double w0 = 0.0, w1 = 0.0;
-                    if (k < ntap[i]) {
-                        const float2 v = sm(k);
-                        const double mult = (f[i] == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
-                        const double x = (double)(i ? v.y : v.x) * mult * invN;
-                        double lam;
-                        t0 = sample_knot(a, kd, bn, p0 + i, k, f[i], lam);
-                        w1 = lam * x;
-                        w0 = x - w1;
+                for (int i = 0; i < 2; ++i) {
+                    if (apart && i != r) continue;
+                    for (int k0 = 32 * wid; k0 < ntap[i]; k0 += 32 * bn.warps) {
+                        const int k = k0 + lane;
+                        int t0 = -1;
+                        double w0 = 0.0, w1 = 0.0;
+                        if (k < ntap[i]) {
+                            const float2 v = sm(k);
+                            const double mult = (f[i] == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
+                            const double x = (double)(i ? v.y : v.x) * mult * invN;
+                            double lam;
+                            t0 = sample_knot(a, kd, bn, p0 + i, k, f[i], lam);
+                            w1 = lam * x;
+                            w0 = x - w1;
+                        }
+                        warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
                     }
-                    warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
                 }
+            }
+            if (apart) __syncthreads();
         }
     }
 };

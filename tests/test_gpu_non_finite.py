@@ -49,3 +49,41 @@ def test_non_finite_pixel_stays_in_its_band(spec, support, form):
                 assert ((~a.isfinite()) | (a == c)).all(), (ring, i)
             else:
                 assert not a.isfinite().any(), (ring, i)
+
+
+@pytest.mark.parametrize("ring", [2, 5, 8, 20, 60])
+@pytest.mark.parametrize("form", ["fp32", "tf32"])
+def test_knots_that_a_non_finite_pixel_reaches(ring, form):
+    """With many knots some segments hold no sample of the bad ring's pairs: their gradients stay, to the
+    relative 2-norm of 1e-5 of the other knot-gradient tests (pairs next to the poles are projected two to
+    a transform, and alone where one of the two is not finite, which rounds differently)."""
+    import torch
+
+    import paper_1104_0672_gb300 as ark
+    nside, gmax, T = 256, 2.0 * inputs.DEG, 4096
+    g = ark.Grid.healpix(nside)
+    k = ark.Kernel(g, inputs.gaussian_knots(0.4 * gmax, gmax, T), gmax)
+    flags = ark.FLAG_NO_POLE_FIX | (ark.FLAG_3XTF32 if form == "tf32" else 0)
+    x, gr = (torch.from_numpy(inputs.white_noise(g.npix, 1, config=29, salt=s)).cuda() for s in (0, 1))
+    clean = ark.convolve_backward(g, k, x, gr, False, True, flags)[1][0].cpu().numpy()
+    theta, _, _, n, off = oracle.geometry(("healpix", nside))
+    x[0, int(off[ring]) + 1] = float("nan")
+    bad = ark.convolve_backward(g, k, x, gr, False, True, flags)[1][0].cpu().numpy()
+    # knots of the samples of the pairs (i, ring): cap rings of different lengths sample at 2 pi k / N
+    N, ut = 4 * nside, 4.0 * np.sin(0.5 * gmax * np.arange(T) / (T - 1)) ** 2
+    s2 = np.sin(np.pi * np.arange(N // 2 + 1) / N) ** 2
+    reached = np.zeros(T, bool)
+    for i in range(2 * ring + 200):
+        if abs(theta[i] - theta[ring]) > gmax:
+            continue
+        A, B = np.sin(0.5 * (theta[i] + theta[ring])) ** 2, np.sin(0.5 * (theta[i] - theta[ring])) ** 2
+        u = 4.0 * (B * (1.0 - s2) + A * s2)
+        for v in (u * (1.0 - 1e-12), u, u * (1.0 + 1e-12)):  # (either segment where a sample lies on a knot)
+            t = np.clip(np.searchsorted(ut, v[v <= ut[-1] * (1.0 + 1e-12)], "right") - 1, 0, T - 2)
+            reached[t] = reached[t + 1] = True
+    finite = np.isfinite(bad)
+    assert not finite[0]
+    assert not (~finite & ~reached).any()
+    assert np.linalg.norm(bad[finite] - clean[finite]) < 1e-5 * np.linalg.norm(clean[finite])
+    assert ring > 20 or (~reached).sum() > 100
+
