@@ -242,6 +242,8 @@ __device__ __forceinline__ void warp_deposit(double *bins, int t0, double w0, do
     }
 }
 
+constexpr int kProjTaps = 8, kProjReseed = 16, kProjWarps = 8;  // k_knot_deposit, k_knot_proj
+
 // Warps of a deposit CTA with bins of their own, and whether the table of reciprocal knot spacings has
 // room beside them.
 struct BinShape {
@@ -286,6 +288,14 @@ BinShape bin_shape(int T, int most, size_t other)
     const int64_t rows = std::max<int64_t>(0, 200 * 1024 - (int64_t)other) / row;
     const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(most, rows - 2));
     return BinShape{warps, (int64_t)other + (2 + warps) * row <= 227 * 1024};
+}
+// The same for k_knot_proj, whose warps all project: bins of their own or shared by turns, within a third
+// of an SM, with the table where it fits beside them.
+BinShape proj_shape(int T)
+{
+    int warps = kProjWarps;
+    while (warps > 1 && (size_t)(1 + warps) * T * sizeof(double) > 74 * 1024) warps /= 2;
+    return BinShape{warps, (size_t)(2 + warps) * T * sizeof(double) <= 74 * 1024};
 }
 size_t bin_bytes(int T, BinShape bs) { return (size_t)(1 + bs.table + bs.warps) * T * sizeof(double); }
 
@@ -387,7 +397,6 @@ __global__ void __launch_bounds__(kXWarps * 32) k_knot_proj_f32(const __grid_con
 // 1 - lam and lam.  A warp takes four pairs at a time, eight lanes to a pair and its taps, and adds
 // into its own bins; the CTA writes their sum as its row of partial sums.  FP64 bounds it: 0.08 ms
 // for one nside-2048 kernel, 0.57 ms with a round's deposits staged for one thread to add.
-constexpr int kProjTaps = 8, kProjReseed = 16, kProjWarps = 8;
 
 __global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_constant__ KnotGradArgs a, BinShape bs)
 {
@@ -433,14 +442,17 @@ __global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_c
 // (pair, kProjTaps consecutive taps), from a table built with the kernel.  A warp takes one unit
 // at a time with its lanes over the modes m = lane + 32 t (coalesced Q loads) and, per tap, the
 // phasor z = exp(i m x_k) advanced by exp(i 32 x_k) each step and reseeded from exact values every
-// kProjReseed steps.  The lane sums are reduced by shuffles and deposited in the warp's bins.
+// kProjReseed steps.  The lane sums are reduced by shuffles and deposited in the warp's bins; with many
+// knots several warps share bins and deposit in turn, so that three CTAs (as many as the registers
+// allow) still fit an SM: the phasors need the warps (nside 2000, 2048 knots, backward: 9.1 ms, 17.1 ms
+// with bins for every warp and one CTA per SM; 4096 knots 9.2 and 29.7 ms).
+template <bool SHARED>  // some bins belong to several warps
 __global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_constant__ KnotGradArgs a, BinShape bs)
 {
     extern __shared__ double ksm[];
     const int kb = blockIdx.y;
     const KernDev &kd = a.kd[kb];
     KnotBins bn(ksm, kd, bs);
-    const int nw = bs.warps;
     chain_wait();
     chain_allow_next();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -448,9 +460,11 @@ __global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_cons
     const double invN = 1.0 / (double)N;
     const int2 *units = a.shift_fix ? kd.unit_fix : kd.unit_nofix;
     const int nunits = a.shift_fix ? kd.nunit_fix : kd.nunit_nofix;
-    if (wid < nw) {
-        for (int u = blockIdx.x * nw + wid; u < nunits; u += gridDim.x * nw) {
-            const int2 un = __ldg(&units[u]);
+    for (int u0 = blockIdx.x * kProjWarps; u0 < nunits; u0 += gridDim.x * kProjWarps) {
+        int t0 = -1;
+        double w0 = 0.0, w1 = 0.0;
+        if (u0 + wid < nunits) {
+            const int2 un = __ldg(&units[u0 + wid]);
             const int p = un.x, k0 = un.y;
             const int f = a.shift_fix ? kd.fl[p] : 0;
             const int ntap = (f ? kd.S1[p] : kd.S0[p]) + 1;
@@ -493,8 +507,6 @@ __global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_cons
                 if (lane == j) mine = v;
             }
             const int k = k0 + lane;
-            int t0 = -1;
-            double w0 = 0.0, w1 = 0.0;
             if (lane < kProjTaps && k < ntap) {
                 const double mult = (f == 0 && (k == 0 || 2 * k == N)) ? 1.0 : 2.0;
                 const double x = (double)mine * mult * invN;
@@ -503,6 +515,13 @@ __global__ void __launch_bounds__(kProjWarps * 32) k_knot_proj(const __grid_cons
                 w1 = lam * x;
                 w0 = x - w1;
             }
+        }
+        if constexpr (SHARED) {
+            for (int turn = 0; turn < kProjWarps / bs.warps; ++turn) {
+                if (wid / bs.warps == turn) warp_deposit(bn.bins + wid % bs.warps * bn.T, t0, w0, w1);
+                __syncthreads();
+            }
+        } else {
             warp_deposit(bn.bins + wid * bn.T, t0, w0, w1);
         }
     }
@@ -739,9 +758,9 @@ cudaError_t launch_knot_proj_f32(const KnotGradArgs &a, const float *ctabP, int 
 
 cudaError_t launch_knot_grad_proj(const KnotGradArgs &a, bool have_x, int T, cudaStream_t st)
 {
-    const BinShape bs = bin_shape(T, kProjWarps, 0);
+    const BinShape bs = have_x ? bin_shape(T, kProjWarps, 0) : proj_shape(T);
     const size_t smem = bin_bytes(T, bs);
-    const auto kernel = have_x ? k_knot_deposit : k_knot_proj;
+    const auto kernel = have_x ? k_knot_deposit : bs.warps < kProjWarps ? k_knot_proj<true> : k_knot_proj<false>;
     cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_chained(kernel, dim3(knot_proj_blocks(), a.nk), kProjWarps * 32, smem, st, true, 1, a, bs);

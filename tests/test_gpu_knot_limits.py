@@ -29,6 +29,29 @@ def test_knot_gradient_of_many_knots_on_the_longest_grid(T):
     assert err < 1e-5, err
 
 
+# Pairs of more than 128 samples without a transform, projected by warps with bins of their own (up to
+# 1052 knots) or that 2, 4 and 8 warps share.
+@pytest.mark.parametrize("T", [1052, 1053, 1894, 1895, 3157, 3158, 4096])
+def test_knot_gradient_of_many_knots_without_a_transform(T):
+    import torch
+
+    import paper_1104_0672_gb300 as ark
+    assert torch.cuda.is_available()
+    spec, supports = ("ecp", 17, 600), [35.3, 24.7]
+    g = ark.Grid.ecp(*spec[1:])
+    prof = [(inputs.gaussian_knots(0.4 * s * inputs.DEG, s * inputs.DEG, T), s * inputs.DEG) for s in supports]
+    ks = [ark.Kernel(g, k, gm) for k, gm in prof]
+    x, gr = (inputs.white_noise(inputs.npix(spec), 2, config=30, salt=s) for s in (0, 1))
+    xt, gt = torch.from_numpy(x).cuda(), torch.from_numpy(gr).cuda()
+    _, gk = ark.convolve_backward(g, ks, xt, gt, False, True)
+    for b in range(2):
+        _, one = ark.convolve_backward(g, ks[b], xt[b:b + 1], gt[b:b + 1], False, True)
+        assert torch.equal(one[0], gk[b])
+        ref = oracle.knot_grad(spec, prof[b][0], prof[b][1], x[b].astype(np.float64), gr[b].astype(np.float64))
+        err = float(np.linalg.norm(gk[b].cpu().numpy() - ref) / np.linalg.norm(ref))
+        assert err < 1e-5, (b, err)
+
+
 def test_workspace_of_many_kernels_stays_bounded():
     """Kernels of one call share launches in batches; what a batch adds for its kernels -- rows of Q,
     projections and FP64 partial sums together -- stays within 256 MiB, or what one kernel needs."""
