@@ -333,8 +333,8 @@ struct TcTables {
     const float2 *cos2n;  // cos(pi t / N), t < 2N (hi, lo)
     int nkc;
 };
-cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int nchunks, const TcTables &tb,
-                               int srows, int want_nbuf, cudaStream_t st);
+cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int union4, int nchunks,
+                               const TcTables &tb, int srows, int want_nbuf, cudaStream_t st);
 cudaError_t launch_contract_tc_wide(const ContractArgs &a, bool f32, int nchunks, const TcTables &tb, int srows,
                                     cudaStream_t st);
 int contract_tc_nbuf(int rb, int srows, int want_nbuf);

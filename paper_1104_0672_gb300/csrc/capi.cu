@@ -800,7 +800,7 @@ arkcos_status run_contract(const Grid &g, const arkcos_kernel *ks, int64_t nk, c
             CK(launch_polar_rho(a, (int)cnt, maxpolar, g.d_tw, g.twM, g.d_cos2n, st));
             ++sc.launches;
         }
-        if (narrow) CK(launch_contract_tc(a, tc_rb, tc_gs, !tf32, nchunks, tb, tc_srows, tc_want, st));
+        if (narrow) CK(launch_contract_tc(a, tc_rb, tc_gs, !tf32, maxunion4, nchunks, tb, tc_srows, tc_want, st));
         else CK(launch_contract_tc_wide(a, !tf32, nchunks, tb, wrows, st));
     }
     return ARKCOS_OK;

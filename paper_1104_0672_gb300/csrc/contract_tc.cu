@@ -110,13 +110,15 @@ __device__ __forceinline__ void stage_rows(float4 *dst, const float4 *__restrict
     cp_async_commit();
 }
 
-template <int RB, int G, bool WIDE, bool F32>
+// SLOTS: slots that the groups' bands reach (the plain form of narrow bands has one for 16 of the 32)
+template <int RB, int G, bool WIDE, bool F32, int SLOTS = kTcBand>
 __global__ void __launch_bounds__(TcShape<RB, G>::kThreads, 16 / RB)
 k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__restrict__ cos2n, int nkc_tab, int srows,
               int nbuf, uint32_t rows0, uint32_t ctl)
 {
     using Sh = TcShape<RB, G>;
-    constexpr int kTcN = Sh::kN, kTile = Sh::kTile;
+    constexpr int kTcN = Sh::kN, kTile = Sh::kTile, NY = SLOTS / 8;  // NY: quads of columns per ring and tile
+    static_assert(SLOTS == kTcBand || (F32 && !WIDE));
     extern __shared__ __align__(1024) unsigned char smem[];
     // per stage: cosines hi | lo of tile 0, of tile 1, samples hi | lo of every column; then
     // reused for the staged spectra; at ctl the MMA barriers and the tensor-memory address
@@ -336,17 +338,17 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                         };
 #pragma unroll 1
                         for (int rp = 0; rp < (wv ? G / 2 : 0); ++rp) {
-                            float2 sum[2][2][8];  // [ring][tile][column pair]
+                            float2 sum[2][2][2 * NY];  // [ring][tile][column pair]
                             const int l0 = G * grp + 2 * rp;
 #pragma unroll
                             for (int x = 0; x < 4; ++x) {
-                                uint32_t old[16];
+                                uint32_t old[4 * NY];
                                 if (i > 0) {
                                     tmem_ld_async(lane_base + (uint32_t)((x & 1) * kTile + (l0 + x / 2) * 16), old);
                                     tmem_wait_ld();
                                 }
 #pragma unroll
-                                for (int j = 0; j < 8; ++j)
+                                for (int j = 0; j < 2 * NY; ++j)
                                     sum[x / 2][x & 1][j] = i > 0 ? make_float2(__uint_as_float(old[2 * j]), __uint_as_float(old[2 * j + 1]))
                                                                  : make_float2(0.f, 0.f);
                             }
@@ -366,19 +368,19 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                                         const float4 *t4 = reinterpret_cast<const float4 *>(
                                             ts + (4 * q + j) * kTcN + (x & 1) * kTile + (l0 + x / 2) * 16);
 #pragma unroll
-                                        for (int y = 0; y < 4; ++y) fma4(sum[x / 2][x & 1][2 * y], sum[x / 2][x & 1][2 * y + 1], c, t4[y]);
+                                        for (int y = 0; y < NY; ++y) fma4(sum[x / 2][x & 1][2 * y], sum[x / 2][x & 1][2 * y + 1], c, t4[y]);
                                     }
                                 }
                             }
 #pragma unroll
                             for (int x = 0; x < 4; ++x) {
-                                float out[16];
+                                float out[4 * NY];
 #pragma unroll
-                                for (int j = 0; j < 8; ++j) {
+                                for (int j = 0; j < 2 * NY; ++j) {
                                     out[2 * j] = sum[x / 2][x & 1][j].x;
                                     out[2 * j + 1] = sum[x / 2][x & 1][j].y;
                                 }
-                                tmem_st16(lane_base + (uint32_t)((x & 1) * kTile + (l0 + x / 2) * 16), out);
+                                tmem_st(lane_base + (uint32_t)((x & 1) * kTile + (l0 + x / 2) * 16), out);
                             }
                         }
                     }
@@ -535,7 +537,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                             const int c = tile * kTile + c0 + u;
                             r[u] = mv && s_S[c] >= 0 ? __ldg(&pr[(int64_t)s_p[c] * a.NH + m]) : 0.f;
                         }
-                        tmem_st8(lane_base + (uint32_t)(tile * kTile + c0), r);
+                        tmem_st(lane_base + (uint32_t)(tile * kTile + c0), r);
                     }
                 }
                 __syncthreads();
@@ -595,7 +597,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                     // CH slots at a time, in the order of the input rings (whatever the groups): the
                     // coefficients of the G rings (a ring's even and odd slots lie in different
                     // tiles), then the staged values, each used by all G rings
-                    constexpr int CH = 8, UNROLL = WIDE ? 1 : kTcBand / CH;  // (wide: less code, 4.5 against 5.1 ms)
+                    constexpr int CH = 8, UNROLL = WIDE ? 1 : SLOTS / CH;  // (wide: less code, 4.5 against 5.1 ms)
                     uint32_t cr[G][2][CH / 2];
                     auto coeffs = [&](int h) {
 #pragma unroll
@@ -607,7 +609,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                         tmem_wait_ld();
                     };
 #pragma unroll(UNROLL)
-                    for (int h = 0; h < kTcBand; h += CH) {
+                    for (int h = 0; h < SLOTS; h += CH) {
                         coeffs(h);
                         if (!crosses && (!WIDE || inner)) {
 #pragma unroll
@@ -648,7 +650,7 @@ k_contract_tc(ContractArgs a, const float *__restrict__ ctab, const float2 *__re
                                 acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
                             }
 #pragma unroll 1
-                            for (int h = 0; h < kTcBand; h += CH) {
+                            for (int h = 0; h < SLOTS; h += CH) {
                                 coeffs(h);
 #pragma unroll
                                 for (int u = 0; u < CH; ++u) {
@@ -938,25 +940,30 @@ int contract_band_limit() { return kTcBand; }
 
 namespace {
 
-template <int RB, int G, bool WIDE, bool F32>
+template <int RB, int G, bool WIDE, bool F32, int SLOTS = kTcBand>
 cudaError_t launch_tc(const ContractArgs &a, int nchunks, const TcTables &tb, int srows, int nbuf, cudaStream_t st)
 {
     const size_t ctl = tc_ctl(RB, nbuf, srows), smem = ctl + 32;
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_tc<RB, G, WIDE, F32>,
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_contract_tc<RB, G, WIDE, F32, SLOTS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.NH + kTcModes - 1) / kTcModes, (a.nrep + RB - 1) / RB, nchunks);
-    return launch_chained(k_contract_tc<RB, G, WIDE, F32>, grid, TcShape<RB, G>::kThreads, smem, st, true, 1, a, tb.ctab,
+    return launch_chained(k_contract_tc<RB, G, WIDE, F32, SLOTS>, grid, TcShape<RB, G>::kThreads, smem, st, true, 1, a, tb.ctab,
                           tb.cos2n, tb.nkc, srows, nbuf, tc_rows0(RB, srows), (uint32_t)ctl);
 }
 
 }  // namespace
 
-cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int nchunks, const TcTables &tb,
-                               int srows, int want_nbuf, cudaStream_t st)
+// union4: widest union band of a group of four.  Where it reaches 16 slots at most, the plain form sums no
+// more: on few CTAs its sums are the longest part (one 90 x 180 map, supports of 4 and 10 degrees: 49.1 and
+// 53.9 us, 65.5 and 70.0 with all 32 slots; five maps: 60.3 and 65 us, 77.4 and 82.3).
+cudaError_t launch_contract_tc(const ContractArgs &a, int rb, int gs, bool f32, int union4, int nchunks,
+                               const TcTables &tb, int srows, int want_nbuf, cudaStream_t st)
 {
     const int nbuf = contract_tc_nbuf(rb, srows, want_nbuf);
-    if (f32) return launch_tc<8, 4, false, true>(a, nchunks, tb, srows, nbuf, st);
+    if (f32)
+        return union4 <= 16 ? launch_tc<8, 4, false, true, 16>(a, nchunks, tb, srows, nbuf, st)
+                            : launch_tc<8, 4, false, true>(a, nchunks, tb, srows, nbuf, st);
     if (rb == 16)
         return gs == 4 ? launch_tc<16, 4, false, false>(a, nchunks, tb, srows, nbuf, st)
                        : launch_tc<16, 2, false, false>(a, nchunks, tb, srows, nbuf, st);

@@ -119,7 +119,7 @@ __device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[4])
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // 32 lanes x 8 columns into tensor memory, completed before returning
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8])
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[8])
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                  ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
@@ -130,7 +130,7 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8])
 }
 
 // 32 lanes x 16 columns into tensor memory, completed before returning
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[16])
 {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "

@@ -51,3 +51,28 @@ def test_per_map_beams_of_which_some_are_wide(spec, supports, form):
     y = ark.convolve(g, ks, x, flags)
     for b, k in enumerate(ks):
         assert torch.equal(ark.convolve(g, k, x[b], flags), y[b]), b
+
+
+@pytest.mark.parametrize("spec,supports", [
+    (("ecp", 64, 128), [17.4, 20.2]),     # groups of four reach 16 and 18 slots
+    (("ecp", 64, 128), [17.4, 8.0]),
+    (("healpix", 32), [7.3, 9.0, 11.5]),  # 14 to 22 slots
+])
+@pytest.mark.parametrize("form", ["fp32", "tf32"])
+def test_narrow_bands_around_sixteen_slots(spec, supports, form):
+    import torch
+
+    import paper_1104_0672_gb300 as ark
+    assert torch.cuda.is_available()
+    g = ark.Grid.healpix(spec[1]) if spec[0] == "healpix" else ark.Grid.ecp(spec[1], spec[2])
+    prof = [(inputs.gaussian_knots(0.4 * s * inputs.DEG, s * inputs.DEG, 80), s * inputs.DEG) for s in supports]
+    ks = [ark.Kernel(g, k, gm) for k, gm in prof]
+    x = inputs.white_noise(inputs.npix(spec), len(ks), config=31)
+    xt = torch.from_numpy(x).cuda()
+    flags = ark.FLAG_3XTF32 if form == "tf32" else 0
+    y = ark.convolve(g, ks, xt, flags)
+    for b, k in enumerate(ks):
+        assert torch.equal(ark.convolve(g, k, xt[b], flags), y[b]), b
+        ref = oracle.convolve(spec, *prof[b], x[b].astype(np.float64))
+        err = float(np.linalg.norm(y[b].cpu().numpy() - ref) / np.linalg.norm(ref))
+        assert err < 1e-5, (b, err)
