@@ -397,7 +397,6 @@ __global__ void __launch_bounds__(kXWarps * 32) k_knot_proj_f32(const __grid_con
 // 1 - lam and lam.  A warp takes four pairs at a time, eight lanes to a pair and its taps, and adds
 // into its own bins; the CTA writes their sum as its row of partial sums.  FP64 bounds it: 0.08 ms
 // for one nside-2048 kernel, 0.57 ms with a round's deposits staged for one thread to add.
-
 __global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_constant__ KnotGradArgs a, BinShape bs)
 {
     extern __shared__ double ksm[];
@@ -441,7 +440,7 @@ __global__ void __launch_bounds__(kProjWarps * 32) k_knot_deposit(const __grid_c
 // Projection and deposits of pairs of more than 128 samples without the FFT form: work unit =
 // (pair, kProjTaps consecutive taps), from a table built with the kernel.  A warp takes one unit
 // at a time with its lanes over the modes m = lane + 32 t (coalesced Q loads) and, per tap, the
-// phasor z = exp(i m x_k) advanced by exp(i 32 x_k) each step and reseeded from exact values every
+// phasor z = exp(i m x_k) advanced by exp(i 32 x_k) each step and reseeded from computed ones every
 // kProjReseed steps.  The lane sums are reduced by shuffles and deposited in the warp's bins; with many
 // knots several warps share bins and deposit in turn, so that three CTAs (as many as the registers
 // allow) still fit an SM: the phasors need the warps (nside 2000, 2048 knots, backward: 9.1 ms, 17.1 ms
